@@ -1481,6 +1481,14 @@ def main():
                                    "twin handles), so a pass's events also span the passes "
                                    "beside it and its mean duration overstates its own time"
                                    if cocg else ""))
+        if dom["kernel"] == "fft_direct_solve":
+            roofline["bytes_model"] = ("one direct FP32 correction: the residual read and the solution "
+                                       "read and written in FP64, the half spectrum moved through "
+                                       "the x, y, z, y, x transforms once each way")
+            roofline["note"] = ("latency-bound: at 96^3 every field stays in L2 and a correction is "
+                                "a chain of dependent launches of a few microseconds each; up to "
+                                "four solves run at once (a chain of twin handles), so the mean "
+                                "duration also spans the work beside it")
     roofline_320 = roofline_320_f64 = alu = None
     if stencil320:
         roofline_320 = {"kernel": "stencil2_kernel (of_laplacian_apply, FP32, order 12, 320^3)",

@@ -65,11 +65,15 @@ typedef struct of_precond of_precond;   /* learned preconditioner (of_precond_cr
 
 /* Krylov solve options.  tol is the target of the true FP64 relative residual
  * ||b - A x|| / ||b||.  precision OF_F64: CG/COCG entirely in FP64.  OF_F32: iterative
- * refinement -- FP64 residual, FP32 Krylov solve of the correction to inner_tol (or only to
- * half of what the solve still needs, when that is less), FP64 update -- repeated until tol;
- * the FP32 Poisson CG is preconditioned by a multigrid
- * V-cycle unless no_multigrid is set, or by the learned network when precond is set (see
- * of_precond_create).  Zero fields take defaults (tol 1e-10, max_iter 20000, inner_tol 1e-5,
+ * refinement -- FP64 residual, FP32 solve of the correction, FP64 update -- repeated until tol.
+ * The correction of each pass is direct (the periodic operator is diagonal in Fourier space; a
+ * pass counts as one iteration) on grids of at most 2048 points per axis, unless no_multigrid or
+ * precond is set.  Else it is an FP32 Krylov solve to inner_tol (or only to half of what the solve
+ * still needs, when that is less): preconditioned by a multigrid V-cycle beyond 2048 points
+ * (Poisson and shifted systems whose grid coarsens), plain with no_multigrid, or with the learned
+ * network when precond is set (see of_precond_create).  A direct pass that gains less than a
+ * factor of ten (a shifted system that is singular to FP32) also continues with those.
+ * Zero fields take defaults (tol 1e-10, max_iter 20000, inner_tol 1e-5,
  * check_every 8, precond_theta 0.3). */
 typedef struct {
     double tol;
@@ -77,8 +81,8 @@ typedef struct {
     int precision;
     double inner_tol;
     int check_every;
-    int no_multigrid;      /* 1: plain FP32 CG inner solve for Poisson (no V-cycle) */
-    of_precond* precond;   /* non-NULL with OF_F32, in place of the V-cycle: the FP32 inner
+    int no_multigrid;      /* 1: plain FP32 CG / COCG passes (no direct solve, no V-cycle) */
+    of_precond* precond;   /* non-NULL with OF_F32, in place of the direct solve: the FP32 inner
                               solve is flexible CG preconditioned by this network (Poisson),
                               or flexible GMRES(8) preconditioned by a few flexible-CG steps
                               with this network on -L_h + kf2 |Q|, applied to the real and
@@ -161,15 +165,15 @@ typedef struct {
                                whose gradient is the Hamiltonian's; OF_VW_GRADIENT (lambda/2)
                                int |grad_h u|^2 with the order-2N gradient (Eq.
                                gradient:approximate).  The minimisation is the same. */
-    double nlcg_precond_shift;  /* > 0: the NLCG direction is preconditioned by one multigrid
-                               V-cycle of -L_h + shift (bohr^-2) applied to the gradient, with the
-                               Polak-Ribiere update in its preconditioned form: the real-space
-                               preconditioner for Algorithm NLCG that Sec. 5.5 calls for.  Needs a
-                               grid the multigrid can coarsen (else ignored).  0 (default): the
+    double nlcg_precond_shift;  /* > 0: the NLCG direction is preconditioned by (-L_h + shift)^{-1}
+                               (shift in bohr^-2) applied to the gradient in FP32, with the
+                               Polak-Ribiere update in its preconditioned form: the preconditioner
+                               for Algorithm NLCG that Sec. 5.5 calls for.  The inverse is direct on
+                               grids of at most 2048 points per axis, one multigrid V-cycle beyond
+                               (ignored there when the grid does not coarsen).  0 (default): the
                                plain NLCG of App. C */
     double nlcg_precond_low;    /* > 0 with nlcg_precond_shift > 0: the two-shift form
-                               (-L_h + low)(-L_h + shift)^{-2}, two V-cycles and one FP32 sweep,
-                               which follows the energy's curvature at both ends of the spectrum:
+                               (-L_h + low)(-L_h + shift)^{-2}, which follows the energy's curvature at both ends of the spectrum:
                                ~k^2 at large wave numbers (vW), ~1/k^2 at small ones (Hartree).
                                0 (default): the one-shift form */
 } of_scf_opts;
@@ -245,8 +249,9 @@ of_status of_poisson_solve_noalloc(int n1, int n2, int n3, double L1, double L2,
  *    and the lockstep FP32 CG iterations (FP64 refinement as in the OF_F32 mode) are replayed
  *    from one CUDA graph; the z extent of the stencil blocks is chosen per set of grid shapes
  *    by timing candidates on the first call.
- *  - OF_F32 with multigrid (the default no_multigrid = 0, every cell coarsenable): each cell
- *    runs the multigrid-preconditioned solve of of_poisson_solve, the cells spread over up to 8
+ *  - OF_F32 with no_multigrid = 0 (every cell within 2048 points per axis, or coarsenable): each
+ *    cell runs the direct (or multigrid-preconditioned) solve of of_poisson_solve, the cells
+ *    spread over up to 8
  *    internal streams driven by host threads so that their kernels overlap; the call orders
  *    them after the work queued on the shared stream and the shared stream after them.  The
  *    grids must not be used by other threads meanwhile.

@@ -540,9 +540,9 @@ static of_status poisson_batched(int nc, of_grid* const* gs, const double* const
 using namespace of;
 
 namespace of {
-// Multigrid form of the batched solve: the multigrid-preconditioned solver is host-driven per
-// cell and, on cells of this size, latency bound, so the cells run on the stream pool and
-// their kernels overlap on the GPU.
+// Concurrent form of the batched solve: the direct (or multigrid-preconditioned) solver is
+// host-driven per cell and, on cells of this size, latency bound, so the cells run on the stream
+// pool and their kernels overlap on the GPU.
 static of_status poisson_concurrent(int ncells, of_grid* const* grids, const double* const* rho,
                                     double* const* phi, const KrylovOpts& o, of_solve_info* infos) {
     return run_on_stream_pool(ncells, grids, [&](int c) {
@@ -568,7 +568,7 @@ extern "C" of_status of_poisson_solve_batched(int ncells, of_grid* const* grids,
                                grids[c]->device == grids[0]->device, OF_EINVAL,
                            "batched solve: cell %d differs in stream or device from cell 0", c);
                 OF_REQUIRE(rho[c] && phi[c], OF_EINVAL, "batched solve: null field for cell %d", c);
-                mg = mg_available(grids[c]);
+                mg = fft_available(grids[c]) || mg_available(grids[c]);
             }
             if (mg) return poisson_concurrent(ncells, grids, rho, phi, o, infos);
         }

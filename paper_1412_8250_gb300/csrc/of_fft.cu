@@ -1,0 +1,464 @@
+// Direct FP32 solves with translation-invariant operators on the periodic grid.
+//
+// The order-2N Laplacian of Eq. FD:Laplacian commutes with lattice translations, so the discrete
+// Fourier transform diagonalises it: -L_h has the eigenvalue l(k) = l_x + l_y + l_z with
+// l_a = sum_p 4 w_p sin^2(p theta_a / 2).  One forward transform, a division by the symbol
+// (l for Poisson, a l + Q for the shifted systems, (l + s0) / (l + s1)^2 for the NLCG's
+// preconditioner) and one inverse transform therefore apply the exact inverse.  In FP32 that is
+// the correction of one refinement pass of the mixed-precision solves: the FP64 residual of
+// each pass drops by the FP32 rounding (1e-4 .. 1e-6), where a multigrid-preconditioned Krylov
+// pass took 4 .. 30 iterations of ~17 dependent launches for the same drop.
+//
+// Five launches: x forward, y forward, z forward * symbol * z inverse, y inverse, x inverse,
+// each moving the half spectrum once (4 B per point and direction; 8 B for complex fields).
+// Real fields: two x rows are the real and imaginary part of one line, separated into
+// their half spectra (n1 / 2 + 1 points) on the way out and combined again on the way back.
+// A block transforms a tile of TX = 16 lines (128-byte segments of global memory for the y and
+// z lines) in shared memory, of_fft.cuh.
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <vector>
+
+#include "of_fft.cuh"
+#include "of_krylov.cuh"
+
+namespace of {
+
+struct Fft {
+    bool ok = false;
+    FftPlan plan[3];
+    const float* sym[3];     // l_a(k), k < n_a
+};
+
+void fft_destroy(Fft* f) { delete f; }
+
+static Fft& fft_of(of_grid* g) {
+    if (!g->fft) g->fft = new Fft();
+    return *g->fft;
+}
+
+bool fft_available(of_grid* g) {
+    return g->d.n1 <= FFT_MAX_N && g->d.n2 <= FFT_MAX_N && g->d.n3 <= FFT_MAX_N;
+}
+
+// Plans, twiddles and symbol tables (host FP64, rounded once), built with the first direct solve
+static Fft& fft_tables(of_grid* g) {
+    Fft& f = fft_of(g);
+    if (f.ok) return f;
+    const int n[3] = {g->d.n1, g->d.n2, g->d.n3};
+    std::vector<float> host;
+    size_t off[6];
+    for (int a = 0; a < 3; ++a) {
+        OF_REQUIRE(fft_make_plan(n[a], f.plan[a]), OF_EINVAL, "direct solve: no transform of %d points", n[a]);
+        off[a] = host.size();
+        for (int k = 0; k < n[a]; ++k) {
+            const double t = -2.0 * M_PI * k / n[a];
+            host.push_back((float)std::cos(t));
+            host.push_back((float)std::sin(t));
+        }
+        off[3 + a] = host.size();
+        for (int k = 0; k < n[a]; ++k) {
+            double l = 0.0;
+            for (int p = 1; p <= g->N; ++p) {
+                const double s = std::sin(M_PI * (double)((long long)p * k % n[a]) / n[a]);
+                l += 4.0 * g->w64.w[a][p] * s * s;
+            }
+            host.push_back((float)l);
+        }
+        if (host.size() & 1) host.push_back(0.f);   // the twiddles of the next axis are float2
+    }
+    float* dev = (float*)ws(g, WS_FFTT, sizeof(float) * host.size());
+    OF_CUDA(cudaMemcpyAsync(dev, host.data(), sizeof(float) * host.size(), cudaMemcpyHostToDevice, g->stream));
+    OF_CUDA(cudaStreamSynchronize(g->stream));   // the host vector goes out of scope
+    for (int a = 0; a < 3; ++a) {
+        f.plan[a].tw = (const float2*)(dev + off[a]);
+        f.sym[a] = dev + off[3 + a];
+    }
+    f.ok = true;
+    return f;
+}
+
+// ------------------------------------------------------------- FP64 <-> scaled FP32 by bits
+// v 2^-sh rounded to FP32 (values below its normal range become zero) and back: by integer
+// arithmetic on the bits, as GB300 converts and multiplies FP64 at 2 per clock and SM.
+__device__ __forceinline__ float narrow_scaled(double v, int sh) {
+    const int hi = __double2hiint(v);
+    const unsigned lo = (unsigned)__double2loint(v);
+    const int e = ((hi >> 20) & 0x7ff) - (1023 - 127) - sh;
+    const unsigned sign = (unsigned)hi & 0x80000000u;
+    unsigned m = (((unsigned)hi & 0xfffffu) << 3) | (lo >> 29);
+    m += ((unsigned)max(e, 0) << 23) + ((lo >> 28) & 1u);   // round half away; a carry moves the exponent
+    m = e >= 255 ? 0x7f800000u : m;
+    return __uint_as_float(e <= 0 ? sign : (sign | m));
+}
+__device__ __forceinline__ double widen_scaled(float v, int sh) {
+    const unsigned b = __float_as_uint(v);
+    const int e = (int)((b >> 23) & 0xffu);
+    const unsigned hi = (b & 0x80000000u) | ((unsigned)(e + (1023 - 127) + sh) << 20) | ((b & 0x7fffffu) >> 3);
+    return e == 0 ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// ------------------------------------------------------------------- loads and stores
+// The residual enters a correction divided by the state's scale 2^sh, and the correction is
+// added to the solution times it.
+__device__ __forceinline__ int scale_exponent(const KState* st) {
+    return ((__double2hiint(st->scale) >> 20) & 0x7ff) - 1023;
+}
+struct LdReal32 {
+    const float* p;
+    __device__ void begin() {}
+    __device__ float at(long long i) const { return p[i]; }
+};
+struct LdReal64 {
+    const double* p;
+    const KState* st;
+    int sh;
+    __device__ void begin() { sh = scale_exponent(st); }
+    __device__ float at(long long i) const { return narrow_scaled(p[i], sh); }
+};
+struct LdCplx64 {
+    const double2* p;
+    const KState* st;
+    int sh;
+    __device__ void begin() { sh = scale_exponent(st); }
+    __device__ float2 at(long long i) const {
+        const double2 v = p[i];
+        return make_float2(narrow_scaled(v.x, sh), narrow_scaled(v.y, sh));
+    }
+};
+struct StReal32 {
+    float* p;
+    __device__ void begin() {}
+    __device__ void put(long long i, float v) const { p[i] = v; }
+};
+struct StAccum64 {
+    double* p;
+    const KState* st;
+    int sh;
+    __device__ void begin() { sh = scale_exponent(st); }
+    __device__ void put(long long i, float v) const { p[i] += widen_scaled(v, sh); }
+};
+struct StAccumCplx64 {
+    double2* p;
+    const KState* st;
+    int sh;
+    __device__ void begin() { sh = scale_exponent(st); }
+    __device__ void put(long long i, float2 v) const {
+        double2 x = p[i];
+        x.x += widen_scaled(v.x, sh);
+        x.y += widen_scaled(v.y, sh);
+        p[i] = x;
+    }
+};
+
+// ----------------------------------------------------------------------------- kernels
+constexpr int FFT_THREADS = 256;
+
+__device__ __forceinline__ float2* fft_smem_tables(const FftPlan& P) {
+    extern __shared__ float2 fft_smem[];
+    for (int k = threadIdx.x; k < P.n; k += blockDim.x) fft_smem[k] = P.tw[k];
+    return fft_smem;
+}
+
+// All steps of the tile in a (other buffer b); returns the buffer that holds the result.  The
+// caller's writes to a are made visible here.
+__device__ __forceinline__ float2* fft_tile(const FftPlan& P, float2* a, float2* b, const float2* tw, int rs, int lg) {
+    __syncthreads();
+    for (int st = 0; st < P.nst; ++st) {
+        fft_any_step(P, st, a, b, tw, rs, lg, threadIdx.x, blockDim.x);
+        __syncthreads();
+        float2* t = a;
+        a = b;
+        b = t;
+    }
+    return a;
+}
+
+// x lines forward.  Real: line l of the tile is rows 2 (TX blk + l) and + 1; out gets nh = n / 2 + 1
+// points per row.  Complex: line l is row TX blk + l, nh = n.
+template <bool CPLX, class LD>
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_x_forward(FftPlan P, int lg, long long rows, int nh, LD ld,
+                                                               float2* __restrict__ out, const double* done) {
+    pdl_enter();
+    if (*done != 0.0) return;
+    ld.begin();
+    const int TX = 1 << lg, rs = TX + 1, n = P.n;
+    const float2* tw = fft_smem_tables(P);
+    float2* A = const_cast<float2*>(tw) + n;
+    float2* Bf = A + n * rs;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const long long row0 = (long long)blockIdx.x * TX * (CPLX ? 1 : 2);
+    for (int l = warp; l < TX; l += nw) {
+        if constexpr (CPLX) {
+            const long long r = row0 + l;
+            if (r >= rows) continue;
+#pragma unroll 4
+            for (int i = lane; i < n; i += 32) A[i * rs + l] = ld.at(r * n + i);
+        } else {
+            const long long r = row0 + 2 * l;
+            if (r >= rows) continue;
+            const bool two = r + 1 < rows;
+#pragma unroll 4
+            for (int i = lane; i < n; i += 32)
+                A[i * rs + l] = make_float2(ld.at(r * n + i), two ? ld.at((r + 1) * n + i) : 0.f);
+        }
+    }
+    const float2* R = fft_tile(P, A, Bf, tw, rs, lg);
+    for (int l = warp; l < TX; l += nw) {
+        if constexpr (CPLX) {
+            const long long r = row0 + l;
+            if (r >= rows) continue;
+#pragma unroll 4
+            for (int k = lane; k < n; k += 32) out[r * nh + k] = R[k * rs + l];
+        } else {
+            const long long r = row0 + 2 * l;
+            if (r >= rows) continue;
+            const bool two = r + 1 < rows;
+#pragma unroll 2
+            for (int k = lane; k < nh; k += 32) {
+                const float2 c = R[k * rs + l], d = R[(k == 0 ? 0 : n - k) * rs + l];
+                // the spectra of the real and the imaginary part
+                out[r * nh + k] = make_float2(0.5f * (c.x + d.x), 0.5f * (c.y - d.y));
+                if (two) out[(r + 1) * nh + k] = make_float2(0.5f * (c.y + d.y), 0.5f * (d.x - c.x));
+            }
+        }
+    }
+}
+
+// x lines inverse (forward transform of swapped values, swapped back on the way out)
+template <bool CPLX, class ST>
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_x_inverse(FftPlan P, int lg, long long rows, int nh,
+                                                               const float2* __restrict__ in, ST st,
+                                                               const double* done) {
+    pdl_enter();
+    if (*done != 0.0) return;
+    st.begin();
+    const int TX = 1 << lg, rs = TX + 1, n = P.n;
+    const float2* tw = fft_smem_tables(P);
+    float2* A = const_cast<float2*>(tw) + n;
+    float2* Bf = A + n * rs;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const long long row0 = (long long)blockIdx.x * TX * (CPLX ? 1 : 2);
+    for (int l = warp; l < TX; l += nw) {
+        if constexpr (CPLX) {
+            const long long r = row0 + l;
+            if (r >= rows) continue;
+#pragma unroll 4
+            for (int k = lane; k < n; k += 32) {
+                const float2 v = in[r * nh + k];
+                A[k * rs + l] = make_float2(v.y, v.x);
+            }
+        } else {
+            const long long r = row0 + 2 * l;
+            if (r >= rows) continue;
+            const bool two = r + 1 < rows;
+#pragma unroll 4
+            for (int k = lane; k < nh; k += 32) {
+                float2 a = in[r * nh + k], b = two ? in[(r + 1) * nh + k] : make_float2(0.f, 0.f);
+                const int m = k == 0 ? 0 : n - k;
+                if (m == k) a.y = b.y = 0.f;   // the spectrum of a real row is real there
+                // a + i b at k, conj(a) + i conj(b) at n - k, real and imaginary part swapped
+                A[k * rs + l] = make_float2(a.y + b.x, a.x - b.y);
+                if (m != k) A[m * rs + l] = make_float2(b.x - a.y, a.x + b.y);
+            }
+        }
+    }
+    const float2* R = fft_tile(P, A, Bf, tw, rs, lg);
+    for (int l = warp; l < TX; l += nw) {
+        if constexpr (CPLX) {
+            const long long r = row0 + l;
+            if (r >= rows) continue;
+#pragma unroll 4
+            for (int i = lane; i < n; i += 32) {
+                const float2 v = R[i * rs + l];
+                st.put(r * n + i, make_float2(v.y, v.x));
+            }
+        } else {
+            const long long r = row0 + 2 * l;
+            if (r >= rows) continue;
+            const bool two = r + 1 < rows;
+#pragma unroll 4
+            for (int i = lane; i < n; i += 32) {
+                const float2 v = R[i * rs + l];
+                st.put(r * n + i, v.y);
+                if (two) st.put((r + 1) * n + i, v.x);
+            }
+        }
+    }
+}
+
+// Lines with stride: column c of `cols` starts at (c / group) * gstride + c % group, its points
+// are `stride` apart (y: group = nh, gstride = n2 nh, stride = nh; z: group = cols, stride = cols).
+struct FftCols {
+    long long cols, group, gstride, stride;
+};
+
+__device__ __forceinline__ void cols_load(const float2* F, const FftCols& C, int n, int lg, bool act,
+                                          long long base, bool swap, float2* A) {
+    const int line = threadIdx.x & ((1 << lg) - 1);
+#pragma unroll 4
+    for (int i = threadIdx.x >> lg; i < n; i += blockDim.x >> lg) {
+        const float2 v = act ? F[base + i * C.stride] : make_float2(0.f, 0.f);
+        A[(i << lg) + line] = swap ? make_float2(v.y, v.x) : v;
+    }
+}
+__device__ __forceinline__ void cols_store(float2* F, const FftCols& C, int n, int lg, bool act, long long base,
+                                           bool swap, const float2* R) {
+    const int line = threadIdx.x & ((1 << lg) - 1);
+    if (!act) return;
+#pragma unroll 4
+    for (int i = threadIdx.x >> lg; i < n; i += blockDim.x >> lg) {
+        const float2 v = R[(i << lg) + line];
+        F[base + i * C.stride] = swap ? make_float2(v.y, v.x) : v;
+    }
+}
+
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_y(FftPlan P, int lg, FftCols C, float2* F, int inverse,
+                                                       const double* done) {
+    pdl_enter();
+    if (*done != 0.0) return;
+    const float2* tw = fft_smem_tables(P);
+    float2* A = const_cast<float2*>(tw) + P.n;
+    float2* Bf = A + (P.n << lg);
+    const long long col = ((long long)blockIdx.x << lg) + (threadIdx.x & ((1 << lg) - 1));
+    const bool act = col < C.cols;
+    const long long grp = col / C.group, base = grp * C.gstride + (col - grp * C.group);
+    cols_load(F, C, P.n, lg, act, base, inverse != 0, A);
+    const float2* R = fft_tile(P, A, Bf, tw, 1 << lg, lg);
+    cols_store(F, C, P.n, lg, act, base, inverse != 0, R);
+}
+
+// symbol of the inverse: kind 0: 1 / l (0 for the constant mode); 1: 1 / (l + s1);
+// 2: (l + s0) / (l + s1)^2; 3: 1 / (a l + Q).  norm = 1 / (n1 n2 n3).
+struct FftFilter {
+    int kind;
+    float a, qr, qi, s0, s1, norm;
+    const float *lx, *ly, *lz;
+};
+
+// z lines: forward, times the symbol, inverse
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_z_filter(FftPlan P, int lg, FftCols C, int nh, float2* F,
+                                                              FftFilter f, const double* done) {
+    pdl_enter();
+    if (*done != 0.0) return;
+    const float2* tw = fft_smem_tables(P);
+    float2* A = const_cast<float2*>(tw) + P.n;
+    float2* Bf = A + (P.n << lg);
+    const int line = threadIdx.x & ((1 << lg) - 1);
+    const long long col = ((long long)blockIdx.x << lg) + line;
+    const bool act = col < C.cols;
+    cols_load(F, C, P.n, lg, act, col, false, A);
+    const int ky = act ? (int)(col / nh) : 0, kx = act ? (int)(col - (long long)ky * nh) : 0;
+    const float lxy = f.lx[kx] + f.ly[ky];
+    for (int pass = 0; pass < 2; ++pass) {
+        float2* R = fft_tile(P, A, Bf, tw, 1 << lg, lg);
+        if (pass == 1) {
+            cols_store(F, C, P.n, lg, act, col, true, R);
+            break;
+        }
+        for (int i = threadIdx.x >> lg; i < P.n; i += blockDim.x >> lg) {
+            const float2 v = R[(i << lg) + line];
+            const float l = lxy + f.lz[i];
+            float2 o;
+            if (f.kind == 3) {
+                const float dr = fmaf(f.a, l, f.qr), di = f.qi;
+                const float den = fmaf(dr, dr, di * di);
+                const float m = den > 1e-30f ? f.norm / den : 0.f;   // a singular mode is left alone
+                const float gr = dr * m, gi = -di * m;
+                o = make_float2(gr * v.x - gi * v.y, gr * v.y + gi * v.x);
+            } else {
+                float m;
+                if (f.kind == 0) m = l > 0.f ? f.norm / l : 0.f;
+                else {
+                    const float q = 1.f / (l + f.s1);
+                    m = f.norm * q;
+                    if (f.kind == 2) m *= (l + f.s0) * q;
+                }
+                o = make_float2(m * v.x, m * v.y);
+            }
+            R[(i << lg) + line] = make_float2(o.y, o.x);
+        }
+        Bf = R == A ? Bf : A;
+        A = R;
+    }
+}
+
+// ------------------------------------------------------------------------------- host
+// raises a kernel's dynamic shared memory limit where it needs that (once per thread and device)
+static void allow_smem(of_grid* g, const void* kernel, size_t smem) {
+    if (smem <= 40 * 1024) return;
+    static thread_local std::vector<std::pair<const void*, int>> raised;
+    const std::pair<const void*, int> key(kernel, g->device);
+    if (std::find(raised.begin(), raised.end(), key) != raised.end()) return;
+    OF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    raised.push_back(key);
+}
+
+// log2 of the lines per tile: 16, fewer for long lines (two tiles and the twiddles within 227 KB)
+// and where 16 would leave SMs without a block
+static int tile_lg(int n, long long lines) {
+    int lg = n <= 512 ? 4 : n <= 1024 ? 3 : 2;
+    while (lg > 2 && (lines >> lg) < num_sms()) --lg;
+    return lg;
+}
+
+template <bool CPLX, class LD, class ST>
+static void fft_apply(of_grid* g, LD ld, ST st, FftFilter f, const double* done) {
+    Fft& T = fft_tables(g);
+    const Dims& d = g->d;
+    const int nh = CPLX ? d.n1 : d.n1 / 2 + 1;
+    const long long rows = (long long)d.n2 * d.n3;
+    float2* F = (float2*)ws(g, WS_FFT, sizeof(float2) * (size_t)rows * nh);
+    f.norm = (float)(1.0 / (double)d.n);
+    f.lx = T.sym[0];
+    f.ly = T.sym[1];
+    f.lz = T.sym[2];
+    const double word = 4.0 * (CPLX ? 2 : 1) * (double)d.n;
+    ProfScope ps(g, PC_FFT, 10.0 * word + 3.0 * 2.0 * word);
+    auto blocks = [](long long lines, int lg) { return (unsigned)((lines + (1 << lg) - 1) >> lg); };
+    // x forward
+    const long long xl = CPLX ? rows : (rows + 1) / 2;
+    const int lgx = tile_lg(d.n1, xl), lgy = tile_lg(d.n2, (long long)nh * d.n3), lgz = tile_lg(d.n3, (long long)nh * d.n2);
+    const size_t sx = sizeof(float2) * (size_t)d.n1 * (1 + 2 * ((1 << lgx) + 1));
+    const size_t sy = sizeof(float2) * (size_t)d.n2 * (1 + 2 * (1 << lgy));
+    const size_t sz = sizeof(float2) * (size_t)d.n3 * (1 + 2 * (1 << lgz));
+    const FftCols cy{(long long)nh * d.n3, nh, (long long)d.n2 * nh, nh};
+    const FftCols cz{(long long)nh * d.n2, (long long)nh * d.n2, 0, (long long)nh * d.n2};
+    allow_smem(g, (const void*)k_fft_x_forward<CPLX, LD>, sx);
+    allow_smem(g, (const void*)k_fft_x_inverse<CPLX, ST>, sx);
+    allow_smem(g, (const void*)k_fft_y, sy);
+    allow_smem(g, (const void*)k_fft_z_filter, sz);
+    launch_pdl(k_fft_x_forward<CPLX, LD>, blocks(xl, lgx), FFT_THREADS, sx, g->stream, T.plan[0], lgx, rows, nh, ld, F, done);
+    if (d.n2 > 1)
+        launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, 0, done);
+    launch_pdl(k_fft_z_filter, blocks(cz.cols, lgz), FFT_THREADS, sz, g->stream, T.plan[2], lgz, cz, nh, F, f, done);
+    if (d.n2 > 1)
+        launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, 1, done);
+    launch_pdl(k_fft_x_inverse<CPLX, ST>, blocks(xl, lgx), FFT_THREADS, sx, g->stream, T.plan[0], lgx, rows, nh,
+               (const float2*)F, st, done);
+}
+
+void fft_correct(of_grid* g, const double* r, double* x, const KState* st) {
+    FftFilter f{};
+    fft_apply<false>(g, LdReal64{r, st, 0}, StAccum64{x, st, 0}, f, &st->done);
+}
+
+void fft_correct_shifted(of_grid* g, const double2* r, double2* x, double a, double2 Q, const KState* st) {
+    FftFilter f{};
+    f.kind = 3;
+    f.a = (float)a;
+    f.qr = (float)Q.x;
+    f.qi = (float)Q.y;
+    fft_apply<true>(g, LdCplx64{r, st, 0}, StAccumCplx64{x, st, 0}, f, &st->done);
+}
+
+void fft_inverse_real(of_grid* g, const float* r, float* z, double shift, double low, const double* done) {
+    FftFilter f{};
+    f.kind = low > 0.0 ? 2 : 1;
+    f.s0 = (float)low;
+    f.s1 = (float)shift;
+    fft_apply<false>(g, LdReal32{r}, StReal32{z}, f, done);
+}
+
+}  // namespace of

@@ -1,0 +1,280 @@
+// Mixed-radix complex FFT of a tile of lines held in shared memory, FP32.
+//
+// A tile holds TX lines of n points as tile[i * rs + line] (line fastest), so that a warp's
+// accesses of one radix step are contiguous whatever the radix.  Stockham's autosort form:
+// step with radix r after a product L of earlier radices takes, for b in [0, n/r), the points
+// b + s n/r (s < r), twiddles them by exp(-2 pi i q s / (L r)), q = b mod L, applies the r-point
+// DFT and writes the points (b / L) L r + q + s L of the other buffer; one barrier per step,
+// results in natural order.  Radices 2..10, 12 and 16 are unrolled in registers (composite
+// ones by Cooley-Tukey over their factors); any other prime factor takes a direct O(r) sum per
+// output, so every extent is accepted.  The inverse is the forward transform with real and
+// imaginary parts swapped before and after.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace of {
+
+constexpr int FFT_MAX_N = 2048;      // points of one line (two tiles of lines in shared memory)
+constexpr int FFT_MAX_STAGES = 12;
+
+struct FftPlan {
+    int n, nst;
+    int r[FFT_MAX_STAGES];           // radix of each step
+    int L[FFT_MAX_STAGES];           // product of the radices before it
+    int T[FFT_MAX_STAGES];           // n / r
+    int tl[FFT_MAX_STAGES];          // n / (r L): twiddle step
+    unsigned mL[FFT_MAX_STAGES];     // floor(2^32 / L) + 1 (0 for L = 1): b / L = mulhi(b, mL)
+    unsigned mT[FFT_MAX_STAGES];     // the same for T
+    const float2* tw;                // exp(-2 pi i k / n), k < n
+};
+
+inline bool fft_unrolled(int r) { return (r >= 2 && r <= 10) || r == 12 || r == 16; }
+
+#define OF_HD __host__ __device__ __forceinline__
+
+OF_HD unsigned fft_mulhi(unsigned a, unsigned b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (unsigned)(((unsigned long long)a * b) >> 32);
+#endif
+}
+OF_HD int fft_div(int v, unsigned magic) { return magic ? (int)fft_mulhi((unsigned)v, magic) : v; }
+
+OF_HD float2 cxadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+OF_HD float2 cxsub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+OF_HD float2 cxmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
+
+// exp(-2 pi i k / N) as compile-time constants (Taylor series after reduction to |t| <= pi / 4)
+template <int N>
+struct FftRoots {
+    float c[N], s[N];
+    static constexpr double taylor(double t, bool odd) {
+        double term = odd ? t : 1.0, sum = term;
+        for (int k = odd ? 1 : 0; k < 24; k += 2) {
+            term *= -t * t / ((k + 1.0) * (k + 2.0));
+            sum += term;
+        }
+        return sum;
+    }
+    constexpr FftRoots() : c(), s() {
+        for (int k = 0; k < N; ++k) {
+            // angle 2 pi k / N = (pi / 2) quarter + t, 8 k = 2 quarter N + rest with |rest| <= N
+            const int quarter = (4 * k + N / 2) / N;
+            const double t = 6.283185307179586476925 * ((double)k / N - 0.25 * quarter);
+            const double ct = taylor(t, false), st = taylor(t, true);
+            const int h = quarter % 4;
+            c[k] = (float)(h == 0 ? ct : h == 1 ? -st : h == 2 ? -ct : st);
+            s[k] = (float)(h == 0 ? -st : h == 1 ? -ct : h == 2 ? st : ct);
+        }
+    }
+};
+
+// v times the compile-time root (c, s)
+OF_HD float2 cxroot(float2 v, float c, float s) {
+    if (s == 0.f && c == 1.f) return v;
+    if (s == 0.f && c == -1.f) return make_float2(-v.x, -v.y);
+    if (c == 0.f && s == -1.f) return make_float2(v.y, -v.x);
+    if (c == 0.f && s == 1.f) return make_float2(-v.y, v.x);
+    return make_float2(v.x * c - v.y * s, v.x * s + v.y * c);
+}
+
+template <int R> struct Dft;
+template <> struct Dft<2> {
+    static OF_HD void run(float2 (&v)[2]) {
+        const float2 a = v[0], b = v[1];
+        v[0] = cxadd(a, b);
+        v[1] = cxsub(a, b);
+    }
+};
+template <> struct Dft<4> {
+    static OF_HD void run(float2 (&v)[4]) {
+        const float2 a = cxadd(v[0], v[2]), b = cxsub(v[0], v[2]);
+        const float2 c = cxadd(v[1], v[3]), d = cxsub(v[1], v[3]);
+        v[0] = cxadd(a, c);
+        v[2] = cxsub(a, c);
+        v[1] = make_float2(b.x + d.y, b.y - d.x);   // b - i d
+        v[3] = make_float2(b.x - d.y, b.y + d.x);
+    }
+};
+// odd R: pairs s_k = v_k + v_{R-k}, d_k = v_k - v_{R-k}
+template <int R> struct DftOdd {
+    static OF_HD void run(float2 (&v)[R]) {
+        constexpr FftRoots<R> W{};
+        constexpr int H = R / 2;
+        float2 s[H], d[H];
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            s[k] = cxadd(v[k + 1], v[R - 1 - k]);
+            d[k] = cxsub(v[k + 1], v[R - 1 - k]);
+        }
+        const float2 v0 = v[0];
+        float2 sum = v0;
+#pragma unroll
+        for (int k = 0; k < H; ++k) sum = cxadd(sum, s[k]);
+        v[0] = sum;
+#pragma unroll
+        for (int m = 1; m <= H; ++m) {
+            float2 re = v0, im = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                const int t = (m * (k + 1)) % R;
+                re.x += W.c[t] * s[k].x;
+                re.y += W.c[t] * s[k].y;
+                im.x += W.s[t] * d[k].x;
+                im.y += W.s[t] * d[k].y;
+            }
+            // re + i im and re - i im
+            v[m] = make_float2(re.x - im.y, re.y + im.x);
+            v[R - m] = make_float2(re.x + im.y, re.y - im.x);
+        }
+    }
+};
+template <> struct Dft<3> : DftOdd<3> {};
+template <> struct Dft<5> : DftOdd<5> {};
+template <> struct Dft<7> : DftOdd<7> {};
+// R = A B: n = B n1 + n2, k = k1 + A k2
+template <int A, int B> struct DftPair {
+    static OF_HD void run(float2 (&v)[A * B]) {
+        constexpr FftRoots<A * B> W{};
+        float2 y[B][A];
+#pragma unroll
+        for (int n2 = 0; n2 < B; ++n2) {
+            float2 a[A];
+#pragma unroll
+            for (int n1 = 0; n1 < A; ++n1) a[n1] = v[B * n1 + n2];
+            Dft<A>::run(a);
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) y[n2][k1] = cxroot(a[k1], W.c[(n2 * k1) % (A * B)], W.s[(n2 * k1) % (A * B)]);
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) {
+            float2 b[B];
+#pragma unroll
+            for (int n2 = 0; n2 < B; ++n2) b[n2] = y[n2][k1];
+            Dft<B>::run(b);
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = b[k2];
+        }
+    }
+};
+template <> struct Dft<6> : DftPair<2, 3> {};
+template <> struct Dft<8> : DftPair<4, 2> {};
+template <> struct Dft<9> : DftPair<3, 3> {};
+template <> struct Dft<10> : DftPair<2, 5> {};
+template <> struct Dft<12> : DftPair<4, 3> {};
+template <> struct Dft<16> : DftPair<4, 4> {};
+
+// One butterfly of an unrolled step: line `line`, index b
+template <int R>
+OF_HD void fft_butterfly(const float2* in, float2* out, const float2* tw, int L, int T, int tl, unsigned mL,
+                         int rs, int line, int b) {
+    const int p = fft_div(b, mL), q = b - p * L;
+    float2 v[R];
+#pragma unroll
+    for (int s = 0; s < R; ++s) v[s] = in[(b + s * T) * rs + line];
+    if (L > 1) {
+        const int step = q * tl;
+#pragma unroll
+        for (int s = 1; s < R; ++s) v[s] = cxmul(v[s], tw[s * step]);
+    }
+    Dft<R>::run(v);
+    const int o = p * L * R + q;
+#pragma unroll
+    for (int s = 0; s < R; ++s) out[(o + s * L) * rs + line] = v[s];
+}
+
+// One output of a step with a large prime radix r: u = s T + b
+OF_HD void fft_direct_output(const float2* in, float2* out, const float2* tw, int n, int r, int L, int T, int tl,
+                             unsigned mL, unsigned mT, int rs, int line, int u) {
+    const int s = fft_div(u, mT), b = u - s * T;
+    const int p = fft_div(b, mL), q = b - p * L;
+    const int step = (s * T + q * tl) % n;
+    float2 acc = make_float2(0.f, 0.f);
+    int k = 0;
+    for (int t = 0; t < r; ++t) {
+        const float2 x = in[(b + t * T) * rs + line], w = tw[k];
+        acc.x = fmaf(x.x, w.x, fmaf(-x.y, w.y, acc.x));
+        acc.y = fmaf(x.x, w.y, fmaf(x.y, w.x, acc.y));
+        k += step;
+        if (k >= n) k -= n;
+    }
+    out[(p * L * r + q + s * L) * rs + line] = acc;
+}
+
+// One step for the work items first, first + stride, ... (item = butterfly or output of a line,
+// line fastest: line = item mod 2^lg)
+template <int R>
+OF_HD void fft_step(const FftPlan& P, int st, const float2* in, float2* out, const float2* tw, int rs, int lg,
+                    int first, int stride) {
+    const int items = P.T[st] << lg;
+    for (int w = first; w < items; w += stride)
+        fft_butterfly<R>(in, out, tw, P.L[st], P.T[st], P.tl[st], P.mL[st], rs, w & ((1 << lg) - 1), w >> lg);
+}
+OF_HD void fft_any_step(const FftPlan& P, int st, const float2* in, float2* out, const float2* tw, int rs, int lg,
+                        int first, int stride) {
+    switch (P.r[st]) {
+        case 2: fft_step<2>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 3: fft_step<3>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 4: fft_step<4>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 5: fft_step<5>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 6: fft_step<6>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 7: fft_step<7>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 8: fft_step<8>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 9: fft_step<9>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 10: fft_step<10>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 12: fft_step<12>(P, st, in, out, tw, rs, lg, first, stride); break;
+        case 16: fft_step<16>(P, st, in, out, tw, rs, lg, first, stride); break;
+        default: {
+            const int items = P.n << lg;
+            for (int w = first; w < items; w += stride)
+                fft_direct_output(in, out, tw, P.n, P.r[st], P.L[st], P.T[st], P.tl[st], P.mL[st], P.mT[st], rs,
+                                  w & ((1 << lg) - 1), w >> lg);
+        }
+    }
+}
+
+// Radices of n: the fewest steps, small radices among equals
+inline bool fft_make_plan(int n, FftPlan& P) {
+    if (n < 1 || n > FFT_MAX_N) return false;
+    struct Best { double cost; int r; };
+    // cost[m] over the divisors of n: cheapest sequence of radices with product m
+    static const int radices[] = {16, 12, 10, 9, 8, 7, 6, 5, 4, 3, 2};
+    double cost[FFT_MAX_N + 1];
+    int first[FFT_MAX_N + 1];
+    for (int m = 0; m <= n; ++m) { cost[m] = 1e30; first[m] = 0; }
+    cost[1] = 0.0;
+    for (int m = 2; m <= n; ++m) {
+        if (n % m) continue;
+        auto take = [&](int r, double c) {
+            if (m % r == 0 && cost[m / r] + c < cost[m]) { cost[m] = cost[m / r] + c; first[m] = r; }
+        };
+        for (int r : radices) take(r, 1.0 + 0.04 * r);
+        for (int r = 11; r <= m; r += 2) {
+            bool prime = true;
+            for (int d = 3; d * d <= r; d += 2) prime = prime && r % d != 0;
+            if (prime) take(r, 1.0 + 0.3 * r);
+        }
+    }
+    P.n = n;
+    P.nst = 0;
+    P.tw = nullptr;
+    int m = n, L = 1;
+    while (m > 1) {
+        if (P.nst == FFT_MAX_STAGES || first[m] < 2) return false;
+        const int k = P.nst++, r = first[m];
+        auto magic = [](int d) { return d == 1 ? 0u : (unsigned)((1ull << 32) / (unsigned)d + 1); };
+        P.r[k] = r;
+        P.L[k] = L;
+        P.T[k] = n / r;
+        P.tl[k] = n / (r * L);
+        P.mL[k] = magic(L);
+        P.mT[k] = magic(P.T[k]);
+        L *= r;
+        m /= r;
+    }
+    return true;
+}
+
+}  // namespace of

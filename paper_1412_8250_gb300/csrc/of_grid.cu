@@ -191,6 +191,7 @@ of_status of_grid_destroy(of_grid* g) {
     if (g->twin_in) cudaEventDestroy(g->twin_in);
     if (g->twin_out) cudaEventDestroy(g->twin_out);
     if (g->mg) mg_destroy(g->mg);
+    if (g->fft) fft_destroy(g->fft);
     if (g->graphs) destroy_graphs(g->graphs);
     if (g->cap_stream) cudaStreamDestroy(g->cap_stream);
     if (g->cap_stream2) cudaStreamDestroy(g->cap_stream2);
@@ -236,7 +237,7 @@ const char* of_kernel_class_name(int cls) {
                                       "krylov_update", "mg_smooth", "mg_transfer",
                                       "line_energy", "ions", "other", "mg_pcg_pass_graph",
                                       "cg_cocg_iteration_pair_graph", "precond_net",
-                                      "mg_cocg_pass_graph"};
+                                      "mg_cocg_pass_graph", "fft_direct_solve"};
     return (cls >= 0 && cls < PC_N) ? names[cls] : "";
 }
 

@@ -95,7 +95,7 @@ inline void launch_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t 
 // Sampled per-class kernel timing with CUDA events on the launching stream.
 enum ProfClass {
     PC_STENCIL_F64 = 0, PC_STENCIL_F32, PC_CG_F64, PC_CG_F32, PC_COCG_F64, PC_COCG_F32,
-    PC_UPDATE, PC_MG_SMOOTH, PC_MG_TRANSFER, PC_LINE, PC_ATOMS, PC_OTHER, PC_PCG_GRAPH, PC_KRYLOV_GRAPH, PC_NET, PC_PCOCG_GRAPH, PC_N
+    PC_UPDATE, PC_MG_SMOOTH, PC_MG_TRANSFER, PC_LINE, PC_ATOMS, PC_OTHER, PC_PCG_GRAPH, PC_KRYLOV_GRAPH, PC_NET, PC_PCOCG_GRAPH, PC_FFT, PC_N
 };
 
 // While a CUDA graph is being captured, ProfScope adds the algorithmic bytes of each captured
@@ -175,6 +175,8 @@ struct Buffer {
 
 struct MG;
 void mg_destroy(MG* m);
+struct Fft;
+void fft_destroy(Fft* f);
 
 }  // namespace of
 
@@ -191,6 +193,7 @@ struct of_grid {
     of::Scratch s;
     std::vector<of::Buffer> pool;    // named workspace slots, see of::ws()
     of::MG* mg = nullptr;            // multigrid hierarchy (built on first use)
+    of::Fft* fft = nullptr;          // transform plans of the direct solves (built on first use)
     of::Prof* prof = nullptr;        // kernel timing (of_profile_enable)
     cudaStream_t cap_stream = nullptr;   // private stream for CUDA-graph capture
     cudaStream_t cap_stream2 = nullptr;  // second capture stream (bodies of conditional nodes)
@@ -266,6 +269,9 @@ enum Slot {
     WS_NLCGP,    // preconditioned NLCG: the gradient in FP32, its V-cycle, the FP64 direction
     WS_FGM,      // flexible GMRES: Arnoldi and preconditioned vectors
     WS_IMG,      // periodic images of the ions and their lists per z-slab (nuclear charge)
+    WS_FFT,      // half spectrum of a direct solve
+    WS_FFTT,     // its twiddles and symbol tables
+    WS_RB,       // right-hand side and FP64 residual of a Krylov solve
     WS_FF,       // a field split into double-float pairs (the mixed form's residual sweeps)
     WS_NSLOTS
 };

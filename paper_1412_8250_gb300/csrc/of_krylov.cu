@@ -7,11 +7,11 @@
 //    Q: the matrix is complex symmetric (A^T = A), so COCG (CG with the bilinear form r^T r)
 //    is used in place of the paper's GMRES on the real/imaginary split.
 //
-// Both run either in FP64, or as iterative refinement: an FP64 residual, an FP32 Krylov
-// solve of the correction to a loose relative tolerance, an FP64 update -- repeated until the
-// true FP64 residual meets the tolerance.
+// Both run either in FP64, or as iterative refinement: an FP64 residual, an FP32 solve of the
+// correction, an FP64 update -- repeated until the true FP64 residual meets the tolerance.  The
+// correction is direct (of_fft.cu), else a Krylov solve to a loose relative tolerance.
 //
-// Every iteration is two kernels: the stencil sweep forms p = r + beta p on the fly (halo
+// Every Krylov iteration is two kernels: the stencil sweep forms p = r + beta p on the fly (halo
 // points included), writes p and A p and reduces p^T A p; the update kernel applies alpha,
 // updates x and r and reduces r^T r and |r|^2.  alpha, beta and the stopping flag live in
 // device memory, so the host only synchronises every `check_every` iterations.
@@ -493,8 +493,13 @@ struct OpResidualFF {
     RedCtx rc;
     double a;
     double2 Q;
+    bool direct, first;
+    long long n;
     double acc[3];
-    __device__ bool begin() { acc[0] = acc[1] = acc[2] = 0.0; return true; }
+    __device__ bool begin() {
+        acc[0] = acc[1] = acc[2] = 0.0;
+        return !direct || first || st->done == 0.0;
+    }
     __device__ TF load(long long i) const { return xf[i]; }
     __device__ void store(long long i, TF, TF lap) {
         const T64 rv = vsub(b[i], apply_A(x[i], ff_to(lap), a, Q));
@@ -506,15 +511,8 @@ struct OpResidualFF {
     }
     __device__ void end() {
         if (grid_reduce<3>(acc, rc.partials, rc.counter, st->red) &&
-            threadIdx.x == 0 && threadIdx.y == 0) {
-            st->rr = acc[0];
-            st->rho_re = acc[1];
-            st->rho_im = acc[2];
-            st->beta_re = st->beta_im = 0.0;
-            st->breakdown = 0.0;
-            st->zshift = 0.0;
-            st->done = (acc[0] <= st->tol2) ? 1.0 : 0.0;
-        }
+            threadIdx.x == 0 && threadIdx.y == 0)
+            residual_finish(acc, st, direct, first, n);
     }
 };
 
@@ -526,35 +524,56 @@ constexpr double FF_MIN_TOL = 1e-11;
 // residuals); else in FP64
 template <typename T>
 static void residual(of_grid* g, int st_off, const T* x, const T* b, T* r, double a, double2 Q,
-                     bool ff = false) {
+                     bool ff = false, bool direct = false, bool first = true) {
     constexpr int RY = KT<T>::cplx ? 1 : 2;
     if (ff) {
         using TF = typename OpResidualFF<T>::TF;
         const long long n = g->d.n;
         TF* xf = (TF*)ws(g, WS_FF, sizeof(TF) * (size_t)n);
         launch(k_ff_split<T, TF>, vec_blocks(n), 256, g->stream, n, x, xf);
-        OpResidualFF<T> op{xf, x, b, r, kstate(g, st_off), red_ctx(g, 0), a, Q};
+        OpResidualFF<T> op{xf, x, b, r, kstate(g, st_off), red_ctx(g, 0), a, Q, direct, first, n};
         launch_stencil<TF, RY>(g, ff_weights(g->w64), op);
         return;
     }
-    OpResidual<T> op{x, b, r, kstate(g, st_off), red_ctx(g, 0), (typename KT<T>::R)a, Q};
+    OpResidual<T> op{x, b, r, kstate(g, st_off), red_ctx(g, 0), (typename KT<T>::R)a, Q, direct, first, g->d.n};
     launch_stencil<T, RY>(g, g->w64, op);
 }
 
-// Solve A x = b (b already formed in arena b64, FP64), A = a(-L) + Q.  x: FP64 guess/solution.
+// Whether the FP32 corrections of a mixed-precision solve are direct: the Poisson operator and
+// the shifted ones, unless the caller asks for plain Krylov passes or the learned network.
+template <typename T32>
+static bool direct_form(of_grid* g, double a, double2 Q, const KrylovOpts& o) {
+    if (o.precision != OF_F32 || o.no_multigrid || o.precond || !fft_available(g)) return false;
+    const bool shifted = Q.x != 0.0 || Q.y != 0.0;
+    return std::is_same<T32, float2>::value ? shifted : a == 1.0 && !shifted;
+}
+
+// Solve A x = b (b already formed in rhs_res, FP64), A = a(-L) + Q.  x: FP64 guess/solution.
 template <typename T64, typename T32>
 static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const KrylovOpts& o,
                               of_solve_info* info) {
-    Arena ar = arena(g);
+    const RhsRes rb = rhs_res(g);
     const long long n = g->d.n;
     KState* st = kstate(g, KS64);
-    T64* b = (T64*)ar.b64;
-    T64* r = (T64*)ar.r64;
+    T64* b = (T64*)rb.b64;
+    T64* r = (T64*)rb.r64;
+    const bool direct = direct_form<T32>(g, a, Q, o);
     launch(k_init_state, 1, 1, g->stream, st, o.max_iter);
     launch(k_norm_to_tol<T64>, vec_blocks(n), 256, g->stream, n, b, o.tol, st, red_ctx(g, 0));
     OF_LAUNCH_CHECK();
     const bool ff_res = o.precision == OF_F32 && o.tol >= FF_MIN_TOL;
-    residual<T64>(g, KS64, x, b, r, a, Q, ff_res);
+    residual<T64>(g, KS64, x, b, r, a, Q, ff_res, direct);
+    // The direct solve's passes: each drops the residual by the FP32 rounding (1e-4 the first time,
+    // 1e-6 once the residual is rough), so this many are queued before the host looks; those
+    // after the one that converged find the done flag set and return.
+    auto direct_passes = [&](int k) {
+        for (; k > 0; --k) {
+            if constexpr (std::is_same<T32, float2>::value) fft_correct_shifted(g, r, x, a, Q, st);
+            else fft_correct(g, r, x, st);
+            residual<T64>(g, KS64, x, b, r, a, Q, ff_res, true, false);
+        }
+    };
+    if (direct) direct_passes(std::min(o.max_iter, o.tol >= 1e-4 ? 1 : o.tol >= 1e-8 ? 2 : 3));
     KState h;
     fetch_scalars(g, KS64, KSTATE_DOUBLES, (double*)&h);
     const double bb = h.tol2 / (o.tol * o.tol);
@@ -563,15 +582,27 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
     OF_REQUIRE(std::isfinite(bb), OF_EINVAL, "Krylov solve: the right-hand side is not finite");
     OF_REQUIRE(std::isfinite(h.rr), OF_EINVAL,
                "Krylov solve: the initial guess gives a non-finite residual");
-    int total_iters = 0, refinements = 1;
+    int total_iters = direct ? (int)h.iters : 0, refinements = 1 + total_iters;
     double net_steps = 0.0;
     of_status status = OF_OK;
     if (!(bb > 0.0)) {   // zero right-hand side: the solution is zero
         OF_CUDA(cudaMemsetAsync(x, 0, sizeof(T64) * n, g->stream));
         h.rr = 0.0;
     }
+    // further direct passes while each gains a factor of ten; a system whose symbol nearly vanishes
+    // somewhere (a l + Q close to 0) gains less and is left to the Krylov solvers below
+    for (bool gains = direct; gains && bb > 0.0 && h.rr > h.tol2 && total_iters < o.max_iter;) {
+        const double before = h.rr;
+        direct_passes(1);
+        fetch_scalars(g, KS64, KSTATE_DOUBLES, (double*)&h);
+        total_iters = (int)h.iters;
+        refinements = 1 + total_iters;
+        gains = h.rr < 0.01 * before;
+    }
+    Arena ar{};
     while (bb > 0.0 && h.rr > h.tol2) {
         if (total_iters >= o.max_iter || refinements > 200) { status = OF_ENOCONV; break; }
+        if (!ar.r64) ar = arena(g);
         bool residual_done = false;   // this pass read the true residual back already
         if (o.precision == OF_F32) {
             KState* s32 = kstate(g, KS32);
@@ -700,10 +731,9 @@ static void remove_mean(of_grid* g, double* x) {
 static of_status poisson_impl(of_grid* g, const double* a, const double* b, double* phi,
                               const KrylovOpts& o, of_solve_info* info) {
     const long long n = g->d.n;
-    Arena ar = arena(g);
     launch(k_sum_product, vec_blocks(n), 256, g->stream, n, a, b, red_ctx(g, 120));
     launch(k_form_rhs, vec_blocks(n), 256, g->stream, n, a, b, g->s.scalars + 120, 4.0 * M_PI,
-                                                     (double*)ar.b64);
+                                                     (double*)rhs_res(g).b64);
     OF_LAUNCH_CHECK();
     of_status st = solve_formed<double, float>(g, phi, 1.0, make_double2(0.0, 0.0), o, info);
     remove_mean(g, phi);
@@ -723,8 +753,7 @@ of_status poisson_product(of_grid* g, const double* a, const double* b, double* 
 of_status shifted(of_grid* g, const double* f, double2 P, double2 Q, double kf2, double2* W,
                   const KrylovOpts& o, of_solve_info* info) {
     const long long n = g->d.n;
-    Arena ar = arena(g);
-    launch(k_scale_complex, vec_blocks(n), 256, g->stream, n, f, P, (double2*)ar.b64);
+    launch(k_scale_complex, vec_blocks(n), 256, g->stream, n, f, P, (double2*)rhs_res(g).b64);
     OF_LAUNCH_CHECK();
     return solve_formed<double2, float2>(g, W, 1.0 / kf2, Q, o, info);
 }

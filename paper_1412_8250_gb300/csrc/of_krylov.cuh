@@ -25,7 +25,8 @@ struct KState {
     double breakdown;           // 13
     double red[4];              // 14 reduction outputs
     double zshift;              // 18 mean of the preconditioned vector (projected PCG), else 0
-    double scale;               // 19 FP32 inner solve: correction = scale * FP32 solution
+    double scale;               // 19 FP32 inner solve: correction = scale * FP32 solution (the
+                                //    outer state: the power of two next below the residual's RMS)
 };
 constexpr int KSTATE_DOUBLES = sizeof(KState) / sizeof(double);
 constexpr int KS64 = 128;   // offsets in g->s.scalars
@@ -104,6 +105,27 @@ __device__ __forceinline__ T apply_A(T c, T lap, typename KT<T>::R a, double2 Q)
 }
 
 // ---------------------------------------------------------------- fused stencil ops
+// State from the reduced sums (|r|^2, r^T r) of a true residual.  direct: a residual of the
+// direct solves' refinement, which counts its passes in iters, stops on non-finite values and a
+// zero right-hand side, and needs the residual's scale.
+__device__ __forceinline__ void residual_finish(const double (&acc)[3], KState* st, bool direct, bool first,
+                                                long long n) {
+    st->rr = acc[0];
+    st->rho_re = acc[1];
+    st->rho_im = acc[2];
+    st->beta_re = st->beta_im = 0.0;
+    st->breakdown = 0.0;
+    st->zshift = 0.0;
+    st->done = (acc[0] <= st->tol2) ? 1.0 : 0.0;
+    if (direct) {
+        if (!first) st->iters += 1.0;
+        if (!(acc[0] > st->tol2 && st->tol2 > 0.0 && isfinite(acc[0]))) st->done = 1.0;
+        // 2^floor(log2 RMS), from the exponent of |r|^2 / n
+        const int e = ((__double2hiint(acc[0] / (double)n) >> 20) & 0x7ff) - 1023;
+        st->scale = __hiloint2double(((e >> 1) + 1023) << 20, 0);
+    }
+}
+
 // r = b - A x ; reduces |r|^2 and r^T r into the state and resets the iteration scalars.
 template <typename T>
 struct OpResidual {
@@ -115,8 +137,13 @@ struct OpResidual {
     RedCtx rc;
     typename KT<T>::R a;
     double2 Q;
+    bool direct, first;      // residual_finish; a direct residual after the first is skipped once done
+    long long n;
     double acc[3];
-    __device__ bool begin() { acc[0] = acc[1] = acc[2] = 0.0; return true; }
+    __device__ bool begin() {
+        acc[0] = acc[1] = acc[2] = 0.0;
+        return !direct || first || st->done == 0.0;
+    }
     __device__ T load(long long i) const { return x[i]; }
     __device__ void store(long long i, T c, T lap) {
         const T rv = vsub(b[i], apply_A(c, lap, a, Q));
@@ -128,15 +155,8 @@ struct OpResidual {
     }
     __device__ void end() {
         if (grid_reduce<3>(acc, rc.partials, rc.counter, st->red) &&
-            threadIdx.x == 0 && threadIdx.y == 0) {
-            st->rr = acc[0];
-            st->rho_re = acc[1];
-            st->rho_im = acc[2];
-            st->beta_re = st->beta_im = 0.0;
-            st->breakdown = 0.0;
-            st->zshift = 0.0;
-            st->done = (acc[0] <= st->tol2) ? 1.0 : 0.0;
-        }
+            threadIdx.x == 0 && threadIdx.y == 0)
+            residual_finish(acc, st, direct, first, n);
     }
 };
 
@@ -366,6 +386,17 @@ bool mg_vcycle_shifted_beta(of_grid* g, const float2* r, float2* z, KState* st, 
                             double sigma);
 
 
+// Right-hand side and true residual of a solve (FP64, complex-sized): all that a direct solve
+// needs beside its spectrum.
+struct RhsRes {
+    void *b64, *r64;
+};
+inline RhsRes rhs_res(of_grid* g) {
+    const size_t s64 = (((size_t)g->d.n * sizeof(double2) + 255) / 256) * 256;
+    char* base = (char*)ws(g, WS_RB, 2 * s64);
+    return RhsRes{base, base + s64};
+}
+
 // Arena of Krylov vectors: FP64 (r, pa, pb, Ap, b) and FP32 (r, pa, pb, Ap, e), complex-sized.
 struct Arena {
     void* r64; void* pa64; void* pb64; void* Ap64; void* b64;
@@ -376,11 +407,12 @@ inline Arena arena(of_grid* g) {
     const size_t n = (size_t)g->d.n;
     const size_t s64 = ((n * sizeof(double2) + 255) / 256) * 256;
     const size_t s32 = ((n * sizeof(float2) + 255) / 256) * 256;
-    char* base = (char*)ws(g, WS_K0, 5 * s64 + 6 * s32);
+    const RhsRes rb = rhs_res(g);
+    char* base = (char*)ws(g, WS_K0, 3 * s64 + 6 * s32);
     Arena a;
-    a.r64 = base; a.pa64 = base + s64; a.pb64 = base + 2 * s64; a.Ap64 = base + 3 * s64;
-    a.b64 = base + 4 * s64;
-    char* b32 = base + 5 * s64;
+    a.r64 = rb.r64; a.b64 = rb.b64;
+    a.pa64 = base; a.pb64 = base + s64; a.Ap64 = base + 2 * s64;
+    char* b32 = base + 3 * s64;
     a.r32 = b32; a.pa32 = b32 + s32; a.pb32 = b32 + 2 * s32; a.Ap32 = b32 + 3 * s32;
     a.e32 = b32 + 4 * s32;
     a.z32 = b32 + 5 * s32;
@@ -401,6 +433,13 @@ KState iterate_fcg(of_grid* g, of_precond* P, double theta, int st_off, float* x
 // inner iterations and the final |b - A x|^2 in rr.
 KState iterate_fgmres(of_grid* g, of_precond* P, double theta, int st_off, float2* x, const float2* b,
                       float* z, float* rs, float a, double2 Q, double* net_steps);
+
+// Direct solves (of_fft.cu), for grids of at most FFT_MAX_N points per axis: x += A^{-1} r for the
+// residual r of the state (its scale, and nothing done once its flag is set), A = -L_h on the
+// mean-free fields or a (-L_h) + Q.
+bool fft_available(of_grid* g);
+void fft_correct(of_grid* g, const double* r, double* x, const KState* st);
+void fft_correct_shifted(of_grid* g, const double2* r, double2* x, double a, double2 Q, const KState* st);
 
 // CUDA graphs of the preconditioned CG: "init" (V-cycle + first r^T z) and "pair" (two full
 // iterations, ping and pong of the direction buffers).  Every kernel reads its scalars and the

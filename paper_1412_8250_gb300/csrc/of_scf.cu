@@ -45,7 +45,7 @@ enum {
     SC_FP = 32,        // |f|^2, |Vhat|^2
     SC_GRAM = 40,      // Anderson Gram entries
     SC_ZR = 104,       // <z, r>, <z, r_prev> of the preconditioned NLCG
-    SC_ZERO = 106      // always 0: the V-cycle's stop flag in the preconditioned NLCG
+    SC_ZERO = 106      // always 0: the preconditioner's stop flag in the preconditioned NLCG
 };
 
 static inline int vb(long long n) { return red_blocks(n, 256 * 4); }
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256) k_direction(long long n, const double* r,
 }
 
 // ---- preconditioned NLCG (nlcg_precond_shift > 0)
-// r32 = r / s with s = RMS of r (from the reduced |r|^2), so that the FP32 V-cycle sees unit scale
+// r32 = r / s with s = RMS of r (from the reduced |r|^2), so that the FP32 preconditioner sees unit scale
 __global__ void __launch_bounds__(256) k_grad_demote(long long n, const double* r, const double* rr,
                                                      float* r32) {
     const double inv = rsqrt(fmax(*rr / (double)n, 1e-300));
@@ -871,13 +871,13 @@ static bool nlcg(of_grid* g, const FnParams& fn, double Ne, ScfVecs& v, double* 
                  int line_search, const KrylovOpts& po, ScfStats& st, double pshift, double plow) {
     const long long n = g->d.n;
     const double dV = g->dV;
-    // preconditioned NLCG: buffers of the gradient in FP32, its V-cycle and the FP64 direction
+    // preconditioned NLCG: buffers of the gradient in FP32, its preconditioned form and the FP64 direction
     struct {
         float *r32 = nullptr, *z32 = nullptr;
         double* z = nullptr;
     } pc;
     double zr_prev = 0.0;
-    if (pshift > 0.0 && mg_available(g)) {
+    if (pshift > 0.0 && (fft_available(g) || mg_available(g))) {
         char* p = (char*)ws(g, WS_NLCGP, (sizeof(float) * 2 + sizeof(double)) * (size_t)n + 256);
         pc.z = (double*)p;
         pc.r32 = (float*)(p + sizeof(double) * (size_t)n);
@@ -914,14 +914,19 @@ static bool nlcg(of_grid* g, const FnParams& fn, double Ne, ScfVecs& v, double* 
         double xi = 0.0;
         double m[4];
         if (pshift > 0.0) {
-            // preconditioned direction: z = M^{-1} r with M^{-1} one V-cycle of -L_h + pshift,
-            // or (-L_h + plow) times two of them (FP32 on the gradient scaled to unit RMS),
+            // preconditioned direction: z = M^{-1} r with M^{-1} = (-L_h + pshift)^{-1}, or
+            // (-L_h + plow) times its square (FP32 on the gradient scaled to unit RMS; direct, or
+            // V-cycles in place of the inverses beyond the direct solves' extents),
             // Polak-Ribiere in the preconditioned form xi = <z, r - r_prev> / <z_prev, r_prev>,
             // d = z + xi d_prev
             launch(k_grad_demote, nb, 256, g->stream, n, (const double*)v.r,
                    (const double*)(g->s.scalars + SC_RR), pc.r32);
-            mg_vcycle_real_shifted(g, pc.r32, pc.z32, g->s.scalars + SC_ZERO, pshift);
-            if (plow > 0.0) {
+            if (fft_available(g)) {
+                fft_inverse_real(g, pc.r32, pc.z32, pshift, plow, g->s.scalars + SC_ZERO);
+            } else {
+                mg_vcycle_real_shifted(g, pc.r32, pc.z32, g->s.scalars + SC_ZERO, pshift);
+            }
+            if (plow > 0.0 && !fft_available(g)) {
                 mg_vcycle_real_shifted(g, pc.z32, pc.r32, g->s.scalars + SC_ZERO, pshift);
                 launch_stencil<float, 2>(g, g->w32, OpShiftedNegLap32{pc.r32, pc.z32, (float)plow});
             }

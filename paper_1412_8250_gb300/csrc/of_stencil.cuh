@@ -744,6 +744,9 @@ bool mg_available(of_grid* g);
 void mg_vcycle(of_grid* g, const float* r, float* z, const double* done);
 // z = one V-cycle of (-L_h + sigma) applied to r, sigma > 0 (real fields)
 void mg_vcycle_real_shifted(of_grid* g, const float* r, float* z, const double* done, double sigma);
+// z = (-L_h + shift)^{-1} r, or (-L_h + low)(-L_h + shift)^{-2} r for low > 0, directly (of_fft.cu)
+bool fft_available(of_grid* g);
+void fft_inverse_real(of_grid* g, const float* r, float* z, double shift, double low, const double* done);
 // the same for complex fields and A = -L + sigma (sigma > 0), real and imaginary parts alike
 void mg_vcycle_shifted(of_grid* g, const float2* r, float2* z, const double* done, double sigma);
 
