@@ -1,0 +1,363 @@
+// FP64 Laplacian sweeps summed exactly in 64-bit fixed point on the integer pipes.
+//
+// GB300 issues 2 FP64 operations per clock and SM but 60 mad.wide.s32 (32 x 32 + 64 bits): the
+// order-12 sum of an FP64 field, 37 FP64 operations per point, is bound by the FP64 pipe at
+// 13 GPts/s.  The weights of Eq. FD:Laplacian are integers over a common denominator,
+//   N = 6: w_p h^2 = {1425600, -222750, 44000, -7425, 864, -50} / 831600, centre -2480478 / 831600,
+// so with the field in fixed point, X = x 2^k in 60 bits, the sum over the neighbours is an exact
+// integer sum, each weight multiplying the two 32-bit limbs of the 64-bit sum of the neighbours
+// at its distance (six with equal spacings, two else): about 8 integer operations per distance and
+// no FP64 operation until one conversion and one multiplication per point (per axis when the
+// spacings differ).
+//
+// Brick of 16 units x 8 rows x 8 planes per block of 128 threads, a unit being two neighbouring
+// doubles of a row (two real points, or one complex point).  The brick and its x-y halo are staged
+// once in shared memory as fixed point; each thread takes the z halo of its own column straight
+// from global memory.  The block's exponent is
+// two above the largest of its z halo and first staged third.  A staged value beyond that, a value
+// that is not finite, or a stretch of staged values (2 x 1 x 8 points) that is not zero but 2^6 and
+// more below the largest, for which 60 bits would keep less than the 53 of FP64, makes the block
+// take FP64 arithmetic instead.  So a value's error is at most 2^-53 of the largest value of its
+// stretch, and ordinary fields take the integer path everywhere.
+//
+// Measured on a GB300 (order 12): 96^3 69.1 -> 12.7 us, 320^3 2.4 ms -> 0.41 ms (13.7 -> 80 GPts/s); now
+// bound by instruction issue and latency at 12 warps per SM (157 registers; 4.9 staged values per
+// point with their conversions, ~8 integer operations per distance).  Tried: both loads and
+// conversions of two slots in flight 13.8 us / 74 GPts/s (spills), two blocks per SM without spills
+// 16.1 / 80, 4 planes per brick 16.1 / 70, 16 rows 16.3 / 81, 16 rows of 4 planes 18.2 / 69.
+#pragma once
+
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+
+#include "of_stencil.cuh"
+
+namespace of {
+
+#define OF_FIX_HD __host__ __device__ __forceinline__
+
+// W_p (p = 0: the centre, once per axis) and the common denominator
+template <int N> OF_FIX_HD constexpr int fix_weight(int p) {
+    if (N == 1) return p == 0 ? -2 : 1;
+    if (N == 3) return p == 0 ? -490 : p == 1 ? 270 : p == 2 ? -27 : 2;
+    return p == 0 ? -2480478 : p == 1 ? 1425600 : p == 2 ? -222750 : p == 3 ? 44000 : p == 4 ? -7425 : p == 5 ? 864 : -50;
+}
+// low bits left out of the integer sum's conversion: the sum is at most 2^60 times the 12, 3264 or
+// 17.6e6 of three axes' absolute weights, below 2^(63 + SH)
+OF_FIX_HD constexpr int fix_shift(int N) { return N == 1 ? 2 : N == 3 ? 10 : 22; }
+inline double fix_denominator(int N) { return N == 1 ? 1.0 : N == 3 ? 180.0 : 831600.0; }
+
+// double -> fixed point with exponent E (biased, >= 128): the mantissa as a 60-bit integer shifted
+// right by E - e (towards zero), in units of 2^(E - 1082); |x| < 2^(E - 1022).  Subnormals are 0.
+OF_FIX_HD long long fix_from_bits(int hi, unsigned lo, int E) {
+    const int e = (hi >> 20) & 0x7ff;
+    const unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    const int s = E - e < 63 ? E - e : 63;   // 63 leaves nothing of 60 bits
+    const long long v = (long long)((m << 7) >> s), sign = (long long)(hi >> 31);
+    return (v ^ sign) - sign;
+}
+
+// A sum s of neighbours (64 bits) times W, by its two 32-bit limbs: the sum of W s is h 2^32 + p - n
+struct FixAcc {
+    long long h = 0;
+    unsigned long long p = 0, n = 0;
+    OF_FIX_HD void add(long long s, int W) {
+        const int hi = (int)(s >> 32);
+        const unsigned lo = (unsigned)s;
+        h += (long long)hi * W;
+        if (W > 0) p += (unsigned long long)lo * (unsigned)W;
+        else n += (unsigned long long)lo * (unsigned)(-W);
+    }
+    // the sum times 2^-SH, rounded to FP64; 2^(63 + SH) is above the largest sum
+    template <int SH>
+    OF_FIX_HD double value() const {
+        const long long lo = (long long)(p - n);
+        const long long t = h + (lo >> 32);
+        return (double)(long long)(((unsigned long long)t << (32 - SH)) | ((unsigned long long)(unsigned)lo >> SH));
+    }
+};
+
+constexpr int FX_UX = 16, FX_BY = 8, FX_THREADS = FX_UX * FX_BY;
+template <int N> struct FixDepth { static constexpr int value = 8; };   // planes per brick
+
+struct FixScale {
+    double s[3];   // 2^fix_shift / (D h_a^2)
+};
+
+template <int N, bool CPLX>
+constexpr int fix_row_width() { return 32 + 2 * (CPLX ? 2 * N : ((N + 1) & ~1)); }
+template <int N, bool CPLX>
+constexpr size_t fix_smem_bytes() {
+    return sizeof(long long) * (size_t)FixDepth<N>::value * (FX_BY + 2 * N) * fix_row_width<N, CPLX>();
+}
+
+// The Laplacian at the planes k < nz of a thread's two columns, from the fixed-point column (z) and
+// tile (own: this unit's first value in the tile's first plane): put(k, l0, l1).  With equal
+// spacings the six neighbours at distance p are summed before the two multiplications by W_p
+// (s0 = s1 = s2); else each axis has its sum and its scale.
+template <int N, bool CPLX, bool ISO, int BZ, class Put>
+__device__ __forceinline__ void fix_planes(const longlong2 (&col)[BZ + 2 * N], const long long* own, int nz, double s0,
+                                           double s1, double s2, Put&& put) {
+    constexpr int RW = fix_row_width<N, CPLX>(), CPL = (FX_BY + 2 * N) * RW, SH = fix_shift(N);
+    constexpr int HX = (N + 1) & ~1;
+#pragma unroll
+    for (int k = 0; k < BZ; ++k) {
+        if (k >= nz) break;
+        const long long* b = own + k * CPL;
+        const longlong2 c = col[N + k];
+        long long xv[2 * HX + 2];   // real: row values -HX .. HX + 1 around the unit
+        if constexpr (!CPLX) {
+#pragma unroll
+            for (int m = 0; m <= HX; ++m) {
+                const longlong2 t = *reinterpret_cast<const longlong2*>(b - HX + 2 * m);
+                xv[2 * m] = t.x;
+                xv[2 * m + 1] = t.y;
+            }
+        }
+        auto xsum = [&](int p) {
+            if constexpr (CPLX) {
+                const longlong2 u = *reinterpret_cast<const longlong2*>(b + 2 * p);
+                const longlong2 v = *reinterpret_cast<const longlong2*>(b - 2 * p);
+                return make_longlong2(u.x + v.x, u.y + v.y);
+            } else {
+                return make_longlong2(xv[HX + p] + xv[HX - p], xv[HX + 1 + p] + xv[HX + 1 - p]);
+            }
+        };
+        auto ysum = [&](int p) {
+            const longlong2 u = *reinterpret_cast<const longlong2*>(b + p * RW);
+            const longlong2 v = *reinterpret_cast<const longlong2*>(b - p * RW);
+            return make_longlong2(u.x + v.x, u.y + v.y);
+        };
+        auto zsum = [&](int p) {
+            return make_longlong2(col[N + k + p].x + col[N + k - p].x, col[N + k + p].y + col[N + k - p].y);
+        };
+        double l0 = 0.0, l1 = 0.0;
+        if constexpr (ISO) {
+            FixAcc a0, a1;
+            a0.add(c.x, 3 * fix_weight<N>(0));
+            a1.add(c.y, 3 * fix_weight<N>(0));
+#pragma unroll
+            for (int p = 1; p <= N; ++p) {
+                const longlong2 x = xsum(p), y = ysum(p), z = zsum(p);
+                a0.add(x.x + y.x + z.x, fix_weight<N>(p));
+                a1.add(x.y + y.y + z.y, fix_weight<N>(p));
+            }
+            l0 = s0 * a0.template value<SH>();
+            l1 = s0 * a1.template value<SH>();
+        } else {
+            auto axis = [&](auto&& sum, double s) {
+                FixAcc a0, a1;
+                a0.add(c.x, fix_weight<N>(0));
+                a1.add(c.y, fix_weight<N>(0));
+#pragma unroll
+                for (int p = 1; p <= N; ++p) {
+                    const longlong2 t = sum(p);
+                    a0.add(t.x, fix_weight<N>(p));
+                    a1.add(t.y, fix_weight<N>(p));
+                }
+                l0 = fma(s, a0.template value<SH>(), l0);
+                l1 = fma(s, a1.template value<SH>(), l1);
+            };
+            axis(xsum, s0);
+            axis(ysum, s1);
+            axis(zsum, s2);
+        }
+        put(k, l0, l1);
+    }
+}
+
+template <int N, bool CPLX, bool ISO, class Op>
+__global__ void __launch_bounds__(FX_THREADS, 3)
+fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int bricks, Op op) {
+    pdl_enter();
+    if (!op.begin()) return;
+    constexpr int BZ = FixDepth<N>::value;
+    constexpr int HX = CPLX ? 2 * N : ((N + 1) & ~1);   // staged halo doubles each side in x
+    constexpr int RW = fix_row_width<N, CPLX>();
+    constexpr int ROWS = FX_BY + 2 * N;
+    constexpr int CPL = ROWS * RW;
+    constexpr int XC = RW / 2;                          // two-double chunks of a core row
+    constexpr int SLOTS = 2 * N * FX_UX + FX_BY * XC;   // halo rows: core columns only
+    constexpr int SPT = (SLOTS + FX_THREADS - 1) / FX_THREADS;
+    extern __shared__ __align__(16) long long fix_smem[];
+    __shared__ int yoff[ROWS], zoff[BZ + 2 * N], xoff[RW];   // periodic offsets in doubles (< 2^31)
+    __shared__ int wmax[FX_THREADS / 32];
+    const double* x = op.field();
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + FX_UX * ty;
+    const int RF = CPLX ? 2 * d.n1 : d.n1, PF = RF * d.n2;
+    // staged row and first column of each of this thread's slots
+    int srow[SPT], scol[SPT];
+#pragma unroll
+    for (int m = 0; m < SPT; ++m) {
+        const int sl = tid + m * FX_THREADS;
+        if (sl < FX_BY * XC) {
+            srow[m] = N + sl / XC;
+            scol[m] = 2 * (sl % XC);
+        } else {
+            const int hr = (sl - FX_BY * XC) / FX_UX;
+            srow[m] = hr < N ? hr : hr + FX_BY;
+            scol[m] = HX + 2 * ((sl - FX_BY * XC) % FX_UX);
+        }
+        if (sl >= SLOTS) srow[m] = -1;
+    }
+    // two doubles of a chunk: one 16-byte load where rows and the field allow it (a chunk
+    // starts at an even double and is contiguous across the wrap when rows are even)
+    auto load2 = [&](int base, int x0, int x1) -> double2 {
+        if (vec) return *reinterpret_cast<const double2*>(x + (unsigned)(base + x0));
+        return make_double2(x[(unsigned)(base + x0)], x[(unsigned)(base + x1)]);
+    };
+    auto expo = [](double a) { return (__double2hiint(a) >> 20) & 0x7ff; };
+
+    for (int brick = blockIdx.x; brick < bricks; brick += gridDim.x) {
+        const int kb = brick / (bx * by), rem = brick - kb * bx * by, jb = rem / bx, ib = rem - jb * bx;
+        const int x0 = ib * 32, y0 = jb * FX_BY, z0 = kb * BZ;
+        __syncthreads();   // the previous brick's readers of the tables and the tile
+        for (int t = tid; t < BZ + 2 * N; t += FX_THREADS) zoff[t] = wrap_index(z0 - N + t, d.n3) * PF;
+        for (int t = tid; t < ROWS; t += FX_THREADS) yoff[t] = wrap_index(y0 - N + t, d.n2) * RF;
+        for (int t = tid; t < RW; t += FX_THREADS) {
+            if constexpr (CPLX) xoff[t] = 2 * wrap_index((x0 - HX) / 2 + (t >> 1), d.n1) + (t & 1);
+            else xoff[t] = wrap_index(x0 - HX + t, d.n1);
+        }
+        __syncthreads();
+        // the z halo of this thread's own column and its first slot in every plane; the largest
+        // exponent among them, plus two, is the block's
+        const int own = yoff[N + ty], oc0 = xoff[HX + 2 * tx], oc1 = xoff[HX + 2 * tx + 1];
+        longlong2 col[BZ + 2 * N];
+        double2 v[BZ];
+        auto load_slot = [&](int m, double2 (&v)[BZ]) {
+            if (srow[m] < 0) return;
+            const int o = yoff[srow[m]], c0 = xoff[scol[m]], c1 = xoff[scol[m] + 1];
+#pragma unroll
+            for (int k = 0; k < BZ; ++k) v[k] = load2(zoff[N + k] + o, c0, c1);
+        };
+        auto top = [&](double2 q) { return max(expo(q.x), expo(q.y)); };
+        double2 zr[2 * N];
+#pragma unroll
+        for (int j = 0; j < 2 * N; ++j) zr[j] = load2(zoff[j < N ? j : j + BZ] + own, oc0, oc1);
+        load_slot(0, v);
+        int emax = 0;
+#pragma unroll
+        for (int j = 0; j < 2 * N; ++j) emax = max(emax, top(zr[j]));
+#pragma unroll
+        for (int k = 0; k < BZ; ++k) emax = max(emax, top(v[k]));
+        emax = __reduce_max_sync(0xffffffffu, emax);
+        if ((tid & 31) == 0) wmax[tid >> 5] = emax;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < FX_THREADS / 32; ++w) emax = max(emax, wmax[w]);
+        const int E = max(emax + 2, 128);   // 128: zeros stay zeros, what else is that small takes FP64
+        bool bad = E > 2046;
+        auto fix = [&](double2 q) {
+            return make_longlong2(fix_from_bits(__double2hiint(q.x), (unsigned)__double2loint(q.x), E),
+                                  fix_from_bits(__double2hiint(q.y), (unsigned)__double2loint(q.y), E));
+        };
+        auto stage = [&](int m, double2 (&v)[BZ]) {
+            if (srow[m] < 0) return;
+            int lo = 0;   // largest exponent of the stretch
+            long long* dst = fix_smem + srow[m] * RW + scol[m];
+#pragma unroll
+            for (int k = 0; k < BZ; ++k) {
+                lo = max(lo, top(v[k]));
+                *reinterpret_cast<longlong2*>(dst + k * CPL) = fix(v[k]);
+            }
+            bad |= lo > E || (lo != 0 && lo < E - 7);
+        };
+#pragma unroll
+        for (int j = 0; j < 2 * N; ++j) col[j < N ? j : j + BZ] = fix(zr[j]);
+#pragma unroll
+        for (int m = 0; m < SPT; ++m) {
+            if (m > 0) load_slot(m, v);
+            stage(m, v);
+        }
+        const bool fp64 = __syncthreads_or(bad) != 0;
+        const int y = y0 + ty, xe = x0 + 2 * tx;         // first double of this thread's unit
+        const bool act0 = y < d.n2 && xe < RF, act1 = act0 && xe + 1 < RF;
+        const long long i0 = (long long)y * d.n1 + (CPLX ? xe / 2 : xe);
+        const int nz = min(BZ, d.n3 - z0);
+        auto put = [&](int k, double l0, double l1) {
+            const long long i = (long long)(z0 + k) * d.n1 * d.n2 + i0;
+            if constexpr (CPLX) {
+                if (act0) op.store(i, op.load(i), make_double2(l0, l1));
+            } else {
+                if (act0) op.store(i, op.load(i), l0);
+                if (act1) op.store(i + 1, op.load(i + 1), l1);
+            }
+        };
+        if (!fp64) {
+            const long long* own_s = fix_smem + (ty + N) * RW + HX + 2 * tx;
+#pragma unroll
+            for (int k = 0; k < BZ; ++k) col[N + k] = *reinterpret_cast<const longlong2*>(own_s + k * CPL);
+            const double unit = __hiloint2double((E - 1082 + 1023) << 20, 0);
+            fix_planes<N, CPLX, ISO, BZ>(col, own_s, nz, fs.s[0] * unit, fs.s[1] * unit, fs.s[2] * unit, put);
+        } else {
+            // FP64 arithmetic, straight from global memory
+            constexpr int XS = CPLX ? 2 : 1;
+            const int cx = HX + 2 * tx, ry = N + ty;
+            for (int k = 0; k < nz; ++k) {
+                double l[2];
+                for (int q = 0; q < 2; ++q) {
+                    auto at = [&](int j, int r, int c) { return x[(unsigned)(zoff[j] + yoff[r] + xoff[c + q])]; };
+                    double acc = W.centre * at(N + k, ry, cx);
+                    for (int p = 1; p <= N; ++p) {
+                        acc = fma(W.w[2][p], at(N + k + p, ry, cx) + at(N + k - p, ry, cx), acc);
+                        acc = fma(W.w[0][p], at(N + k, ry, cx + p * XS) + at(N + k, ry, cx - p * XS), acc);
+                        acc = fma(W.w[1][p], at(N + k, ry + p, cx) + at(N + k, ry - p, cx), acc);
+                    }
+                    l[q] = acc;
+                }
+                put(k, l[0], l[1]);
+            }
+        }
+    }
+    op.end();
+}
+
+template <int N, bool CPLX, bool ISO, class Op>
+void launch_fix_kernel(of_grid* g, const FixScale& fs, Op op) {
+    const Dims& d = g->d;
+    const long long RF = CPLX ? 2LL * d.n1 : d.n1;
+    const bool vec = RF % 2 == 0 && ((uintptr_t)op.field() & 15) == 0;
+    const int bx = (int)((RF + 31) / 32), by = (d.n2 + FX_BY - 1) / FX_BY;
+    const int bricks = bx * by * ((d.n3 + FixDepth<N>::value - 1) / FixDepth<N>::value);
+    // one block per brick, up to the reductions' limit
+    const unsigned grid = (unsigned)std::min(bricks, OF_MAX_RED_BLOCKS);
+    constexpr size_t smem = fix_smem_bytes<N, CPLX>();
+    if constexpr (smem > 40 * 1024) {
+        static thread_local int configured_device = -1;
+        if (configured_device != g->device) {
+            OF_CUDA(cudaFuncSetAttribute(fix_kernel<N, CPLX, ISO, Op>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem));
+            configured_device = g->device;
+        }
+    }
+    launch_pdl(fix_kernel<N, CPLX, ISO, Op>, dim3(grid), dim3(FX_UX, FX_BY), smem, g->stream, d, g->w64, fs, vec, bx,
+               by, bricks, op);
+}
+
+// Sweeps a plain FP64 field (op.field(): the doubles of a real or, CPLX, an interleaved complex
+// field; op.load / op.store as for the other sweeps) of the grid with the fixed-point kernel.
+template <bool CPLX, class Op>
+void launch_field(of_grid* g, Op op) {
+    if ((CPLX ? 2 : 1) * g->d.n >= (1LL << 31)) {   // beyond the kernel's 32-bit offsets
+        using T = typename std::conditional<CPLX, double2, double>::type;
+        launch_stencil<T, CPLX ? 1 : 2>(g, g->w64, op);
+        return;
+    }
+    const int cls = OpInfo<Op>::cls >= 0 ? OpInfo<Op>::cls : PC_STENCIL_F64;
+    ProfScope ps(g, cls, (double)OpInfo<Op>::words * (CPLX ? 16.0 : 8.0) * (double)g->d.n);
+    FixScale fs;
+    for (int a = 0; a < 3; ++a) fs.s[a] = std::ldexp(1.0, fix_shift(g->N)) / (fix_denominator(g->N) * g->h[a] * g->h[a]);
+    const bool iso = fs.s[0] == fs.s[1] && fs.s[1] == fs.s[2];
+    switch (g->N * 2 + (iso ? 1 : 0)) {
+        case 2: launch_fix_kernel<1, CPLX, false>(g, fs, op); break;
+        case 3: launch_fix_kernel<1, CPLX, true>(g, fs, op); break;
+        case 6: launch_fix_kernel<3, CPLX, false>(g, fs, op); break;
+        case 7: launch_fix_kernel<3, CPLX, true>(g, fs, op); break;
+        case 12: launch_fix_kernel<6, CPLX, false>(g, fs, op); break;
+        case 13: launch_fix_kernel<6, CPLX, true>(g, fs, op); break;
+        default: OF_REQUIRE(false, OF_EINVAL, "unsupported finite-difference half order %d", g->N);
+    }
+}
+
+}  // namespace of

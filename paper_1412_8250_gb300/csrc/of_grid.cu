@@ -6,7 +6,7 @@
 #include <cstring>
 #include <cmath>
 
-#include "of_stencil.cuh"
+#include "of_fix.cuh"
 
 namespace of {
 
@@ -100,6 +100,7 @@ struct OpLap {
     const T* x;
     T* y;
     __device__ bool begin() { return true; }
+    __host__ __device__ const T* field() const { return x; }
     __device__ T load(long long i) const { return __ldg(x + i); }
     // two neighbours at an even index (FP32 fast path)
     template <typename U = T, typename = std::enable_if_t<std::is_same<U, float>::value>>
@@ -112,7 +113,7 @@ struct OpLap {
 
 void laplacian(of_grid* g, of_dtype dt, const void* x, void* y) {
     if (dt == OF_F64) {
-        launch_stencil<double, 2>(g, g->w64, OpLap<double>{(const double*)x, (double*)y});
+        launch_field<false>(g, OpLap<double>{(const double*)x, (double*)y});
     } else if (dt == OF_F32) {
         launch_stencil<float, 2>(g, g->w32, OpLap<float>{(const float*)x, (float*)y});
     } else {

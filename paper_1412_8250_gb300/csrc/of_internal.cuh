@@ -272,7 +272,6 @@ enum Slot {
     WS_FFT,      // half spectrum of a direct solve
     WS_FFTT,     // its twiddles and symbol tables
     WS_RB,       // right-hand side and FP64 residual of a Krylov solve
-    WS_FF,       // a field split into double-float pairs (the mixed form's residual sweeps)
     WS_NSLOTS
 };
 

@@ -23,7 +23,7 @@
 #include <mutex>
 #include <type_traits>
 
-#include "of_ff.cuh"
+#include "of_fix.cuh"
 #include "of_krylov.cuh"
 
 namespace of {
@@ -477,66 +477,14 @@ static KState iterate_pcg(of_grid* g, int st_off, float* x, float* r, float* pa,
     return h;
 }
 
-// r = b - A x like OpResidual, with the Laplacian of x from its double-float split xf, summed on
-// the FP32 pipes and returned to FP64 for the rest: within ~1e-13 of the FP64 sweep's value
-// relative to the largest tap term, in half its time (the FP64 sweep is bound by GB300's FP64
-// rate).
-template <typename T64>
-struct OpResidualFF {
-    using TF = typename std::conditional<KT<T64>::cplx, FF2, FF>::type;
-    static constexpr int kClass = KT<T64>::cplx ? PC_COCG_F64 : PC_STENCIL_F64, kWords = 3;
-    const TF* xf;
-    const T64* x;
-    const T64* b;
-    T64* r;
-    KState* st;
-    RedCtx rc;
-    double a;
-    double2 Q;
-    bool direct, first;
-    long long n;
-    double acc[3];
-    __device__ bool begin() {
-        acc[0] = acc[1] = acc[2] = 0.0;
-        return !direct || first || st->done == 0.0;
-    }
-    __device__ TF load(long long i) const { return xf[i]; }
-    __device__ void store(long long i, TF, TF lap) {
-        const T64 rv = vsub(b[i], apply_A(x[i], ff_to(lap), a, Q));
-        r[i] = rv;
-        acc[0] += hn2(rv);
-        const double2 s = bil(rv, rv);
-        acc[1] += s.x;
-        acc[2] += s.y;
-    }
-    __device__ void end() {
-        if (grid_reduce<3>(acc, rc.partials, rc.counter, st->red) &&
-            threadIdx.x == 0 && threadIdx.y == 0)
-            residual_finish(acc, st, direct, first, n);
-    }
-};
-
-// The double-float sweep's accuracy floor (~1e-13 of the largest tap term) sits well below the
-// tolerances it serves; tighter solves keep the FP64 sweep.
-constexpr double FF_MIN_TOL = 1e-11;
-
-// ff: the Laplacian in double-float arithmetic (the mixed-precision form's refinement
-// residuals); else in FP64
+// r = b - A x in FP64; direct: for the passes of a direct solve (OpResidualDirect)
 template <typename T>
 static void residual(of_grid* g, int st_off, const T* x, const T* b, T* r, double a, double2 Q,
-                     bool ff = false, bool direct = false, bool first = true) {
-    constexpr int RY = KT<T>::cplx ? 1 : 2;
-    if (ff) {
-        using TF = typename OpResidualFF<T>::TF;
-        const long long n = g->d.n;
-        TF* xf = (TF*)ws(g, WS_FF, sizeof(TF) * (size_t)n);
-        launch(k_ff_split<T, TF>, vec_blocks(n), 256, g->stream, n, x, xf);
-        OpResidualFF<T> op{xf, x, b, r, kstate(g, st_off), red_ctx(g, 0), a, Q, direct, first, n};
-        launch_stencil<TF, RY>(g, ff_weights(g->w64), op);
-        return;
-    }
-    OpResidual<T> op{x, b, r, kstate(g, st_off), red_ctx(g, 0), (typename KT<T>::R)a, Q, direct, first, g->d.n};
-    launch_stencil<T, RY>(g, g->w64, op);
+                     bool direct = false, bool first = true) {
+    if (direct)
+        launch_field<KT<T>::cplx>(g, OpResidualDirect<T>{x, b, r, kstate(g, st_off), red_ctx(g, 0), a, Q, first, g->d.n});
+    else
+        launch_field<KT<T>::cplx>(g, OpResidual<T>{x, b, r, kstate(g, st_off), red_ctx(g, 0), (typename KT<T>::R)a, Q});
 }
 
 // Whether the FP32 corrections of a mixed-precision solve are direct: the Poisson operator and
@@ -561,8 +509,7 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
     launch(k_init_state, 1, 1, g->stream, st, o.max_iter);
     launch(k_norm_to_tol<T64>, vec_blocks(n), 256, g->stream, n, b, o.tol, st, red_ctx(g, 0));
     OF_LAUNCH_CHECK();
-    const bool ff_res = o.precision == OF_F32 && o.tol >= FF_MIN_TOL;
-    residual<T64>(g, KS64, x, b, r, a, Q, ff_res, direct);
+    residual<T64>(g, KS64, x, b, r, a, Q, direct);
     // The direct solve's passes: each drops the residual by the FP32 rounding (1e-4 the first time,
     // 1e-6 once the residual is rough), so this many are queued before the host looks; those
     // after the one that converged find the done flag set and return.
@@ -570,7 +517,7 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
         for (; k > 0; --k) {
             if constexpr (std::is_same<T32, float2>::value) fft_correct_shifted(g, r, x, a, Q, st);
             else fft_correct(g, r, x, st);
-            residual<T64>(g, KS64, x, b, r, a, Q, ff_res, true, false);
+            residual<T64>(g, KS64, x, b, r, a, Q, true, false);
         }
     };
     if (direct) direct_passes(std::min(o.max_iter, o.tol >= 1e-4 ? 1 : o.tol >= 1e-8 ? 2 : 3));
@@ -674,7 +621,7 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
             if (hi.done == -1.0) {
                 // one read-back for both states: the inner pass and the true residual after it
                 // (a pass that broke down at its start has a zero correction)
-                residual<T64>(g, KS64, x, b, r, a, Q, ff_res);
+                residual<T64>(g, KS64, x, b, r, a, Q);
                 static_assert(KS32 > KS64, "KState layout");
                 double both[KS32 - KS64 + KSTATE_DOUBLES];
                 fetch_scalars(g, KS64, KS32 - KS64 + KSTATE_DOUBLES, both);
@@ -704,7 +651,7 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
             }
         }
         if (!residual_done) {
-            residual<T64>(g, KS64, x, b, r, a, Q, ff_res);   // true residual; restarts the recurrence
+            residual<T64>(g, KS64, x, b, r, a, Q);   // true residual; restarts the recurrence
             fetch_scalars(g, KS64, KSTATE_DOUBLES, (double*)&h);
         }
         ++refinements;

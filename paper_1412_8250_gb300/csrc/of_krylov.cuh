@@ -137,13 +137,9 @@ struct OpResidual {
     RedCtx rc;
     typename KT<T>::R a;
     double2 Q;
-    bool direct, first;      // residual_finish; a direct residual after the first is skipped once done
-    long long n;
     double acc[3];
-    __device__ bool begin() {
-        acc[0] = acc[1] = acc[2] = 0.0;
-        return !direct || first || st->done == 0.0;
-    }
+    __device__ bool begin() { acc[0] = acc[1] = acc[2] = 0.0; return true; }
+    __host__ __device__ const double* field() const { return reinterpret_cast<const double*>(x); }
     __device__ T load(long long i) const { return x[i]; }
     __device__ void store(long long i, T c, T lap) {
         const T rv = vsub(b[i], apply_A(c, lap, a, Q));
@@ -156,7 +152,50 @@ struct OpResidual {
     __device__ void end() {
         if (grid_reduce<3>(acc, rc.partials, rc.counter, st->red) &&
             threadIdx.x == 0 && threadIdx.y == 0)
-            residual_finish(acc, st, direct, first, n);
+            residual_finish(acc, st, false, true, 0);
+    }
+};
+
+// The residual of the direct solves' passes (skipped once the state is done): r = b + L x for the
+// Poisson operator, r = b + a L x - Q x for a shifted one, and |r|^2 alone: FP64 operations
+// count (2 per clock and SM), so nothing that the passes do not use is formed.
+template <typename T>
+struct OpResidualDirect {
+    static constexpr int kClass = KT<T>::cplx ? PC_COCG_F64 : PC_STENCIL_F64, kWords = 3;
+    const T* x;
+    const T* b;
+    T* r;
+    KState* st;
+    RedCtx rc;
+    double a;
+    double2 Q;
+    bool first;
+    long long n;
+    double acc[1];
+    __device__ bool begin() {
+        acc[0] = 0.0;
+        return first || st->done == 0.0;
+    }
+    __host__ __device__ const double* field() const { return reinterpret_cast<const double*>(x); }
+    __device__ T load(long long i) const { return x[i]; }
+    __device__ void store(long long i, T c, T lap) {
+        if constexpr (KT<T>::cplx) {
+            const double2 bi = b[i];
+            const double2 rv = make_double2(fma(a, lap.x, bi.x) - fma(Q.x, c.x, -Q.y * c.y),
+                                            fma(a, lap.y, bi.y) - fma(Q.x, c.y, Q.y * c.x));
+            r[i] = rv;
+            acc[0] = fma(rv.x, rv.x, fma(rv.y, rv.y, acc[0]));
+        } else {
+            const double rv = b[i] + lap;
+            r[i] = rv;
+            acc[0] = fma(rv, rv, acc[0]);
+        }
+    }
+    __device__ void end() {
+        if (grid_reduce<1>(acc, rc.partials, rc.counter, st->red) && threadIdx.x == 0 && threadIdx.y == 0) {
+            const double s[3] = {acc[0], 0.0, 0.0};
+            residual_finish(s, st, true, first, n);
+        }
     }
 };
 

@@ -24,6 +24,7 @@
 #include <thread>
 #include <vector>
 
+#include "of_fix.cuh"
 #include "of_functional.cuh"
 #include "of_pool.cuh"
 #include "of_stencil.cuh"
@@ -70,6 +71,7 @@ struct OpHamiltonian {
     RedCtx rc;
     double acc[2];
     __device__ bool begin() { acc[0] = acc[1] = 0.0; return true; }
+    __host__ __device__ const double* field() const { return u; }
     __device__ double load(long long i) const { return __ldg(u + i); }
     __device__ void store(long long i, double c, double lap) {
         const double rho = c * c;
@@ -95,6 +97,7 @@ struct OpLapDot {
     RedCtx rc;
     double acc[2];
     __device__ bool begin() { acc[0] = acc[1] = 0.0; return true; }
+    __host__ __device__ const double* field() const { return d; }
     __device__ double load(long long i) const { return __ldg(d + i); }
     __device__ void store(long long i, double c, double lap) {
         Ld[i] = lap;
@@ -110,6 +113,7 @@ struct OpScaledLap {
     double* y;
     double scale;
     __device__ bool begin() { return true; }
+    __host__ __device__ const double* field() const { return x; }
     __device__ double load(long long i) const { return __ldg(x + i); }
     __device__ void store(long long i, double, double lap) { y[i] = scale * lap; }
     __device__ void end() {}
@@ -123,6 +127,7 @@ struct OpEnergy {
     RedCtx rc;
     double acc[4];
     __device__ bool begin() { acc[0] = acc[1] = acc[2] = acc[3] = 0.0; return true; }
+    __host__ __device__ const double* field() const { return u; }
     __device__ double load(long long i) const { return __ldg(u + i); }
     __device__ void store(long long i, double c, double lap) {
         const double rho = c * c;
@@ -899,8 +904,7 @@ static bool nlcg(of_grid* g, const FnParams& fn, double Ne, ScfVecs& v, double* 
     double rr_prev = 0.0, s_prev = 1e-2, c_prev = 0.0;
     bool converged = false;
     for (int q = 0; q <= max_iter; ++q) {
-        launch_stencil<double, 2>(g, g->w64,
-                                  OpHamiltonian{u, phi, fn.mu != 0.0 ? V : nullptr, v.Hu, v.Lu, fn,
+        launch_field<false>(g, OpHamiltonian{u, phi, fn.mu != 0.0 ? V : nullptr, v.Hu, v.Lu, fn,
                                                 red_ctx(g, SC_UHU)});
         launch(k_gradient, nb, 256, g->stream, n, v.Hu, u, g->s.scalars + SC_UHU, dV / Ne,
                                               q > 0 ? v.rp : nullptr, v.r, red_ctx(g, SC_RR));
@@ -974,7 +978,7 @@ static bool nlcg(of_grid* g, const FnParams& fn, double Ne, ScfVecs& v, double* 
             pl.tol = std::max(po.tol, tol_line);
             // L d with d^T L d and u^T L d (slots untouched by the solves) beside the twin's solve
             poisson_pair(g, u, v.d, v.B, v.d, v.d, v.C, pl, st, [&](of_grid* h) {
-                launch_stencil<double, 2>(h, h->w64, OpLapDot{v.d, u, v.Ld, red_ctx(h, SC_DLD)});
+                launch_field<false>(h, OpLapDot{v.d, u, v.Ld, red_ctx(h, SC_DLD)});
             });
             launch(k_line_moments, nb, 256, g->stream, n, u, v.d, fn.mu != 0.0 ? V : nullptr, phi,
                    v.D, v.B, v.C, v.b, red_ctx(g, SC_MD));
@@ -1143,8 +1147,8 @@ static double lr_potential_l2(of_grid* g, const of_functional* fn, double kf2, c
     double* f00 = scratch + 6 * n;   // -(1/kf2) L_h u^{2 alpha}, -(1/kf2) L_h u^{2 beta}
     launch(k_powers6, nb, 256, g->stream, n, u, 2.0 * fn->alpha, 2.0 * fn->beta, gp);
     OF_LAUNCH_CHECK();
-    launch_stencil<double, 2>(g, g->w64, OpScaledLap{gp, f00, -1.0 / kf2});
-    launch_stencil<double, 2>(g, g->w64, OpScaledLap{gp + 3 * n, f00 + n, -1.0 / kf2});
+    launch_field<false>(g, OpScaledLap{gp, f00, -1.0 / kf2});
+    launch_field<false>(g, OpScaledLap{gp + 3 * n, f00 + n, -1.0 / kf2});
     // the solves, one per potential and conjugate pair, two at a time (run_pair)
     const int njobs = S.npot * npairs;
     auto solve = [&](of_grid* h, int job, of_solve_info& si) {
@@ -1191,8 +1195,8 @@ static double lr_potential_impl(of_grid* g, const of_functional* fn, double kf2,
     launch(k_powers, nb, 256, g->stream, n, u, 2.0 * fn->alpha, 2.0 * fn->beta, ga, gb);
     OF_LAUNCH_CHECK();
     // f_e = -(1/kf2) L u^{2e}  (the m = n = 0 right-hand side of Sec. 3.1)
-    launch_stencil<double, 2>(g, g->w64, OpScaledLap{ga, fa, -1.0 / kf2});
-    launch_stencil<double, 2>(g, g->w64, OpScaledLap{gb, fb, -1.0 / kf2});
+    launch_field<false>(g, OpScaledLap{ga, fa, -1.0 / kf2});
+    launch_field<false>(g, OpScaledLap{gb, fb, -1.0 / kf2});
     PairPtrs W{};
     W.npairs = npairs;
     // the shifted solves (two exponents x npairs shifts), up to GROUP_MAX at once on the grid
@@ -1316,7 +1320,7 @@ static double grad_sq_sum(of_grid* g, const double* u) {
 static void energy_terms(of_grid* g, const of_functional* fn, const double* u, const double* b,
                          const double* phi, double t_lr_sum, double e_self, double e_c,
                          int vw_energy, of_scf_result* res) {
-    launch_stencil<double, 2>(g, g->w64, OpEnergy{u, b, phi, red_ctx(g, SC_EN)});
+    launch_field<false>(g, OpEnergy{u, b, phi, red_ctx(g, SC_EN)});
     double e[4];
     fetch_scalars(g, SC_EN, 4, e);
     const double dV = g->dV;
@@ -1512,8 +1516,7 @@ of_status of_hamiltonian_apply(of_grid* g, const of_functional* fn, const double
         return OF_EINVAL;
     }
     try {
-        launch_stencil<double, 2>(g, g->w64,
-                                  OpHamiltonian{u, phi, fn->mu != 0.0 ? vlr : nullptr, hu, nullptr,
+        launch_field<false>(g, OpHamiltonian{u, phi, fn->mu != 0.0 ? vlr : nullptr, hu, nullptr,
                                                 fn_params(fn), red_ctx(g, SC_UHU)});
         return OF_OK;
     } catch (const Error& e) {
