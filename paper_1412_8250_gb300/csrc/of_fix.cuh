@@ -13,12 +13,12 @@
 // Brick of 16 units x 8 rows x 8 planes per block of 128 threads, a unit being two neighbouring
 // doubles of a row (two real points, or one complex point).  The brick and its x-y halo are staged
 // once in shared memory as fixed point; each thread takes the z halo of its own column straight
-// from global memory.  The block's exponent is
-// two above the largest of its z halo and first staged third.  A staged value beyond that, a value
-// that is not finite, or a stretch of staged values (2 x 1 x 8 points) that is not zero but 2^6 and
-// more below the largest, for which 60 bits would keep less than the 53 of FP64, makes the block
-// take FP64 arithmetic instead.  So a value's error is at most 2^-53 of the largest value of its
-// stretch, and ordinary fields take the integer path everywhere.
+// from global memory.  The block's exponent is one above the largest of its z halo and of eight
+// staged rows spread over the brick.  A staged value beyond that, a value that is not finite, or a
+// stretch of staged values (8 x 1 x 8 points) that is not zero but 2^6 and more below the largest,
+// for which 60 bits would keep less than the 53 of FP64, makes the block take FP64 arithmetic
+// instead.  So a value's error is at most 2^-53 of the largest value of its stretch, and ordinary
+// fields take the integer path everywhere.
 //
 // Measured on a GB300 (order 12): 96^3 69.1 -> 12.7 us, 320^3 2.4 ms -> 0.41 ms (13.7 -> 80 GPts/s); now
 // bound by instruction issue and latency at 12 warps per SM (157 registers; 4.9 staged values per
@@ -79,7 +79,6 @@ struct FixAcc {
 };
 
 constexpr int FX_UX = 16, FX_BY = 8, FX_THREADS = FX_UX * FX_BY;
-template <int N> struct FixDepth { static constexpr int value = 8; };   // planes per brick
 
 struct FixScale {
     double s[3];   // 2^fix_shift / (D h_a^2)
@@ -87,9 +86,9 @@ struct FixScale {
 
 template <int N, bool CPLX>
 constexpr int fix_row_width() { return 32 + 2 * (CPLX ? 2 * N : ((N + 1) & ~1)); }
-template <int N, bool CPLX>
+template <int N, bool CPLX, int BZ>
 constexpr size_t fix_smem_bytes() {
-    return sizeof(long long) * (size_t)FixDepth<N>::value * (FX_BY + 2 * N) * fix_row_width<N, CPLX>();
+    return sizeof(long long) * (size_t)BZ * (FX_BY + 2 * N) * fix_row_width<N, CPLX>();
 }
 
 // The Laplacian at the planes k < nz of a thread's two columns, from the fixed-point column (z) and
@@ -167,39 +166,54 @@ __device__ __forceinline__ void fix_planes(const longlong2 (&col)[BZ + 2 * N], c
     }
 }
 
-template <int N, bool CPLX, bool ISO, class Op>
+template <int N, bool CPLX, bool ISO, int BZ, class Op>
 __global__ void __launch_bounds__(FX_THREADS, 3)
 fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int bricks, Op op) {
     pdl_enter();
     if (!op.begin()) return;
-    constexpr int BZ = FixDepth<N>::value;
     constexpr int HX = CPLX ? 2 * N : ((N + 1) & ~1);   // staged halo doubles each side in x
     constexpr int RW = fix_row_width<N, CPLX>();
     constexpr int ROWS = FX_BY + 2 * N;
     constexpr int CPL = ROWS * RW;
-    constexpr int XC = RW / 2;                          // two-double chunks of a core row
-    constexpr int SLOTS = 2 * N * FX_UX + FX_BY * XC;   // halo rows: core columns only
+    // slots: the core columns of every staged row (16 chunks of two doubles), then the x halo of the
+    // core rows (PH lanes per side, of which HX / 2 hold a chunk)
+    constexpr int PH = (HX / 2 + 3) / 4 * 4;
+    constexpr int SLOTS = ROWS * FX_UX + FX_BY * 2 * PH;
     constexpr int SPT = (SLOTS + FX_THREADS - 1) / FX_THREADS;
+    constexpr bool ALL = SPT * BZ <= 8;   // thin bricks: every slot's loads in flight at once
     extern __shared__ __align__(16) long long fix_smem[];
     __shared__ int yoff[ROWS], zoff[BZ + 2 * N], xoff[RW];   // periodic offsets in doubles (< 2^31)
     __shared__ int wmax[FX_THREADS / 32];
     const double* x = op.field();
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + FX_UX * ty;
     const int RF = CPLX ? 2 * d.n1 : d.n1, PF = RF * d.n2;
-    // staged row and first column of each of this thread's slots
+    // Staged row and first column of each of this thread's slots.  The first FX_BY rows of the order
+    // are spread evenly over the staged rows, so that the first slot's values (from which, with
+    // the z halo, the block's exponent comes) sample the whole brick.
     int srow[SPT], scol[SPT];
 #pragma unroll
     for (int m = 0; m < SPT; ++m) {
         const int sl = tid + m * FX_THREADS;
-        if (sl < FX_BY * XC) {
-            srow[m] = N + sl / XC;
-            scol[m] = 2 * (sl % XC);
-        } else {
-            const int hr = (sl - FX_BY * XC) / FX_UX;
-            srow[m] = hr < N ? hr : hr + FX_BY;
-            scol[m] = HX + 2 * ((sl - FX_BY * XC) % FX_UX);
+        srow[m] = -1;
+        scol[m] = 0;
+        if (sl < ROWS * FX_UX) {
+            int j = sl / FX_UX;
+            auto spread = [](int i) { return (i * (ROWS - 1) + 3) / (FX_BY - 1); };
+            if (j < FX_BY) {
+                srow[m] = spread(j);
+            } else {
+                j -= FX_BY;   // the j-th row that is not one of those
+                for (int i = 0; i < FX_BY; ++i) j += spread(i) <= j;
+                srow[m] = j;
+            }
+            scol[m] = HX + 2 * (sl % FX_UX);
+        } else if (sl < SLOTS) {
+            const int q = sl - ROWS * FX_UX, side = (q / PH) & 1, c = q % PH;
+            if (c < HX / 2) {
+                srow[m] = N + q / (2 * PH);
+                scol[m] = 2 * c + (side ? HX + 32 : 0);
+            }
         }
-        if (sl >= SLOTS) srow[m] = -1;
     }
     // two doubles of a chunk: one 16-byte load where rows and the field allow it (a chunk
     // starts at an even double and is contiguous across the wrap when rows are even)
@@ -224,7 +238,7 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
         // exponent among them, plus two, is the block's
         const int own = yoff[N + ty], oc0 = xoff[HX + 2 * tx], oc1 = xoff[HX + 2 * tx + 1];
         longlong2 col[BZ + 2 * N];
-        double2 v[BZ];
+        double2 v[ALL ? SPT : 1][BZ];
         auto load_slot = [&](int m, double2 (&v)[BZ]) {
             if (srow[m] < 0) return;
             const int o = yoff[srow[m]], c0 = xoff[scol[m]], c1 = xoff[scol[m] + 1];
@@ -235,40 +249,49 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
         double2 zr[2 * N];
 #pragma unroll
         for (int j = 0; j < 2 * N; ++j) zr[j] = load2(zoff[j < N ? j : j + BZ] + own, oc0, oc1);
-        load_slot(0, v);
+#pragma unroll
+        for (int m = 0; m < (ALL ? SPT : 1); ++m) load_slot(m, v[m]);
         int emax = 0;
 #pragma unroll
         for (int j = 0; j < 2 * N; ++j) emax = max(emax, top(zr[j]));
 #pragma unroll
-        for (int k = 0; k < BZ; ++k) emax = max(emax, top(v[k]));
+        for (int m = 0; m < (ALL ? SPT : 1); ++m)
+            if (srow[m] >= 0) {
+#pragma unroll
+                for (int k = 0; k < BZ; ++k) emax = max(emax, top(v[m][k]));
+            }
         emax = __reduce_max_sync(0xffffffffu, emax);
         if ((tid & 31) == 0) wmax[tid >> 5] = emax;
         __syncthreads();
 #pragma unroll
         for (int w = 0; w < FX_THREADS / 32; ++w) emax = max(emax, wmax[w]);
-        const int E = max(emax + 2, 128);   // 128: zeros stay zeros, what else is that small takes FP64
+        const int E = max(emax + 1, 128);   // 128: zeros stay zeros, what else is that small takes FP64
         bool bad = E > 2046;
         auto fix = [&](double2 q) {
             return make_longlong2(fix_from_bits(__double2hiint(q.x), (unsigned)__double2loint(q.x), E),
                                   fix_from_bits(__double2hiint(q.y), (unsigned)__double2loint(q.y), E));
         };
         auto stage = [&](int m, double2 (&v)[BZ]) {
-            if (srow[m] < 0) return;
-            int lo = 0;   // largest exponent of the stretch
-            long long* dst = fix_smem + srow[m] * RW + scol[m];
+            int lo = 0;   // largest exponent of the stretch: this slot's planes in four neighbouring lanes
+            if (srow[m] >= 0) {
+                long long* dst = fix_smem + srow[m] * RW + scol[m];
 #pragma unroll
-            for (int k = 0; k < BZ; ++k) {
-                lo = max(lo, top(v[k]));
-                *reinterpret_cast<longlong2*>(dst + k * CPL) = fix(v[k]);
+                for (int k = 0; k < BZ; ++k) {
+                    lo = max(lo, top(v[k]));
+                    *reinterpret_cast<longlong2*>(dst + k * CPL) = fix(v[k]);
+                }
             }
-            bad |= lo > E || (lo != 0 && lo < E - 7);
+            bad |= lo > E;
+            lo = max(lo, __shfl_xor_sync(0xffffffffu, lo, 1));
+            lo = max(lo, __shfl_xor_sync(0xffffffffu, lo, 2));
+            bad |= lo != 0 && lo < E - 7;
         };
 #pragma unroll
         for (int j = 0; j < 2 * N; ++j) col[j < N ? j : j + BZ] = fix(zr[j]);
 #pragma unroll
         for (int m = 0; m < SPT; ++m) {
-            if (m > 0) load_slot(m, v);
-            stage(m, v);
+            if (!ALL && m > 0) load_slot(m, v[0]);
+            stage(m, v[ALL ? m : 0]);
         }
         const bool fp64 = __syncthreads_or(bad) != 0;
         const int y = y0 + ty, xe = x0 + 2 * tx;         // first double of this thread's unit
@@ -313,26 +336,36 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
     op.end();
 }
 
-template <int N, bool CPLX, bool ISO, class Op>
+template <int N, bool CPLX, bool ISO, int BZ, class Op>
 void launch_fix_kernel(of_grid* g, const FixScale& fs, Op op) {
     const Dims& d = g->d;
     const long long RF = CPLX ? 2LL * d.n1 : d.n1;
     const bool vec = RF % 2 == 0 && ((uintptr_t)op.field() & 15) == 0;
     const int bx = (int)((RF + 31) / 32), by = (d.n2 + FX_BY - 1) / FX_BY;
-    const int bricks = bx * by * ((d.n3 + FixDepth<N>::value - 1) / FixDepth<N>::value);
+    const int bricks = bx * by * ((d.n3 + BZ - 1) / BZ);
     // one block per brick, up to the reductions' limit
     const unsigned grid = (unsigned)std::min(bricks, OF_MAX_RED_BLOCKS);
-    constexpr size_t smem = fix_smem_bytes<N, CPLX>();
+    constexpr size_t smem = fix_smem_bytes<N, CPLX, BZ>();
     if constexpr (smem > 40 * 1024) {
         static thread_local int configured_device = -1;
         if (configured_device != g->device) {
-            OF_CUDA(cudaFuncSetAttribute(fix_kernel<N, CPLX, ISO, Op>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            OF_CUDA(cudaFuncSetAttribute(fix_kernel<N, CPLX, ISO, BZ, Op>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem));
             configured_device = g->device;
         }
     }
-    launch_pdl(fix_kernel<N, CPLX, ISO, Op>, dim3(grid), dim3(FX_UX, FX_BY), smem, g->stream, d, g->w64, fs, vec, bx,
-               by, bricks, op);
+    launch_pdl(fix_kernel<N, CPLX, ISO, BZ, Op>, dim3(grid), dim3(FX_UX, FX_BY), smem, g->stream, d, g->w64, fs, vec,
+               bx, by, bricks, op);
+}
+
+// Bricks of 8 planes, or of 2 where those leave most SMs without a block (32^3: 16 bricks of 8
+// planes 8.1 us, 64 of 2 planes 4.0 us)
+template <int N, bool CPLX, bool ISO, class Op>
+void launch_fix_depth(of_grid* g, const FixScale& fs, Op op) {
+    const Dims& d = g->d;
+    const long long bricks = ((CPLX ? 2LL : 1LL) * d.n1 + 31) / 32 * ((d.n2 + FX_BY - 1) / FX_BY) * ((d.n3 + 7) / 8);
+    if (bricks < num_sms()) launch_fix_kernel<N, CPLX, ISO, 2>(g, fs, op);
+    else launch_fix_kernel<N, CPLX, ISO, 8>(g, fs, op);
 }
 
 // Sweeps a plain FP64 field (op.field(): the doubles of a real or, CPLX, an interleaved complex
@@ -350,12 +383,12 @@ void launch_field(of_grid* g, Op op) {
     for (int a = 0; a < 3; ++a) fs.s[a] = std::ldexp(1.0, fix_shift(g->N)) / (fix_denominator(g->N) * g->h[a] * g->h[a]);
     const bool iso = fs.s[0] == fs.s[1] && fs.s[1] == fs.s[2];
     switch (g->N * 2 + (iso ? 1 : 0)) {
-        case 2: launch_fix_kernel<1, CPLX, false>(g, fs, op); break;
-        case 3: launch_fix_kernel<1, CPLX, true>(g, fs, op); break;
-        case 6: launch_fix_kernel<3, CPLX, false>(g, fs, op); break;
-        case 7: launch_fix_kernel<3, CPLX, true>(g, fs, op); break;
-        case 12: launch_fix_kernel<6, CPLX, false>(g, fs, op); break;
-        case 13: launch_fix_kernel<6, CPLX, true>(g, fs, op); break;
+        case 2: launch_fix_depth<1, CPLX, false>(g, fs, op); break;
+        case 3: launch_fix_depth<1, CPLX, true>(g, fs, op); break;
+        case 6: launch_fix_depth<3, CPLX, false>(g, fs, op); break;
+        case 7: launch_fix_depth<3, CPLX, true>(g, fs, op); break;
+        case 12: launch_fix_depth<6, CPLX, false>(g, fs, op); break;
+        case 13: launch_fix_depth<6, CPLX, true>(g, fs, op); break;
         default: OF_REQUIRE(false, OF_EINVAL, "unsupported finite-difference half order %d", g->N);
     }
 }
