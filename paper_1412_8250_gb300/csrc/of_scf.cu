@@ -376,25 +376,26 @@ __global__ void __launch_bounds__(256) k_lr_assemble2(long long n, const double*
 
 // V_LR = C_F [alpha u^{2(alpha-1)} V_beta + beta u^{2(beta-1)} V_alpha], V_e = sum over
 // conjugate pairs of 2 Re W ; sum of u^{2 alpha} V_beta + u^{2 beta} V_alpha.
+// ga and gb are the powers u^{2 alpha} and u^{2 beta} of k_powers.
 struct PairPtrs {
     const double2* Wa[4];
     const double2* Wb[4];
     int npairs;
 };
-__global__ void __launch_bounds__(256) k_lr_assemble(long long n, const double* u, PairPtrs W,
-                                                     double alpha, double beta, double* vlr,
-                                                     RedCtx rc) {
+__global__ void __launch_bounds__(256) k_lr_assemble(long long n, const double* u, const double* ga,
+                                                     const double* gb, PairPtrs W, double alpha,
+                                                     double beta, double* vlr, RedCtx rc) {
     double acc[1] = {0.0};
     GRID_LOOP(i, n) {
         double Va = 0.0, Vb = 0.0;
         for (int k = 0; k < W.npairs; ++k) {
-            Va += 2.0 * W.Wa[k][i].x;
-            Vb += 2.0 * W.Wb[k][i].x;
+            Va += W.Wa[k][i].x;
+            Vb += W.Wb[k][i].x;
         }
         const double uf = fmax(u[i], OF_U_FLOOR);
-        const double ra = pow(uf, 2.0 * alpha), rb = pow(uf, 2.0 * beta);
-        vlr[i] = OF_CF * (alpha * (ra / (uf * uf)) * Vb + beta * (rb / (uf * uf)) * Va);
-        acc[0] += ra * Vb + rb * Va;
+        const double ab = 2.0 * (ga[i] * Vb), ba = 2.0 * (gb[i] * Va);
+        vlr[i] = OF_CF * fma(alpha, ab, beta * ba) / (uf * uf);
+        acc[0] += ab + ba;
     }
     grid_reduce<1>(acc, rc.partials, rc.counter, rc.out);
 }
@@ -1224,7 +1225,7 @@ static double lr_potential_impl(of_grid* g, const of_functional* fn, double kf2,
             add_info(info_out, si[q]);
         }
     }
-    launch(k_lr_assemble, nb, 256, g->stream, n, u, W, fn->alpha, fn->beta, vlr, red_ctx(g, SC_TLR));
+    launch(k_lr_assemble, nb, 256, g->stream, n, u, (const double*)ga, (const double*)gb, W, fn->alpha, fn->beta, vlr, red_ctx(g, SC_TLR));
     OF_LAUNCH_CHECK();
     return sc(g, SC_TLR);
 }
