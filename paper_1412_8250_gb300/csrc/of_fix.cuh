@@ -78,6 +78,29 @@ struct FixAcc {
     }
 };
 
+// A sweep's field: a plain one (op.field()), or one the op forms on load, two doubles at a time
+// (op.pair(i0, i1, vec), neighbours or, vec, one 16-byte load; op.bits(): the OR of its addresses).
+template <class Op, class = void>
+struct HasPair { static constexpr bool value = false; };
+template <class Op>
+struct HasPair<Op, decltype((void)std::declval<const Op&>().pair(0u, 0u, true), void())> {
+    static constexpr bool value = true;
+};
+__device__ __forceinline__ double2 fix_pair(const double* x, unsigned i0, unsigned i1, bool vec) {
+    if (vec) return *reinterpret_cast<const double2*>(x + i0);
+    return make_double2(x[i0], x[i1]);
+}
+template <class Op>
+__device__ __forceinline__ double2 fix_load(const Op& op, unsigned i0, unsigned i1, bool vec) {
+    if constexpr (HasPair<Op>::value) return op.pair(i0, i1, vec);
+    else return fix_pair(op.field(), i0, i1, vec);
+}
+template <class Op>
+uintptr_t fix_bits(const Op& op) {
+    if constexpr (HasPair<Op>::value) return op.bits();
+    else return (uintptr_t)op.field();
+}
+
 constexpr int FX_UX = 16, FX_BY = 8, FX_THREADS = FX_UX * FX_BY;
 
 struct FixScale {
@@ -184,7 +207,6 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
     extern __shared__ __align__(16) long long fix_smem[];
     __shared__ int yoff[ROWS], zoff[BZ + 2 * N], xoff[RW];   // periodic offsets in doubles (< 2^31)
     __shared__ int wmax[FX_THREADS / 32];
-    const double* x = op.field();
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + FX_UX * ty;
     const int RF = CPLX ? 2 * d.n1 : d.n1, PF = RF * d.n2;
     // Staged row and first column of each of this thread's slots.  The first FX_BY rows of the order
@@ -218,8 +240,7 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
     // two doubles of a chunk: one 16-byte load where rows and the field allow it (a chunk
     // starts at an even double and is contiguous across the wrap when rows are even)
     auto load2 = [&](int base, int x0, int x1) -> double2 {
-        if (vec) return *reinterpret_cast<const double2*>(x + (unsigned)(base + x0));
-        return make_double2(x[(unsigned)(base + x0)], x[(unsigned)(base + x1)]);
+        return fix_load(op, (unsigned)(base + x0), (unsigned)(base + x1), vec);
     };
     auto expo = [](double a) { return (__double2hiint(a) >> 20) & 0x7ff; };
 
@@ -318,18 +339,22 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
             constexpr int XS = CPLX ? 2 : 1;
             const int cx = HX + 2 * tx, ry = N + ty;
             for (int k = 0; k < nz; ++k) {
-                double l[2];
-                for (int q = 0; q < 2; ++q) {
-                    auto at = [&](int j, int r, int c) { return x[(unsigned)(zoff[j] + yoff[r] + xoff[c + q])]; };
-                    double acc = W.centre * at(N + k, ry, cx);
-                    for (int p = 1; p <= N; ++p) {
-                        acc = fma(W.w[2][p], at(N + k + p, ry, cx) + at(N + k - p, ry, cx), acc);
-                        acc = fma(W.w[0][p], at(N + k, ry, cx + p * XS) + at(N + k, ry, cx - p * XS), acc);
-                        acc = fma(W.w[1][p], at(N + k, ry + p, cx) + at(N + k, ry - p, cx), acc);
-                    }
-                    l[q] = acc;
+                auto at = [&](int j, int r, int c) {
+                    const int o = zoff[j] + yoff[r];
+                    return fix_load(op, (unsigned)(o + xoff[c]), (unsigned)(o + xoff[c + 1]), false);
+                };
+                double2 acc = at(N + k, ry, cx);
+                acc = make_double2(W.centre * acc.x, W.centre * acc.y);
+                auto tap = [&](double w, double2 a, double2 b) {
+                    acc.x = fma(w, a.x + b.x, acc.x);
+                    acc.y = fma(w, a.y + b.y, acc.y);
+                };
+                for (int p = 1; p <= N; ++p) {
+                    tap(W.w[2][p], at(N + k + p, ry, cx), at(N + k - p, ry, cx));
+                    tap(W.w[0][p], at(N + k, ry, cx + p * XS), at(N + k, ry, cx - p * XS));
+                    tap(W.w[1][p], at(N + k, ry + p, cx), at(N + k, ry - p, cx));
                 }
-                put(k, l[0], l[1]);
+                put(k, acc.x, acc.y);
             }
         }
     }
@@ -340,7 +365,7 @@ template <int N, bool CPLX, bool ISO, int BZ, class Op>
 void launch_fix_kernel(of_grid* g, const FixScale& fs, Op op) {
     const Dims& d = g->d;
     const long long RF = CPLX ? 2LL * d.n1 : d.n1;
-    const bool vec = RF % 2 == 0 && ((uintptr_t)op.field() & 15) == 0;
+    const bool vec = RF % 2 == 0 && (fix_bits(op) & 15) == 0;
     const int bx = (int)((RF + 31) / 32), by = (d.n2 + FX_BY - 1) / FX_BY;
     const int bricks = bx * by * ((d.n3 + BZ - 1) / BZ);
     // one block per brick, up to the reductions' limit
@@ -368,8 +393,8 @@ void launch_fix_depth(of_grid* g, const FixScale& fs, Op op) {
     else launch_fix_kernel<N, CPLX, ISO, 8>(g, fs, op);
 }
 
-// Sweeps a plain FP64 field (op.field(): the doubles of a real or, CPLX, an interleaved complex
-// field; op.load / op.store as for the other sweeps) of the grid with the fixed-point kernel.
+// Sweeps an FP64 field of the grid (the doubles of a real or, CPLX, an interleaved complex field;
+// op.load / op.store as for the other sweeps) with the fixed-point kernel.
 template <bool CPLX, class Op>
 void launch_field(of_grid* g, Op op) {
     if ((CPLX ? 2 : 1) * g->d.n >= (1LL << 31)) {   // beyond the kernel's 32-bit offsets

@@ -279,7 +279,8 @@ static void krylov_step(of_grid* g, KState* st, T* x, T* r, T* pin, T* pout, T* 
     const long long n = g->d.n;
     constexpr int RY = KT<T>::cplx ? 1 : 2;
     OpKrylovA<T> op{r, pin, pout, Ap, st, red_ctx(g, 0), a, Q};
-    launch_stencil<T, RY>(g, W, op);
+    if constexpr (sizeof(typename KT<T>::R) == 8) launch_field<KT<T>::cplx>(g, op);
+    else launch_stencil<T, RY>(g, W, op);
     ProfScope ps(g, PC_UPDATE, 6.0 * sizeof(T) * (double)n);
     launch_krylov_update<T, false>(g, n, x, r, pout, Ap, st, red_ctx(g, 0), vec_blocks(n));
 }

@@ -7,7 +7,7 @@
 #include <cstring>
 #include <vector>
 
-#include "of_stencil.cuh"
+#include "of_fix.cuh"
 
 namespace of {
 
@@ -223,10 +223,25 @@ struct OpKrylovA {
         accp[0] = accp[1] = 0;
         return true;
     }
-    // p = (r - zshift) + beta p_in ; zshift is 0 except in the projected PCG
+    // p = (r - zshift) + beta p_in ; zshift is 0 except in the projected PCG (FP32)
     __device__ T load(long long i) const {
-        return vadd(vadd(r[i], cs_mul(shift, one<T>())), cs_mul(beta, pin[i]));
+        if constexpr (std::is_same<T, double>::value) return fma(beta.x, pin[i], r[i]);
+        else if constexpr (std::is_same<T, double2>::value) return combine(r[i], pin[i]);
+        else return vadd(vadd(r[i], cs_mul(shift, one<T>())), cs_mul(beta, pin[i]));
     }
+    __device__ double2 combine(double2 rv, double2 pv) const {
+        return make_double2(fma(beta.x, pv.x, fma(-beta.y, pv.y, rv.x)),
+                            fma(beta.x, pv.y, fma(beta.y, pv.x, rv.y)));
+    }
+    // FP64: two doubles of p for the fixed-point sweep
+    template <typename U = T, typename = std::enable_if_t<sizeof(typename KT<U>::R) == 8>>
+    __device__ double2 pair(unsigned i0, unsigned i1, bool vec) const {
+        const double2 rv = fix_pair(reinterpret_cast<const double*>(r), i0, i1, vec);
+        const double2 pv = fix_pair(reinterpret_cast<const double*>(pin), i0, i1, vec);
+        if constexpr (KT<T>::cplx) return combine(rv, pv);
+        else return make_double2(fma(beta.x, pv.x, rv.x), fma(beta.x, pv.y, rv.y));
+    }
+    uintptr_t bits() const { return (uintptr_t)r | (uintptr_t)pin; }
     template <typename U = T, typename = std::enable_if_t<std::is_same<U, float>::value>>
     __device__ float2 load2(long long i) const {
         const float2 rv = *reinterpret_cast<const float2*>(r + i);
@@ -236,11 +251,18 @@ struct OpKrylovA {
     }
     __device__ void store(long long i, T c, T lap) {
         pout[i] = c;
-        const T av = apply_A(c, lap, a, Q);
-        Ap[i] = av;
-        const auto s = bilf(c, av);
-        accp[0] += s.x;
-        accp[1] += s.y;
+        T av;
+        if constexpr (std::is_same<T, double>::value) {   // FP64 operations count: fused, and real
+            av = fma(Q.x, c, -a * lap);
+            Ap[i] = av;
+            accp[0] = fma(c, av, accp[0]);
+        } else {
+            av = apply_A(c, lap, a, Q);
+            Ap[i] = av;
+            const auto s = bilf(c, av);
+            accp[0] += s.x;
+            accp[1] += s.y;
+        }
     }
     // points i, i + 1 of a real field (i even): the same as two store calls
     template <typename U = T, typename = std::enable_if_t<std::is_same<U, float>::value>>
@@ -300,6 +322,7 @@ __device__ __forceinline__ void krylov_update_finish(const double (&acc)[3], KSt
 }
 
 // x += alpha p ; r -= alpha Ap ; reduces |r|^2 and r^T r ; sets beta, iteration count, done.
+// Four points per thread with their loads in flight at once; one sum where r^T r = |r|^2.
 template <typename T, bool PRECOND = false>
 __global__ void __launch_bounds__(256) krylov_update(long long n, T* __restrict__ x,
                                                      T* __restrict__ r, const T* __restrict__ p,
@@ -307,23 +330,48 @@ __global__ void __launch_bounds__(256) krylov_update(long long n, T* __restrict_
                                                      RedCtx rc) {
     pdl_enter();
     if (st->done != 0.0) return;
+    constexpr bool ONE = PRECOND || !KT<T>::cplx;
     const double2 al = make_double2(st->alpha_re, st->alpha_im);
     typename AccT<typename KT<T>::R>::type a0 = 0, a1 = 0, a2 = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        x[i] = vadd(x[i], cs_mul(al, p[i]));
-        const T rv = vsub(r[i], cs_mul(al, Ap[i]));
-        r[i] = rv;
-        a0 += hn2f(rv);
-        if (!PRECOND) {
-            const auto s = bilf(rv, rv);
-            a1 += s.x;
-            a2 += s.y;
+    for (long long i0 = blockIdx.x * 1024LL + threadIdx.x; i0 < n; i0 += gridDim.x * 1024LL) {
+        T xv[4], rv[4], pv[4], av[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const long long i = i0 + 256 * k;
+            if (i < n) {
+                xv[k] = x[i];
+                rv[k] = r[i];
+                pv[k] = p[i];
+                av[k] = Ap[i];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const long long i = i0 + 256 * k;
+            if (i < n) {
+                x[i] = vadd(xv[k], cs_mul(al, pv[k]));
+                const T v = vsub(rv[k], cs_mul(al, av[k]));
+                r[i] = v;
+                a0 += hn2f(v);
+                if (!ONE) {
+                    const auto s = bilf(v, v);
+                    a1 += s.x;
+                    a2 += s.y;
+                }
+            }
         }
     }
-    double acc[3] = {(double)a0, (double)a1, (double)a2};
-    if (grid_reduce<3>(acc, rc.partials, rc.counter, st->red) && threadIdx.x == 0)
-        krylov_update_finish<PRECOND>(acc, st);
+    if constexpr (ONE) {
+        double acc[1] = {(double)a0};
+        if (grid_reduce<1>(acc, rc.partials, rc.counter, st->red) && threadIdx.x == 0) {
+            const double s[3] = {acc[0], acc[0], 0.0};
+            krylov_update_finish<PRECOND>(s, st);
+        }
+    } else {
+        double acc[3] = {(double)a0, (double)a1, (double)a2};
+        if (grid_reduce<3>(acc, rc.partials, rc.counter, st->red) && threadIdx.x == 0)
+            krylov_update_finish<PRECOND>(acc, st);
+    }
 }
 
 // The same for FP32 fields (real, or complex as float2) moved as 16-byte vectors: nv = the
