@@ -27,7 +27,7 @@ namespace of {
 
 struct Fft {
     bool ok = false;
-    FftPlan plan[3];
+    FftPlan plan[3], z_back;   // z_back: the radices of plan[2] reversed
     const float* sym[3];     // l_a(k), k < n_a
 };
 
@@ -75,6 +75,9 @@ static Fft& fft_tables(of_grid* g) {
         f.plan[a].tw = (const float2*)(dev + off[a]);
         f.sym[a] = dev + off[3 + a];
     }
+    int back[FFT_MAX_STAGES];
+    for (int s = 0; s < f.plan[2].nst; ++s) back[s] = f.plan[2].r[f.plan[2].nst - 1 - s];
+    fft_plan_of(n[2], f.plan[2].nst, back, f.z_back);
     f.ok = true;
     return f;
 }
@@ -288,45 +291,70 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_inverse(FftPlan P, int lg
     }
 }
 
-// Lines with stride: column c of `cols` starts at (c / group) * gstride + c % group, its points
-// are `stride` apart (y: group = nh, gstride = n2 nh, stride = nh; z: group = cols, stride = cols).
+// y lines: column c of `cols` starts at (c / group) * gstride + c % group, its points are `stride`
+// apart (group = nh, gstride = n2 nh, stride = nh)
 struct FftCols {
     long long cols, group, gstride, stride;
 };
 
-__device__ __forceinline__ void cols_load(const float2* F, const FftCols& C, int n, int lg, bool act,
-                                          long long base, bool swap, float2* A) {
-    const int line = threadIdx.x & ((1 << lg) - 1);
-#pragma unroll 4
-    for (int i = threadIdx.x >> lg; i < n; i += blockDim.x >> lg) {
-        const float2 v = act ? F[base + i * C.stride] : make_float2(0.f, 0.f);
-        A[(i << lg) + line] = swap ? make_float2(v.y, v.x) : v;
+// The points of this thread's column in global memory, real and imaginary part swapped or not;
+// columns beyond the last read zeros and store nothing
+struct FftGlobal {
+    float2* p;
+    long long stride;
+    bool act, swap;
+    __device__ float2 operator()(int, int i) const {
+        if (!act) return make_float2(0.f, 0.f);
+        const float2 v = p[i * stride];
+        return swap ? make_float2(v.y, v.x) : v;
     }
+    __device__ void operator()(int, int i, float2 v) const {
+        if (act) p[i * stride] = swap ? make_float2(v.y, v.x) : v;
+    }
+};
+
+// Whether a tile's first step reads and its last step writes global memory, so that a transform of
+// two steps passes shared memory once (320^3: y 83 -> 51 us, z 115 -> 86; 192^3 complex 28 -> 18 and
+// 41 -> 35; 96^3: y 4.4 -> 3.6).  Not with a prime factor above 10, and not where the steps have fewer
+// than 128 butterflies per tile: there all threads copying is the shorter chain (96^3 in tiles of 8
+// lines: z 7.0 against 5.6 us).
+__device__ __forceinline__ bool fft_straight(const FftPlan& P, int lg) {
+    return P.unrolled && P.nst > 1 && (P.T[0] << lg) >= 128;
 }
-__device__ __forceinline__ void cols_store(float2* F, const FftCols& C, int n, int lg, bool act, long long base,
-                                           bool swap, const float2* R) {
-    const int line = threadIdx.x & ((1 << lg) - 1);
-    if (!act) return;
+
+// A tile's lines from global memory and back.  tile: two tiles.
+__device__ __forceinline__ void fft_lines(const FftPlan& P, const FftGlobal& G, float2* tile, const float2* tw,
+                                          int lg) {
+    const int t = threadIdx.x, nt = blockDim.x, rs = 1 << lg, line = t & (rs - 1);
+    float2 *A = tile, *B = tile + (P.n << lg);
+    if (fft_straight(P, lg)) {
+        fft_step(P, 0, G, FftTile{A, rs}, tw, lg, t, nt);
+        __syncthreads();
+        for (int st = 1; st + 1 < P.nst; ++st) {
+            fft_step(P, st, FftTile{A, rs}, FftTile{B, rs}, tw, lg, t, nt);
+            __syncthreads();
+            float2* x = A;
+            A = B;
+            B = x;
+        }
+        fft_step(P, P.nst - 1, FftTile{A, rs}, G, tw, lg, t, nt);
+    } else {
 #pragma unroll 4
-    for (int i = threadIdx.x >> lg; i < n; i += blockDim.x >> lg) {
-        const float2 v = R[(i << lg) + line];
-        F[base + i * C.stride] = swap ? make_float2(v.y, v.x) : v;
+        for (int i = t >> lg; i < P.n; i += nt >> lg) A[(i << lg) + line] = G(line, i);
+        const float2* R = fft_tile(P, A, B, tw, rs, lg);
+        for (int i = t >> lg; i < P.n; i += nt >> lg) G(line, i, R[(i << lg) + line]);
     }
 }
 
-__global__ void __launch_bounds__(FFT_THREADS) k_fft_y(FftPlan P, int lg, FftCols C, float2* F, int inverse,
+// (one kernel for both directions: each launch starts with a cold instruction cache)
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_y(FftPlan P, int lg, FftCols C, float2* F, bool inverse,
                                                        const double* done) {
     pdl_enter();
     if (*done != 0.0) return;
     const float2* tw = fft_smem_tables(P);
-    float2* A = const_cast<float2*>(tw) + P.n;
-    float2* Bf = A + (P.n << lg);
     const long long col = ((long long)blockIdx.x << lg) + (threadIdx.x & ((1 << lg) - 1));
-    const bool act = col < C.cols;
     const long long grp = col / C.group, base = grp * C.gstride + (col - grp * C.group);
-    cols_load(F, C, P.n, lg, act, base, inverse != 0, A);
-    const float2* R = fft_tile(P, A, Bf, tw, 1 << lg, lg);
-    cols_store(F, C, P.n, lg, act, base, inverse != 0, R);
+    fft_lines(P, FftGlobal{F + base, C.stride, col < C.cols, inverse}, const_cast<float2*>(tw) + P.n, tw, lg);
 }
 
 // symbol of the inverse: kind 0: 1 / l (0 for the constant mode); 1: 1 / (l + s1);
@@ -335,52 +363,77 @@ struct FftFilter {
     int kind;
     float a, qr, qi, s0, s1, norm;
     const float *lx, *ly, *lz;
+    // v times the symbol at eigenvalue l, real and imaginary part swapped
+    __device__ __forceinline__ float2 apply(float l, float2 v) const {
+        if (kind == 3) {
+            const float dr = fmaf(a, l, qr), di = qi;
+            const float den = fmaf(dr, dr, di * di);
+            const float m = den > 1e-30f ? norm / den : 0.f;   // a singular mode is left alone
+            const float gr = dr * m, gi = -di * m;
+            return make_float2(gr * v.y + gi * v.x, gr * v.x - gi * v.y);
+        }
+        float m;
+        if (kind == 0) {
+            m = l > 0.f ? norm / l : 0.f;
+        } else {
+            const float q = 1.f / (l + s1);
+            m = norm * q;
+            if (kind == 2) m *= (l + s0) * q;
+        }
+        return make_float2(m * v.y, m * v.x);
+    }
 };
 
-// z lines: forward, times the symbol, inverse
-__global__ void __launch_bounds__(FFT_THREADS) k_fft_z_filter(FftPlan P, int lg, FftCols C, int nh, float2* F,
-                                                              FftFilter f, const double* done) {
+// z lines: forward (plan P), times the symbol, inverse (plan Q, the radices of P reversed: its first
+// step starts from the results the last step of P leaves in registers)
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_z_filter(FftPlan P, FftPlan Q, int lg, long long cols, int nh,
+                                                              float2* F, FftFilter f, const double* done) {
     pdl_enter();
     if (*done != 0.0) return;
     const float2* tw = fft_smem_tables(P);
     float2* A = const_cast<float2*>(tw) + P.n;
-    float2* Bf = A + (P.n << lg);
-    const int line = threadIdx.x & ((1 << lg) - 1);
+    float2* B = A + (P.n << lg);
+    const int t = threadIdx.x, nt = blockDim.x, rs = 1 << lg, line = t & (rs - 1);
     const long long col = ((long long)blockIdx.x << lg) + line;
-    const bool act = col < C.cols;
-    cols_load(F, C, P.n, lg, act, col, false, A);
+    const bool act = col < cols;
     const int ky = act ? (int)(col / nh) : 0, kx = act ? (int)(col - (long long)ky * nh) : 0;
     const float lxy = f.lx[kx] + f.ly[ky];
-    for (int pass = 0; pass < 2; ++pass) {
-        float2* R = fft_tile(P, A, Bf, tw, 1 << lg, lg);
-        if (pass == 1) {
-            cols_store(F, C, P.n, lg, act, col, true, R);
-            break;
+    const FftGlobal in{F + col, cols, act, false};
+    const FftGlobal out{F + col, cols, act, true};
+    auto filter = [&](int i, float2 v) { return f.apply(lxy + f.lz[i], v); };
+    auto swap_tiles = [&]() {
+        __syncthreads();
+        float2* x = A;
+        A = B;
+        B = x;
+    };
+    if (fft_straight(P, lg)) {
+        fft_step(P, 0, in, FftTile{B, rs}, tw, lg, t, nt);
+        swap_tiles();
+        for (int st = 1; st + 1 < P.nst; ++st) {
+            fft_step(P, st, FftTile{A, rs}, FftTile{B, rs}, tw, lg, t, nt);
+            swap_tiles();
         }
-        for (int i = threadIdx.x >> lg; i < P.n; i += blockDim.x >> lg) {
-            const float2 v = R[(i << lg) + line];
-            const float l = lxy + f.lz[i];
-            float2 o;
-            if (f.kind == 3) {
-                const float dr = fmaf(f.a, l, f.qr), di = f.qi;
-                const float den = fmaf(dr, dr, di * di);
-                const float m = den > 1e-30f ? f.norm / den : 0.f;   // a singular mode is left alone
-                const float gr = dr * m, gi = -di * m;
-                o = make_float2(gr * v.x - gi * v.y, gr * v.y + gi * v.x);
-            } else {
-                float m;
-                if (f.kind == 0) m = l > 0.f ? f.norm / l : 0.f;
-                else {
-                    const float q = 1.f / (l + f.s1);
-                    m = f.norm * q;
-                    if (f.kind == 2) m *= (l + f.s0) * q;
-                }
-                o = make_float2(m * v.x, m * v.y);
+        fft_turn_step(P, FftTile{A, rs}, filter, FftTile{B, rs}, tw, lg, t, nt);
+        swap_tiles();
+        for (int st = 1; st + 1 < Q.nst; ++st) {
+            fft_step(Q, st, FftTile{A, rs}, FftTile{B, rs}, tw, lg, t, nt);
+            swap_tiles();
+        }
+        fft_step(Q, Q.nst - 1, FftTile{A, rs}, out, tw, lg, t, nt);
+    } else {
+#pragma unroll 4
+        for (int i = t >> lg; i < P.n; i += nt >> lg) A[(i << lg) + line] = in(line, i);
+        for (int pass = 0; pass < 2; ++pass) {
+            float2* R = fft_tile(P, A, B, tw, rs, lg);
+            for (int i = t >> lg; i < P.n; i += nt >> lg) {
+                const float2 v = R[(i << lg) + line];
+                if (pass) out(line, i, v);
+                else R[(i << lg) + line] = filter(i, v);
             }
-            R[(i << lg) + line] = make_float2(o.y, o.x);
+            B = R == A ? B : A;
+            A = R;
         }
-        Bf = R == A ? Bf : A;
-        A = R;
     }
 }
 
@@ -395,12 +448,15 @@ static void allow_smem(of_grid* g, const void* kernel, size_t smem) {
     raised.push_back(key);
 }
 
-// log2 of the lines per tile: 16, fewer for long lines (two tiles and the twiddles within 227 KB)
-// and where 16 would leave SMs without a block
+// log2 of the lines per tile: 16 while four blocks per SM fit beside each other in shared memory
+// (56 KB each) and every SM has one, else 8, and 4 for very long lines or very few.  320^3: x
+// 93 / 231 -> 72 / 142 us, y 118 -> 83, z 167 -> 115 from 16 to 8 lines; 192^3 complex: y 28, z 41 with
+// 16, 32 and 45 with 8.  8 lines below four blocks per SM took the x lines of one 96^3 solve from
+// 5.5 / 6.3 to 4.8 / 5.3 us but 12 cells on eight streams from 1.87 to 2.09 ms.
 static int tile_lg(int n, long long lines) {
-    int lg = n <= 512 ? 4 : n <= 1024 ? 3 : 2;
-    while (lg > 2 && (lines >> lg) < num_sms()) --lg;
-    return lg;
+    const long long sms = num_sms();
+    if (n * 35LL * (long long)sizeof(float2) <= 56 * 1024 && (lines >> 4) >= sms) return 4;
+    return n <= 1024 && (lines >> 3) >= sms ? 3 : 2;
 }
 
 template <bool CPLX, class LD, class ST>
@@ -424,17 +480,17 @@ static void fft_apply(of_grid* g, LD ld, ST st, FftFilter f, const double* done)
     const size_t sy = sizeof(float2) * (size_t)d.n2 * (1 + 2 * (1 << lgy));
     const size_t sz = sizeof(float2) * (size_t)d.n3 * (1 + 2 * (1 << lgz));
     const FftCols cy{(long long)nh * d.n3, nh, (long long)d.n2 * nh, nh};
-    const FftCols cz{(long long)nh * d.n2, (long long)nh * d.n2, 0, (long long)nh * d.n2};
+    const long long zc = (long long)nh * d.n2;
     allow_smem(g, (const void*)k_fft_x_forward<CPLX, LD>, sx);
     allow_smem(g, (const void*)k_fft_x_inverse<CPLX, ST>, sx);
     allow_smem(g, (const void*)k_fft_y, sy);
     allow_smem(g, (const void*)k_fft_z_filter, sz);
     launch_pdl(k_fft_x_forward<CPLX, LD>, blocks(xl, lgx), FFT_THREADS, sx, g->stream, T.plan[0], lgx, rows, nh, ld, F, done);
     if (d.n2 > 1)
-        launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, 0, done);
-    launch_pdl(k_fft_z_filter, blocks(cz.cols, lgz), FFT_THREADS, sz, g->stream, T.plan[2], lgz, cz, nh, F, f, done);
+        launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, false, done);
+    launch_pdl(k_fft_z_filter, blocks(zc, lgz), FFT_THREADS, sz, g->stream, T.plan[2], T.z_back, lgz, zc, nh, F, f, done);
     if (d.n2 > 1)
-        launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, 1, done);
+        launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, true, done);
     launch_pdl(k_fft_x_inverse<CPLX, ST>, blocks(xl, lgx), FFT_THREADS, sx, g->stream, T.plan[0], lgx, rows, nh,
                (const float2*)F, st, done);
 }

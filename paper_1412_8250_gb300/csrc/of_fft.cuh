@@ -18,8 +18,11 @@ namespace of {
 constexpr int FFT_MAX_N = 2048;      // points of one line (two tiles of lines in shared memory)
 constexpr int FFT_MAX_STAGES = 12;
 
+#define OF_HD __host__ __device__ __forceinline__
+
 struct FftPlan {
     int n, nst;
+    bool unrolled;                   // every radix is
     int r[FFT_MAX_STAGES];           // radix of each step
     int L[FFT_MAX_STAGES];           // product of the radices before it
     int T[FFT_MAX_STAGES];           // n / r
@@ -29,9 +32,7 @@ struct FftPlan {
     const float2* tw;                // exp(-2 pi i k / n), k < n
 };
 
-inline bool fft_unrolled(int r) { return (r >= 2 && r <= 10) || r == 12 || r == 16; }
-
-#define OF_HD __host__ __device__ __forceinline__
+OF_HD bool fft_unrolled(int r) { return (r >= 2 && r <= 10) || r == 12 || r == 16; }
 
 OF_HD unsigned fft_mulhi(unsigned a, unsigned b) {
 #ifdef __CUDA_ARCH__
@@ -166,14 +167,14 @@ template <> struct Dft<10> : DftPair<2, 5> {};
 template <> struct Dft<12> : DftPair<4, 3> {};
 template <> struct Dft<16> : DftPair<4, 4> {};
 
-// One butterfly of an unrolled step: line `line`, index b
-template <int R>
-OF_HD void fft_butterfly(const float2* in, float2* out, const float2* tw, int L, int T, int tl, unsigned mL,
-                         int rs, int line, int b) {
+// One butterfly of an unrolled step: line `line`, index b, from src(line, i) to dst(line, i, v)
+template <int R, class Src, class Dst>
+OF_HD void fft_butterfly(const Src& src, const Dst& dst, const float2* tw, int L, int T, int tl, unsigned mL, int line,
+                         int b) {
     const int p = fft_div(b, mL), q = b - p * L;
     float2 v[R];
 #pragma unroll
-    for (int s = 0; s < R; ++s) v[s] = in[(b + s * T) * rs + line];
+    for (int s = 0; s < R; ++s) v[s] = src(line, b + s * T);
     if (L > 1) {
         const int step = q * tl;
 #pragma unroll
@@ -182,7 +183,26 @@ OF_HD void fft_butterfly(const float2* in, float2* out, const float2* tw, int L,
     Dft<R>::run(v);
     const int o = p * L * R + q;
 #pragma unroll
-    for (int s = 0; s < R; ++s) out[(o + s * L) * rs + line] = v[s];
+    for (int s = 0; s < R; ++s) dst(line, o + s * L, v[s]);
+}
+
+// The last step of a transform, mid(i, X_i) on its results, and the first step of a transform of
+// those (whose first radix is the same): index b's results b + s T are that step's inputs.
+template <int R, class Src, class Mid, class Dst>
+OF_HD void fft_turn(const Src& src, const Mid& mid, const Dst& dst, const float2* tw, int T, int line, int b) {
+    float2 v[R];
+#pragma unroll
+    for (int s = 0; s < R; ++s) v[s] = src(line, b + s * T);
+    if (T > 1) {
+#pragma unroll
+        for (int s = 1; s < R; ++s) v[s] = cxmul(v[s], tw[s * b]);
+    }
+    Dft<R>::run(v);
+#pragma unroll
+    for (int s = 0; s < R; ++s) v[s] = mid(b + s * T, v[s]);
+    Dft<R>::run(v);
+#pragma unroll
+    for (int s = 0; s < R; ++s) dst(line, b * R + s, v[s]);
 }
 
 // One output of a step with a large prime radix r: u = s T + b
@@ -203,35 +223,76 @@ OF_HD void fft_direct_output(const float2* in, float2* out, const float2* tw, in
     out[(p * L * r + q + s * L) * rs + line] = acc;
 }
 
-// One step for the work items first, first + stride, ... (item = butterfly or output of a line,
+// Points of a tile in shared memory
+struct FftTile {
+    float2* p;
+    int rs;
+    OF_HD float2 operator()(int line, int i) const { return p[i * rs + line]; }
+    OF_HD void operator()(int line, int i, float2 v) const { p[i * rs + line] = v; }
+};
+
+// f(constant R) for the unrolled radix r
+#define OF_FFT_RADIX(r, CALL)                                                                   \
+    switch (r) {                                                                                \
+        case 2: { constexpr int R = 2; CALL; } break;                                           \
+        case 3: { constexpr int R = 3; CALL; } break;                                           \
+        case 4: { constexpr int R = 4; CALL; } break;                                           \
+        case 5: { constexpr int R = 5; CALL; } break;                                           \
+        case 6: { constexpr int R = 6; CALL; } break;                                           \
+        case 7: { constexpr int R = 7; CALL; } break;                                           \
+        case 8: { constexpr int R = 8; CALL; } break;                                           \
+        case 9: { constexpr int R = 9; CALL; } break;                                           \
+        case 10: { constexpr int R = 10; CALL; } break;                                         \
+        case 12: { constexpr int R = 12; CALL; } break;                                         \
+        case 16: { constexpr int R = 16; CALL; } break;                                         \
+        default: break;                                                                         \
+    }
+
+// One unrolled step for the work items first, first + stride, ... (item = butterfly of a line,
 // line fastest: line = item mod 2^lg)
-template <int R>
-OF_HD void fft_step(const FftPlan& P, int st, const float2* in, float2* out, const float2* tw, int rs, int lg,
-                    int first, int stride) {
-    const int items = P.T[st] << lg;
-    for (int w = first; w < items; w += stride)
-        fft_butterfly<R>(in, out, tw, P.L[st], P.T[st], P.tl[st], P.mL[st], rs, w & ((1 << lg) - 1), w >> lg);
+template <class Src, class Dst>
+OF_HD void fft_step(const FftPlan& P, int st, const Src& src, const Dst& dst, const float2* tw, int lg, int first,
+                    int stride) {
+    const int items = P.T[st] << lg, mask = (1 << lg) - 1;
+    OF_FFT_RADIX(P.r[st], for (int w = first; w < items; w += stride) fft_butterfly<R>(
+                              src, dst, tw, P.L[st], P.T[st], P.tl[st], P.mL[st], w & mask, w >> lg))
 }
+// fft_turn with the last step of P
+template <class Src, class Mid, class Dst>
+OF_HD void fft_turn_step(const FftPlan& P, const Src& src, const Mid& mid, const Dst& dst, const float2* tw, int lg,
+                         int first, int stride) {
+    const int st = P.nst - 1, items = P.T[st] << lg, mask = (1 << lg) - 1;
+    OF_FFT_RADIX(P.r[st], for (int w = first; w < items; w += stride)
+                              fft_turn<R>(src, mid, dst, tw, P.T[st], w & mask, w >> lg))
+}
+// Any step between two tiles: unrolled, or one output per item
 OF_HD void fft_any_step(const FftPlan& P, int st, const float2* in, float2* out, const float2* tw, int rs, int lg,
                         int first, int stride) {
-    switch (P.r[st]) {
-        case 2: fft_step<2>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 3: fft_step<3>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 4: fft_step<4>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 5: fft_step<5>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 6: fft_step<6>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 7: fft_step<7>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 8: fft_step<8>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 9: fft_step<9>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 10: fft_step<10>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 12: fft_step<12>(P, st, in, out, tw, rs, lg, first, stride); break;
-        case 16: fft_step<16>(P, st, in, out, tw, rs, lg, first, stride); break;
-        default: {
-            const int items = P.n << lg;
-            for (int w = first; w < items; w += stride)
-                fft_direct_output(in, out, tw, P.n, P.r[st], P.L[st], P.T[st], P.tl[st], P.mL[st], P.mT[st], rs,
-                                  w & ((1 << lg) - 1), w >> lg);
-        }
+    if (fft_unrolled(P.r[st])) {
+        fft_step(P, st, FftTile{const_cast<float2*>(in), rs}, FftTile{out, rs}, tw, lg, first, stride);
+    } else {
+        const int items = P.n << lg;
+        for (int w = first; w < items; w += stride)
+            fft_direct_output(in, out, tw, P.n, P.r[st], P.L[st], P.T[st], P.tl[st], P.mL[st], P.mT[st], rs,
+                              w & ((1 << lg) - 1), w >> lg);
+    }
+}
+
+// The plan of n = r[0] r[1] .. r[k - 1], in that order
+inline void fft_plan_of(int n, int k, const int* r, FftPlan& P) {
+    P.n = n;
+    P.nst = k;
+    P.unrolled = true;
+    P.tw = nullptr;
+    auto magic = [](int d) { return d == 1 ? 0u : (unsigned)((1ull << 32) / (unsigned)d + 1); };
+    for (int s = 0, L = 1; s < k; L *= r[s++]) {
+        P.unrolled = P.unrolled && fft_unrolled(r[s]);
+        P.r[s] = r[s];
+        P.L[s] = L;
+        P.T[s] = n / r[s];
+        P.tl[s] = n / (r[s] * L);
+        P.mL[s] = magic(L);
+        P.mT[s] = magic(P.T[s]);
     }
 }
 
@@ -257,23 +318,12 @@ inline bool fft_make_plan(int n, FftPlan& P) {
             if (prime) take(r, 1.0 + 0.3 * r);
         }
     }
-    P.n = n;
-    P.nst = 0;
-    P.tw = nullptr;
-    int m = n, L = 1;
-    while (m > 1) {
-        if (P.nst == FFT_MAX_STAGES || first[m] < 2) return false;
-        const int k = P.nst++, r = first[m];
-        auto magic = [](int d) { return d == 1 ? 0u : (unsigned)((1ull << 32) / (unsigned)d + 1); };
-        P.r[k] = r;
-        P.L[k] = L;
-        P.T[k] = n / r;
-        P.tl[k] = n / (r * L);
-        P.mL[k] = magic(L);
-        P.mT[k] = magic(P.T[k]);
-        L *= r;
-        m /= r;
+    int r[FFT_MAX_STAGES], k = 0;
+    for (int m = n; m > 1; m /= first[m]) {
+        if (k == FFT_MAX_STAGES || first[m] < 2) return false;
+        r[k++] = first[m];
     }
+    fft_plan_of(n, k, r, P);
     return true;
 }
 
