@@ -9,7 +9,7 @@
 // each pass drops by the FP32 rounding (1e-4 .. 1e-6), where a multigrid-preconditioned Krylov
 // pass took 4 .. 30 iterations of ~17 dependent launches for the same drop.
 //
-// Five launches: x forward, y forward, z forward * symbol * z inverse, y inverse, x inverse,
+// Five launches (three on small planes, which x and y share): x forward, y forward, z forward * symbol * z inverse, y inverse, x inverse,
 // each moving the half spectrum once (4 B per point and direction; 8 B for complex fields).
 // Real fields: two x rows are the real and imaginary part of one line, separated into
 // their half spectra (n1 / 2 + 1 points) on the way out and combined again on the way back.
@@ -166,10 +166,12 @@ __device__ __forceinline__ float2* fft_smem_tables(const FftPlan& P) {
 
 // All steps of the tile in a (other buffer b); returns the buffer that holds the result.  The
 // caller's writes to a are made visible here.
-__device__ __forceinline__ float2* fft_tile(const FftPlan& P, float2* a, float2* b, const float2* tw, int rs, int lg) {
+template <class Map>
+__device__ __forceinline__ float2* fft_tile(const FftPlan& P, float2* a, float2* b, const float2* tw, int rs, int ls,
+                                            const Map& map) {
     __syncthreads();
     for (int st = 0; st < P.nst; ++st) {
-        fft_any_step(P, st, a, b, tw, rs, lg, threadIdx.x, blockDim.x);
+        fft_any_step(P, st, FftTile{a, rs, ls}, FftTile{b, rs, ls}, tw, map, threadIdx.x, blockDim.x);
         __syncthreads();
         float2* t = a;
         a = b;
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_forward(FftPlan P, int lg
                 A[i * rs + l] = make_float2(ld.at(r * n + i), two ? ld.at((r + 1) * n + i) : 0.f);
         }
     }
-    const float2* R = fft_tile(P, A, Bf, tw, rs, lg);
+    const float2* R = fft_tile(P, A, Bf, tw, rs, 1, FftPow2{lg});
     for (int l = warp; l < TX; l += nw) {
         if constexpr (CPLX) {
             const long long r = row0 + l;
@@ -267,7 +269,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_x_inverse(FftPlan P, int lg
             }
         }
     }
-    const float2* R = fft_tile(P, A, Bf, tw, rs, lg);
+    const float2* R = fft_tile(P, A, Bf, tw, rs, 1, FftPow2{lg});
     for (int l = warp; l < TX; l += nw) {
         if constexpr (CPLX) {
             const long long r = row0 + l;
@@ -328,20 +330,20 @@ __device__ __forceinline__ void fft_lines(const FftPlan& P, const FftGlobal& G, 
     const int t = threadIdx.x, nt = blockDim.x, rs = 1 << lg, line = t & (rs - 1);
     float2 *A = tile, *B = tile + (P.n << lg);
     if (fft_straight(P, lg)) {
-        fft_step(P, 0, G, FftTile{A, rs}, tw, lg, t, nt);
+        fft_step(P, 0, G, FftTile{A, rs}, tw, FftPow2{lg}, t, nt);
         __syncthreads();
         for (int st = 1; st + 1 < P.nst; ++st) {
-            fft_step(P, st, FftTile{A, rs}, FftTile{B, rs}, tw, lg, t, nt);
+            fft_step(P, st, FftTile{A, rs}, FftTile{B, rs}, tw, FftPow2{lg}, t, nt);
             __syncthreads();
             float2* x = A;
             A = B;
             B = x;
         }
-        fft_step(P, P.nst - 1, FftTile{A, rs}, G, tw, lg, t, nt);
+        fft_step(P, P.nst - 1, FftTile{A, rs}, G, tw, FftPow2{lg}, t, nt);
     } else {
 #pragma unroll 4
         for (int i = t >> lg; i < P.n; i += nt >> lg) A[(i << lg) + line] = G(line, i);
-        const float2* R = fft_tile(P, A, B, tw, rs, lg);
+        const float2* R = fft_tile(P, A, B, tw, rs, 1, FftPow2{lg});
         for (int i = t >> lg; i < P.n; i += nt >> lg) G(line, i, R[(i << lg) + line]);
     }
 }
@@ -408,24 +410,24 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_z_filter(FftPlan P, FftPlan
         B = x;
     };
     if (fft_straight(P, lg)) {
-        fft_step(P, 0, in, FftTile{B, rs}, tw, lg, t, nt);
+        fft_step(P, 0, in, FftTile{B, rs}, tw, FftPow2{lg}, t, nt);
         swap_tiles();
         for (int st = 1; st + 1 < P.nst; ++st) {
-            fft_step(P, st, FftTile{A, rs}, FftTile{B, rs}, tw, lg, t, nt);
+            fft_step(P, st, FftTile{A, rs}, FftTile{B, rs}, tw, FftPow2{lg}, t, nt);
             swap_tiles();
         }
-        fft_turn_step(P, FftTile{A, rs}, filter, FftTile{B, rs}, tw, lg, t, nt);
+        fft_turn_step(P, FftTile{A, rs}, filter, FftTile{B, rs}, tw, FftPow2{lg}, t, nt);
         swap_tiles();
         for (int st = 1; st + 1 < Q.nst; ++st) {
-            fft_step(Q, st, FftTile{A, rs}, FftTile{B, rs}, tw, lg, t, nt);
+            fft_step(Q, st, FftTile{A, rs}, FftTile{B, rs}, tw, FftPow2{lg}, t, nt);
             swap_tiles();
         }
-        fft_step(Q, Q.nst - 1, FftTile{A, rs}, out, tw, lg, t, nt);
+        fft_step(Q, Q.nst - 1, FftTile{A, rs}, out, tw, FftPow2{lg}, t, nt);
     } else {
 #pragma unroll 4
         for (int i = t >> lg; i < P.n; i += nt >> lg) A[(i << lg) + line] = in(line, i);
         for (int pass = 0; pass < 2; ++pass) {
-            float2* R = fft_tile(P, A, B, tw, rs, lg);
+            float2* R = fft_tile(P, A, B, tw, rs, 1, FftPow2{lg});
             for (int i = t >> lg; i < P.n; i += nt >> lg) {
                 const float2 v = R[(i << lg) + line];
                 if (pass) out(line, i, v);
@@ -433,6 +435,118 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_z_filter(FftPlan P, FftPlan
             }
             B = R == A ? B : A;
             A = R;
+        }
+    }
+}
+
+// ------------------------------------------------------------------- x and y in one launch
+// A z plane per block, for planes whose two buffers fit shared memory: the x lines (real: pairs of
+// rows) and then the y lines of the half spectrum without a pass over global memory between.
+constexpr int FFT_PLANE_THREADS = 512;
+
+struct FftPlane {
+    FftPlan px, py;
+    FftAny mx, my;      // lines of the two phases
+    int rx, ry;         // strides of a point: x phase [i][line], y phase [row][k]
+    int buf;            // points of one buffer
+    int n2, nh;
+};
+
+template <bool CPLX, class LD>
+__global__ void __launch_bounds__(FFT_PLANE_THREADS) k_fft_xy_forward(FftPlane G, LD ld, float2* __restrict__ out,
+                                                                      const double* done) {
+    pdl_enter();
+    if (*done != 0.0) return;
+    ld.begin();
+    const int n1 = G.px.n, n2 = G.n2, nh = G.nh;
+    float2* tx = fft_smem_tables(G.px);
+    float2* ty = tx + n1;
+    for (int k = threadIdx.x; k < n2; k += blockDim.x) ty[k] = G.py.tw[k];
+    float2 *A = ty + n2, *B = A + G.buf;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const long long row0 = (long long)blockIdx.x * n2;
+    for (int l = warp; l < G.mx.m; l += nw) {
+        const long long r = CPLX ? row0 + l : row0 + 2 * l;
+        const bool two = !CPLX && 2 * l + 1 < n2;
+#pragma unroll 4
+        for (int i = lane; i < n1; i += 32) {
+            if constexpr (CPLX) A[i * G.rx + l] = ld.at(r * n1 + i);
+            else A[i * G.rx + l] = make_float2(ld.at(r * n1 + i), two ? ld.at((r + 1) * n1 + i) : 0.f);
+        }
+    }
+    float2* R = fft_tile(G.px, A, B, tx, G.rx, 1, G.mx);
+    float2* Y = R == A ? B : A;
+    const float2* Z;
+    int zi, zl;   // strides of a row and of k in Z
+    if constexpr (CPLX) {   // the x phase's lines are the y phase's points
+        Z = fft_tile(G.py, R, Y, ty, 1, G.rx, G.my);
+        zi = 1;
+        zl = G.rx;
+    } else {
+        for (int l = warp; l < G.mx.m; l += nw)
+            for (int k = lane; k < nh; k += 32) {
+                const float2 c = R[k * G.rx + l], d = R[(k == 0 ? 0 : n1 - k) * G.rx + l];
+                Y[2 * l * G.ry + k] = make_float2(0.5f * (c.x + d.x), 0.5f * (c.y - d.y));
+                if (2 * l + 1 < n2) Y[(2 * l + 1) * G.ry + k] = make_float2(0.5f * (c.y + d.y), 0.5f * (d.x - c.x));
+            }
+        Z = fft_tile(G.py, Y, R, ty, G.ry, 1, G.my);
+        zi = G.ry;
+        zl = 1;
+    }
+    for (int j = warp; j < n2; j += nw)
+#pragma unroll 4
+        for (int k = lane; k < nh; k += 32) out[(row0 + j) * nh + k] = Z[j * zi + k * zl];
+}
+
+template <bool CPLX, class ST>
+__global__ void __launch_bounds__(FFT_PLANE_THREADS) k_fft_xy_inverse(FftPlane G, const float2* __restrict__ in, ST st,
+                                                                      const double* done) {
+    pdl_enter();
+    if (*done != 0.0) return;
+    st.begin();
+    const int n1 = G.px.n, n2 = G.n2, nh = G.nh;
+    float2* tx = fft_smem_tables(G.px);
+    float2* ty = tx + n1;
+    for (int k = threadIdx.x; k < n2; k += blockDim.x) ty[k] = G.py.tw[k];
+    float2 *A = ty + n2, *B = A + G.buf;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const long long row0 = (long long)blockIdx.x * n2;
+    const int zi = CPLX ? 1 : G.ry, zl = CPLX ? G.rx : 1;   // complex: already the x phase's tile
+    for (int j = warp; j < n2; j += nw)
+#pragma unroll 4
+        for (int k = lane; k < nh; k += 32) {
+            const float2 v = in[(row0 + j) * nh + k];
+            A[j * zi + k * zl] = make_float2(v.y, v.x);
+        }
+    float2* R = fft_tile(G.py, A, B, ty, zi, zl, G.my);
+    float2* X = R == A ? B : A;
+    const float2* Z;
+    if constexpr (CPLX) {
+        Z = fft_tile(G.px, R, X, tx, G.rx, 1, G.mx);
+    } else {
+        for (int l = warp; l < G.mx.m; l += nw)
+            for (int k = lane; k < nh; k += 32) {
+                float2 a = R[2 * l * G.ry + k];   // swapped
+                float2 b = 2 * l + 1 < n2 ? R[(2 * l + 1) * G.ry + k] : make_float2(0.f, 0.f);
+                const int m = k == 0 ? 0 : n1 - k;
+                if (m == k) a.x = b.x = 0.f;      // the spectrum of a real row is real there
+                X[k * G.rx + l] = make_float2(a.x + b.y, a.y - b.x);
+                if (m != k) X[m * G.rx + l] = make_float2(b.y - a.x, a.y + b.x);
+            }
+        Z = fft_tile(G.px, X, R, tx, G.rx, 1, G.mx);
+    }
+    for (int l = warp; l < G.mx.m; l += nw) {
+        const long long r = CPLX ? row0 + l : row0 + 2 * l;
+        const bool two = !CPLX && 2 * l + 1 < n2;
+#pragma unroll 4
+        for (int i = lane; i < n1; i += 32) {
+            const float2 v = Z[i * G.rx + l];
+            if constexpr (CPLX) {
+                st.put(r * n1 + i, make_float2(v.y, v.x));
+            } else {
+                st.put(r * n1 + i, v.y);
+                if (two) st.put((r + 1) * n1 + i, v.x);
+            }
         }
     }
 }
@@ -447,6 +561,13 @@ static void allow_smem(of_grid* g, const void* kernel, size_t smem) {
     OF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     raised.push_back(key);
 }
+
+// x and y share a launch for planes of at most this shared memory (real 72^2, complex 52^2), of
+// which there are at least 16: two launches less pay while a launch is all latency (Poisson solve
+// 24^3 119 -> 106 us, 32^3 118 -> 109, 45 x 50 x 54 139 -> 131), but one block per plane leaves SMs idle
+// that the larger planes need (96^3 198 -> 202).
+constexpr size_t FFT_PLANE_SMEM = 48 * 1024;
+constexpr int FFT_MIN_PLANES = 16;
 
 // log2 of the lines per tile: 16 while four blocks per SM fit beside each other in shared memory
 // (56 KB each) and every SM has one, else 8, and 4 for very long lines or very few.  320^3: x
@@ -485,14 +606,38 @@ static void fft_apply(of_grid* g, LD ld, ST st, FftFilter f, const double* done)
     allow_smem(g, (const void*)k_fft_x_inverse<CPLX, ST>, sx);
     allow_smem(g, (const void*)k_fft_y, sy);
     allow_smem(g, (const void*)k_fft_z_filter, sz);
-    launch_pdl(k_fft_x_forward<CPLX, LD>, blocks(xl, lgx), FFT_THREADS, sx, g->stream, T.plan[0], lgx, rows, nh, ld, F, done);
-    if (d.n2 > 1)
-        launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, false, done);
+    FftPlane G;
+    G.px = T.plan[0];
+    G.py = T.plan[1];
+    G.mx.m = CPLX ? d.n2 : (d.n2 + 1) / 2;
+    G.my.m = G.nh = nh;
+    G.n2 = d.n2;
+    for (FftAny* m : {&G.mx, &G.my}) m->magic = m->m == 1 ? 0u : (unsigned)((1ull << 32) / (unsigned)m->m + 1);
+    G.rx = G.mx.m | 1;   // odd: a warp's points of one line fall into different banks
+    G.ry = nh | 1;
+    const long long buf = CPLX ? (long long)d.n1 * G.rx : std::max((long long)d.n1 * G.rx, (long long)d.n2 * G.ry);
+    const size_t sp = sizeof(float2) * (size_t)(d.n1 + d.n2 + 2 * buf);
+    G.buf = (int)buf;
+    const bool planes = d.n2 > 1 && d.n3 >= FFT_MIN_PLANES && sp <= FFT_PLANE_SMEM &&
+                        (long long)d.n1 * G.mx.m < 65536 && (long long)d.n2 * nh < 65536;
+    if (planes) {
+        allow_smem(g, (const void*)k_fft_xy_forward<CPLX, LD>, sp);
+        allow_smem(g, (const void*)k_fft_xy_inverse<CPLX, ST>, sp);
+        launch_pdl(k_fft_xy_forward<CPLX, LD>, d.n3, FFT_PLANE_THREADS, sp, g->stream, G, ld, F, done);
+    } else {
+        launch_pdl(k_fft_x_forward<CPLX, LD>, blocks(xl, lgx), FFT_THREADS, sx, g->stream, T.plan[0], lgx, rows, nh, ld, F, done);
+        if (d.n2 > 1)
+            launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, false, done);
+    }
     launch_pdl(k_fft_z_filter, blocks(zc, lgz), FFT_THREADS, sz, g->stream, T.plan[2], T.z_back, lgz, zc, nh, F, f, done);
-    if (d.n2 > 1)
-        launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, true, done);
-    launch_pdl(k_fft_x_inverse<CPLX, ST>, blocks(xl, lgx), FFT_THREADS, sx, g->stream, T.plan[0], lgx, rows, nh,
-               (const float2*)F, st, done);
+    if (planes) {
+        launch_pdl(k_fft_xy_inverse<CPLX, ST>, d.n3, FFT_PLANE_THREADS, sp, g->stream, G, (const float2*)F, st, done);
+    } else {
+        if (d.n2 > 1)
+            launch_pdl(k_fft_y, blocks(cy.cols, lgy), FFT_THREADS, sy, g->stream, T.plan[1], lgy, cy, F, true, done);
+        launch_pdl(k_fft_x_inverse<CPLX, ST>, blocks(xl, lgx), FFT_THREADS, sx, g->stream, T.plan[0], lgx, rows, nh,
+                   (const float2*)F, st, done);
+    }
 }
 
 void fft_correct(of_grid* g, const double* r, double* x, const KState* st) {

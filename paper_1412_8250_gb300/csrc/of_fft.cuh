@@ -1,7 +1,7 @@
 // Mixed-radix complex FFT of a tile of lines held in shared memory, FP32.
 //
-// A tile holds TX lines of n points as tile[i * rs + line] (line fastest), so that a warp's
-// accesses of one radix step are contiguous whatever the radix.  Stockham's autosort form:
+// A tile holds its lines of n points as tile[i * rs + line] (line fastest; or any two strides), so
+// that a warp's accesses of one radix step are contiguous whatever the radix.  Stockham's autosort form:
 // step with radix r after a product L of earlier radices takes, for b in [0, n/r), the points
 // b + s n/r (s < r), twiddles them by exp(-2 pi i q s / (L r)), q = b mod L, applies the r-point
 // DFT and writes the points (b / L) L r + q + s L of the other buffer; one barrier per step,
@@ -206,29 +206,44 @@ OF_HD void fft_turn(const Src& src, const Mid& mid, const Dst& dst, const float2
 }
 
 // One output of a step with a large prime radix r: u = s T + b
-OF_HD void fft_direct_output(const float2* in, float2* out, const float2* tw, int n, int r, int L, int T, int tl,
-                             unsigned mL, unsigned mT, int rs, int line, int u) {
+template <class Src, class Dst>
+OF_HD void fft_direct_output(const Src& src, const Dst& dst, const float2* tw, int n, int r, int L, int T, int tl,
+                             unsigned mL, unsigned mT, int line, int u) {
     const int s = fft_div(u, mT), b = u - s * T;
     const int p = fft_div(b, mL), q = b - p * L;
     const int step = (s * T + q * tl) % n;
     float2 acc = make_float2(0.f, 0.f);
     int k = 0;
     for (int t = 0; t < r; ++t) {
-        const float2 x = in[(b + t * T) * rs + line], w = tw[k];
+        const float2 x = src(line, b + t * T), w = tw[k];
         acc.x = fmaf(x.x, w.x, fmaf(-x.y, w.y, acc.x));
         acc.y = fmaf(x.x, w.y, fmaf(x.y, w.x, acc.y));
         k += step;
         if (k >= n) k -= n;
     }
-    out[(p * L * r + q + s * L) * rs + line] = acc;
+    dst(line, p * L * r + q + s * L, acc);
 }
 
-// Points of a tile in shared memory
+// Points of a tile in shared memory: point i of a line at p[i * rs + line * ls]
 struct FftTile {
     float2* p;
-    int rs;
-    OF_HD float2 operator()(int line, int i) const { return p[i * rs + line]; }
-    OF_HD void operator()(int line, int i, float2 v) const { p[i * rs + line] = v; }
+    int rs, ls = 1;
+    OF_HD float2 operator()(int line, int i) const { return p[i * rs + line * ls]; }
+    OF_HD void operator()(int line, int i, float2 v) const { p[i * rs + line * ls] = v; }
+};
+
+// The lines of a tile, and how a work item splits into a line (fastest) and the rest: a power of two
+// of them, or any number m
+struct FftPow2 {
+    int lg;
+    OF_HD int lines() const { return 1 << lg; }
+    OF_HD int rest(int w) const { return w >> lg; }
+};
+struct FftAny {
+    int m;
+    unsigned magic;   // floor(2^32 / m) + 1 (0 for m = 1): exact for items below 2^16
+    OF_HD int lines() const { return m; }
+    OF_HD int rest(int w) const { return fft_div(w, magic); }
 };
 
 // f(constant R) for the unrolled radix r
@@ -248,33 +263,38 @@ struct FftTile {
         default: break;                                                                         \
     }
 
-// One unrolled step for the work items first, first + stride, ... (item = butterfly of a line,
-// line fastest: line = item mod 2^lg)
-template <class Src, class Dst>
-OF_HD void fft_step(const FftPlan& P, int st, const Src& src, const Dst& dst, const float2* tw, int lg, int first,
-                    int stride) {
-    const int items = P.T[st] << lg, mask = (1 << lg) - 1;
-    OF_FFT_RADIX(P.r[st], for (int w = first; w < items; w += stride) fft_butterfly<R>(
-                              src, dst, tw, P.L[st], P.T[st], P.tl[st], P.mL[st], w & mask, w >> lg))
+// One unrolled step for the work items first, first + stride, ... (item = butterfly of a line)
+template <class Map, class Src, class Dst>
+OF_HD void fft_step(const FftPlan& P, int st, const Src& src, const Dst& dst, const float2* tw, const Map& map,
+                    int first, int stride) {
+    const int nl = map.lines(), items = P.T[st] * nl;
+    OF_FFT_RADIX(P.r[st], for (int w = first; w < items; w += stride) {
+        const int b = map.rest(w);
+        fft_butterfly<R>(src, dst, tw, P.L[st], P.T[st], P.tl[st], P.mL[st], w - b * nl, b);
+    })
 }
 // fft_turn with the last step of P
-template <class Src, class Mid, class Dst>
-OF_HD void fft_turn_step(const FftPlan& P, const Src& src, const Mid& mid, const Dst& dst, const float2* tw, int lg,
-                         int first, int stride) {
-    const int st = P.nst - 1, items = P.T[st] << lg, mask = (1 << lg) - 1;
-    OF_FFT_RADIX(P.r[st], for (int w = first; w < items; w += stride)
-                              fft_turn<R>(src, mid, dst, tw, P.T[st], w & mask, w >> lg))
+template <class Map, class Src, class Mid, class Dst>
+OF_HD void fft_turn_step(const FftPlan& P, const Src& src, const Mid& mid, const Dst& dst, const float2* tw,
+                         const Map& map, int first, int stride) {
+    const int st = P.nst - 1, nl = map.lines(), items = P.T[st] * nl;
+    OF_FFT_RADIX(P.r[st], for (int w = first; w < items; w += stride) {
+        const int b = map.rest(w);
+        fft_turn<R>(src, mid, dst, tw, P.T[st], w - b * nl, b);
+    })
 }
-// Any step between two tiles: unrolled, or one output per item
-OF_HD void fft_any_step(const FftPlan& P, int st, const float2* in, float2* out, const float2* tw, int rs, int lg,
-                        int first, int stride) {
+// Any step between two tiles of the same strides: unrolled, or one output per item
+template <class Map>
+OF_HD void fft_any_step(const FftPlan& P, int st, const FftTile& in, const FftTile& out, const float2* tw,
+                        const Map& map, int first, int stride) {
     if (fft_unrolled(P.r[st])) {
-        fft_step(P, st, FftTile{const_cast<float2*>(in), rs}, FftTile{out, rs}, tw, lg, first, stride);
+        fft_step(P, st, in, out, tw, map, first, stride);
     } else {
-        const int items = P.n << lg;
-        for (int w = first; w < items; w += stride)
-            fft_direct_output(in, out, tw, P.n, P.r[st], P.L[st], P.T[st], P.tl[st], P.mL[st], P.mT[st], rs,
-                              w & ((1 << lg) - 1), w >> lg);
+        const int nl = map.lines(), items = P.n * nl;
+        for (int w = first; w < items; w += stride) {
+            const int u = map.rest(w);
+            fft_direct_output(in, out, tw, P.n, P.r[st], P.L[st], P.T[st], P.tl[st], P.mL[st], P.mT[st], w - u * nl, u);
+        }
     }
 }
 
