@@ -419,7 +419,7 @@ static of_status poisson_batched(int nc, of_grid* const* gs, const double* const
         // right-hand side 4 pi (rho - mean rho) in the cell's own arena
         const long long n = g->d.n;
         launch(k_sum_product, vec_blocks(n), 256, g->stream, n, rho[c], nullptr, red_ctx(g, 120));
-        launch(k_form_rhs, vec_blocks(n), 256, g->stream, n, rho[c], nullptr, g->s.scalars + 120,
+        launch(k_form_rhs, vec_blocks(n), 256, g->stream, n, 1.0 / (double)n, rho[c], nullptr, g->s.scalars + 120,
                4.0 * M_PI, C.b);
         max_vec = std::max(max_vec, n);
     }
@@ -522,7 +522,7 @@ static of_status poisson_batched(int nc, of_grid* const* gs, const double* const
         of_grid* g = gs[c];
         const long long n = g->d.n;
         launch(k_sum_product, vec_blocks(n), 256, g->stream, n, phi[c], nullptr, red_ctx(g, 120));
-        launch(k_sub_mean, vec_blocks(n), 256, g->stream, n, phi[c], g->s.scalars + 120);
+        launch(k_sub_mean, vec_blocks(n), 256, g->stream, n, 1.0 / (double)n, phi[c], g->s.scalars + 120);
         if (infos) {
             const double bb = h64[c].red[1];
             infos[c].iterations = iters[c];

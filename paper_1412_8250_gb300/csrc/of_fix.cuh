@@ -95,6 +95,14 @@ __device__ __forceinline__ double2 fix_load(const Op& op, unsigned i0, unsigned 
     if constexpr (HasPair<Op>::value) return op.pair(i0, i1, vec);
     else return fix_pair(op.field(), i0, i1, vec);
 }
+// What an op reads beside the field at a unit's points (op.pre(i, act0, act1), two neighbouring points
+// of a real field or one of a complex one): loaded a plane ahead, for op.store_pre.
+template <class Op, class = void>
+struct HasPre { static constexpr bool value = false; };
+template <class Op>
+struct HasPre<Op, decltype((void)std::declval<const Op&>().pre(0LL, true, true), void())> {
+    static constexpr bool value = true;
+};
 template <class Op>
 uintptr_t fix_bits(const Op& op) {
     if constexpr (HasPair<Op>::value) return op.bits();
@@ -115,17 +123,19 @@ constexpr size_t fix_smem_bytes() {
 }
 
 // The Laplacian at the planes k < nz of a thread's two columns, from the fixed-point column (z) and
-// tile (own: this unit's first value in the tile's first plane): put(k, l0, l1).  With equal
+// tile (own: this unit's first value in the tile's first plane): put(k, l0, l1), after
+// ahead(k + 1).  With equal
 // spacings the six neighbours at distance p are summed before the two multiplications by W_p
 // (s0 = s1 = s2); else each axis has its sum and its scale.
-template <int N, bool CPLX, bool ISO, int BZ, class Put>
+template <int N, bool CPLX, bool ISO, int BZ, class Ahead, class Put>
 __device__ __forceinline__ void fix_planes(const longlong2 (&col)[BZ + 2 * N], const long long* own, int nz, double s0,
-                                           double s1, double s2, Put&& put) {
+                                           double s1, double s2, Ahead&& ahead, Put&& put) {
     constexpr int RW = fix_row_width<N, CPLX>(), CPL = (FX_BY + 2 * N) * RW, SH = fix_shift(N);
     constexpr int HX = (N + 1) & ~1;
 #pragma unroll
     for (int k = 0; k < BZ; ++k) {
         if (k >= nz) break;
+        ahead(k + 1);
         const long long* b = own + k * CPL;
         const longlong2 c = col[N + k];
         long long xv[2 * HX + 2];   // real: row values -HX .. HX + 1 around the unit
@@ -319,9 +329,20 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
         const bool act0 = y < d.n2 && xe < RF, act1 = act0 && xe + 1 < RF;
         const long long i0 = (long long)y * d.n1 + (CPLX ? xe / 2 : xe);
         const int nz = min(BZ, d.n3 - z0);
+        auto fetch = [&](int k) {
+            if constexpr (HasPre<Op>::value) return op.pre((long long)(z0 + k) * d.n1 * d.n2 + i0, act0, act1);
+            else return 0;
+        };
+        auto cur = fetch(0), next = cur;
+        auto ahead = [&](int k) {
+            if (k < nz) next = fetch(k);
+        };
         auto put = [&](int k, double l0, double l1) {
             const long long i = (long long)(z0 + k) * d.n1 * d.n2 + i0;
-            if constexpr (CPLX) {
+            if constexpr (HasPre<Op>::value) {
+                op.store_pre(i, cur, l0, l1, act0, act1);
+                cur = next;
+            } else if constexpr (CPLX) {
                 if (act0) op.store(i, op.load(i), make_double2(l0, l1));
             } else {
                 if (act0) op.store(i, op.load(i), l0);
@@ -333,12 +354,13 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
 #pragma unroll
             for (int k = 0; k < BZ; ++k) col[N + k] = *reinterpret_cast<const longlong2*>(own_s + k * CPL);
             const double unit = __hiloint2double((E - 1082 + 1023) << 20, 0);
-            fix_planes<N, CPLX, ISO, BZ>(col, own_s, nz, fs.s[0] * unit, fs.s[1] * unit, fs.s[2] * unit, put);
+            fix_planes<N, CPLX, ISO, BZ>(col, own_s, nz, fs.s[0] * unit, fs.s[1] * unit, fs.s[2] * unit, ahead, put);
         } else {
             // FP64 arithmetic, straight from global memory
             constexpr int XS = CPLX ? 2 : 1;
             const int cx = HX + 2 * tx, ry = N + ty;
             for (int k = 0; k < nz; ++k) {
+                ahead(k + 1);
                 auto at = [&](int j, int r, int c) {
                     const int o = zoff[j] + yoff[r];
                     return fix_load(op, (unsigned)(o + xoff[c]), (unsigned)(o + xoff[c + 1]), false);

@@ -298,39 +298,64 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Deterministic grid-wide sum of K per-thread values: block partials are stored in
-// `partials[k * OF_MAX_RED_BLOCKS + block]`; the last block to finish adds them in block
-// order and writes out[k].  Requires blockDim.x * blockDim.y * blockDim.z <= 1024 and a
-// multiple of 32; every thread of the block must call it.
+// Sums of K per-thread values over the block, into sums[K] of shared memory (the caller's barrier
+// makes them visible).  Up to 4 sums of at most 256 threads go through shared memory, warp k adding the
+// values of sum k: an FP64 add occupies the pipe for 16 clocks per warp, and shuffles in every
+// warp took 45 of them per 256 threads and sum where this takes 13.
 template <int K>
-__device__ __forceinline__ bool grid_reduce(double (&v)[K], double* partials,
-                                            unsigned int* counter, double* out) {
-    __shared__ double sh[32][K > 0 ? K : 1];
-    __shared__ bool last;
+__device__ __forceinline__ void block_sums(const double (&v)[K], double* sums) {
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const int nthreads = blockDim.x * blockDim.y * blockDim.z;
     const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
-    const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    const int nblocks = gridDim.x * gridDim.y * gridDim.z;
+    constexpr bool FLAT = K <= 4;
+    __shared__ double sh[FLAT ? 256 : 32][K > 0 ? K : 1];
+    __syncthreads();   // readers of an earlier call's values
+    if (FLAT && nthreads <= 256) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) sh[tid][k] = v[k];
+        __syncthreads();
+        for (int k = warp; k < K; k += nwarps) {
+            double s = 0.0;
+            for (int t = lane; t < nthreads; t += 32) s += sh[t][k];
+            s = warp_sum(s);
+            if (lane == 0) sums[k] = s;
+        }
+        return;
+    }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        double s = warp_sum(v[k]);
+        const double s = warp_sum(v[k]);
         if (lane == 0) sh[warp][k] = s;
     }
     __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            double s = lane < nwarps ? sh[lane][k] : 0.0;
-            s = warp_sum(s);
-            if (lane == 0) partials[k * OF_MAX_RED_BLOCKS + bid] = s;
-        }
+    for (int k = warp; k < K; k += nwarps) {
+        double s = lane < nwarps ? sh[lane][k] : 0.0;
+        s = warp_sum(s);
+        if (lane == 0) sums[k] = s;
     }
-    __threadfence();
+}
+
+// Deterministic grid-wide sum of K per-thread values: block partials are stored in
+// `partials[k * OF_MAX_RED_BLOCKS + block]`; the last block to finish adds them in block
+// order and writes out[k].  Requires blockDim.x * blockDim.y * blockDim.z <= 1024 and a
+// multiple of 32; every thread of the block must call it.  Thread 0 of the last block, for which it
+// returns true, also gets the totals in v.
+template <int K>
+__device__ __forceinline__ bool grid_reduce(double (&v)[K], double* partials,
+                                            unsigned int* counter, double* out) {
+    __shared__ double sums[K > 0 ? K : 1];
+    __shared__ bool last;
+    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+    const int nthreads = blockDim.x * blockDim.y * blockDim.z;
+    const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+    const int nblocks = gridDim.x * gridDim.y * gridDim.z;
+    block_sums<K>(v, sums);
     __syncthreads();
-    if (tid == 0) {
-        unsigned int prev = atomicAdd(counter, 1u);
-        last = (prev == (unsigned int)nblocks - 1u);
+    if (tid < 32) {   // one warp stores the block's partials and announces them
+        for (int k = tid; k < K; k += 32) partials[k * OF_MAX_RED_BLOCKS + bid] = sums[k];
+        __threadfence();
+        __syncwarp();
+        if (tid == 0) last = atomicAdd(counter, 1u) == (unsigned int)nblocks - 1u;
     }
     __syncthreads();
     if (!last) return false;
@@ -353,24 +378,13 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[K], double* partials,
 #pragma unroll
             for (int k = 0; k < K; ++k) tot[k] += t[j][k];
     }
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const double s = warp_sum(tot[k]);
-        if (lane == 0) sh[warp][k] = s;
-    }
+    block_sums<K>(tot, sums);
     __syncthreads();
-    if (warp == 0) {
+    if (tid == 0) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            double s = lane < nwarps ? sh[lane][k] : 0.0;
-            s = warp_sum(s);
-            if (lane == 0) {
-                out[k] = s;
-                v[k] = s;   // thread 0 of the last block also gets the totals
-            }
-        }
+        for (int k = 0; k < K; ++k) out[k] = v[k] = sums[k];
+        *counter = 0u;
     }
-    if (tid == 0) *counter = 0u;
     return true;
 }
 

@@ -70,51 +70,76 @@ __global__ void __launch_bounds__(256) k_pcocg_beta(long long n, const float2* _
 }
 
 // ---------------------------------------------------------------- small vector kernels
+// Four points per thread, 256 apart, their loads in flight together, and no FP64 division per
+// thread (96^3: 9 -> 5 us each; GB300 issues 2 FP64 operations per clock and SM).
+#define OF_FOUR(i, n)                                                                                 \
+    for (long long i##0 = blockIdx.x * 1024LL + threadIdx.x; i##0 < (n); i##0 += gridDim.x * 1024LL)  \
+        _Pragma("unroll") for (int i##k = 0; i##k < 4; ++i##k)                                        \
+            if (const long long i = i##0 + 256 * i##k; i < (n))
+
 // sum of a[i] * (b ? b[i] : 1) over the grid into out[0]
-__global__ void __launch_bounds__(256) k_sum_product(long long n, const double* a, const double* b,
-                                                     RedCtx rc) {
+__global__ void __launch_bounds__(256) k_sum_product(long long n, const double* __restrict__ a,
+                                                     const double* __restrict__ b, RedCtx rc) {
     double acc[1] = {0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        acc[0] += b ? a[i] * b[i] : a[i];
+    if (b) {
+        OF_FOUR(i, n) acc[0] = fma(a[i], b[i], acc[0]);
+    } else {
+        OF_FOUR(i, n) acc[0] += a[i];
+    }
     grid_reduce<1>(acc, rc.partials, rc.counter, rc.out);
 }
 
 // y = scale * (a*b - mean), mean = *sum_dev / n ; b may be null (then a alone)
-__global__ void k_form_rhs(long long n, const double* a, const double* b, const double* sum_dev,
-                           double scale, double* y) {
-    const double mean = *sum_dev / (double)n;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        y[i] = scale * ((b ? a[i] * b[i] : a[i]) - mean);
+__global__ void __launch_bounds__(256) k_form_rhs(long long n, double inv_n, const double* __restrict__ a,
+                                                  const double* __restrict__ b, const double* sum_dev, double scale,
+                                                  double* __restrict__ y) {
+    const double mean = *sum_dev * inv_n;
+    OF_FOUR(i, n) y[i] = scale * (b ? fma(a[i], b[i], -mean) : a[i] - mean);
 }
 
-__global__ void k_sub_mean(long long n, double* x, const double* sum_dev) {
-    const double mean = *sum_dev / (double)n;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        x[i] -= mean;
+__global__ void __launch_bounds__(256) k_sub_mean(long long n, double inv_n, double* x, const double* sum_dev) {
+    const double mean = *sum_dev * inv_n;
+    OF_FOUR(i, n) x[i] -= mean;
 }
 
-// complex rhs b = P f
-__global__ void k_scale_complex(long long n, const double* f, double2 P, double2* b) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        b[i] = make_double2(P.x * f[i], P.y * f[i]);
+// The state of a solve from the reduced |b|^2: tolerance, iteration limit, counters
+__device__ __forceinline__ void start_state(KState* st, double bb, double tol, int maxit) {
+    st->tol2 = tol * tol * bb;
+    st->red[1] = bb;
+    st->zshift = 0.0;
+    st->iters = 0.0;
+    st->maxit = maxit;
+    st->done = 0.0;
+    st->breakdown = 0.0;
 }
 
-// |b|^2 into state tol2 (times tol^2) -- Hermitian norm of a real or complex field
-template <typename T>
-__global__ void __launch_bounds__(256) k_norm_to_tol(long long n, const T* b, double tol,
-                                                     KState* st, RedCtx rc) {
+// k_form_rhs and the start of the solve: y, |y|^2, the state
+__global__ void __launch_bounds__(256) k_start_poisson(long long n, double inv_n, const double* __restrict__ a,
+                                                       const double* __restrict__ b, const double* sum_dev,
+                                                       double scale, double* __restrict__ y, double tol, int maxit,
+                                                       KState* st, RedCtx rc) {
+    const double mean = *sum_dev * inv_n;
     double acc[1] = {0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        acc[0] += hn2(b[i]);
-    if (grid_reduce<1>(acc, rc.partials, rc.counter, st->red) && threadIdx.x == 0) {
-        st->tol2 = tol * tol * acc[0];
-        st->red[1] = acc[0];
+    OF_FOUR(i, n) {
+        const double v = scale * (b ? fma(a[i], b[i], -mean) : a[i] - mean);
+        y[i] = v;
+        acc[0] = fma(v, v, acc[0]);
     }
+    if (grid_reduce<1>(acc, rc.partials, rc.counter, st->red) && threadIdx.x == 0) start_state(st, acc[0], tol, maxit);
+}
+
+// The complex right-hand side b = P f of a shifted system and the start of its solve
+__global__ void __launch_bounds__(256) k_start_shifted(long long n, const double* __restrict__ f, double2 P,
+                                                       double2* __restrict__ b, double tol, int maxit, KState* st,
+                                                       RedCtx rc) {
+    double acc[1] = {0.0};
+    OF_FOUR(i, n) {
+        const double v = f[i];
+        b[i] = make_double2(P.x * v, P.y * v);
+        acc[0] = fma(v, v, acc[0]);
+    }
+    if (grid_reduce<1>(acc, rc.partials, rc.counter, st->red) && threadIdx.x == 0)
+        start_state(st, acc[0] * (P.x * P.x + P.y * P.y), tol, maxit);
 }
 
 // FP64 residual -> FP32 right-hand side; fresh inner state with rr, r^T r in FP64
@@ -201,14 +226,6 @@ __global__ void k_promote_add(long long n, T64* x, const T32* e, const KState* i
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         add_promoted(x[i], e[i], s);
-}
-
-__global__ void k_init_state(KState* st, int maxit) {
-    st->zshift = 0.0;
-    st->iters = 0.0;
-    st->maxit = maxit;
-    st->done = 0.0;
-    st->breakdown = 0.0;
 }
 
 // ---------------------------------------------------------------- host drivers
@@ -497,7 +514,8 @@ static bool direct_form(of_grid* g, double a, double2 Q, const KrylovOpts& o) {
     return std::is_same<T32, float2>::value ? shifted : a == 1.0 && !shifted;
 }
 
-// Solve A x = b (b already formed in rhs_res, FP64), A = a(-L) + Q.  x: FP64 guess/solution.
+// Solve A x = b, A = a(-L) + Q, b already formed in rhs_res and the state started (k_start_*).
+// x: FP64 guess/solution.
 template <typename T64, typename T32>
 static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const KrylovOpts& o,
                               of_solve_info* info) {
@@ -507,13 +525,11 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
     T64* b = (T64*)rb.b64;
     T64* r = (T64*)rb.r64;
     const bool direct = direct_form<T32>(g, a, Q, o);
-    launch(k_init_state, 1, 1, g->stream, st, o.max_iter);
-    launch(k_norm_to_tol<T64>, vec_blocks(n), 256, g->stream, n, b, o.tol, st, red_ctx(g, 0));
-    OF_LAUNCH_CHECK();
     residual<T64>(g, KS64, x, b, r, a, Q, direct);
-    // The direct solve's passes: each drops the residual by the FP32 rounding (1e-4 the first time,
-    // 1e-6 once the residual is rough), so this many are queued before the host looks; those
-    // after the one that converged find the done flag set and return.
+    // The direct solve's passes: each drops the residual by the FP32 rounding (1e-5 the first time,
+    // 3e-7 once the residual is rough: 1e-5, 4e-12, 5e-15 on grids from 32^3 to 320^3), so this many are
+    // queued before the host looks; those after the one that converged find the done flag set
+    // and return.
     auto direct_passes = [&](int k) {
         for (; k > 0; --k) {
             if constexpr (std::is_same<T32, float2>::value) fft_correct_shifted(g, r, x, a, Q, st);
@@ -521,7 +537,7 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
             residual<T64>(g, KS64, x, b, r, a, Q, true, false);
         }
     };
-    if (direct) direct_passes(std::min(o.max_iter, o.tol >= 1e-4 ? 1 : o.tol >= 1e-8 ? 2 : 3));
+    if (direct) direct_passes(std::min(o.max_iter, o.tol >= 2e-5 ? 1 : o.tol >= 5e-12 ? 2 : 3));
     KState h;
     fetch_scalars(g, KS64, KSTATE_DOUBLES, (double*)&h);
     const double bb = h.tol2 / (o.tol * o.tol);
@@ -672,7 +688,7 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
 static void remove_mean(of_grid* g, double* x) {
     const long long n = g->d.n;
     launch(k_sum_product, vec_blocks(n), 256, g->stream, n, x, nullptr, red_ctx(g, 120));
-    launch(k_sub_mean, vec_blocks(n), 256, g->stream, n, x, g->s.scalars + 120);
+    launch(k_sub_mean, vec_blocks(n), 256, g->stream, n, 1.0 / (double)n, x, g->s.scalars + 120);
     OF_LAUNCH_CHECK();
 }
 
@@ -680,8 +696,8 @@ static of_status poisson_impl(of_grid* g, const double* a, const double* b, doub
                               const KrylovOpts& o, of_solve_info* info) {
     const long long n = g->d.n;
     launch(k_sum_product, vec_blocks(n), 256, g->stream, n, a, b, red_ctx(g, 120));
-    launch(k_form_rhs, vec_blocks(n), 256, g->stream, n, a, b, g->s.scalars + 120, 4.0 * M_PI,
-                                                     (double*)rhs_res(g).b64);
+    launch(k_start_poisson, vec_blocks(n), 256, g->stream, n, 1.0 / (double)n, a, b, g->s.scalars + 120, 4.0 * M_PI,
+           (double*)rhs_res(g).b64, o.tol, o.max_iter, kstate(g, KS64), red_ctx(g, 0));
     OF_LAUNCH_CHECK();
     of_status st = solve_formed<double, float>(g, phi, 1.0, make_double2(0.0, 0.0), o, info);
     remove_mean(g, phi);
@@ -701,7 +717,8 @@ of_status poisson_product(of_grid* g, const double* a, const double* b, double* 
 of_status shifted(of_grid* g, const double* f, double2 P, double2 Q, double kf2, double2* W,
                   const KrylovOpts& o, of_solve_info* info) {
     const long long n = g->d.n;
-    launch(k_scale_complex, vec_blocks(n), 256, g->stream, n, f, P, (double2*)rhs_res(g).b64);
+    launch(k_start_shifted, vec_blocks(n), 256, g->stream, n, f, P, (double2*)rhs_res(g).b64, o.tol, o.max_iter,
+           kstate(g, KS64), red_ctx(g, 0));
     OF_LAUNCH_CHECK();
     return solve_formed<double2, float2>(g, W, 1.0 / kf2, Q, o, info);
 }
@@ -879,12 +896,9 @@ extern "C" of_status of_poisson_solve_noalloc(int n1, int n2, int n3, double L1,
         double* b = base + 4 * NOALLOC_VEC;
         // right-hand side 4 pi (rho - mean rho) of Eq. Poisson
         launch(k_sum_product, vec_blocks(n), 256, g.stream, n, rho, nullptr, red_ctx(&g, 120));
-        launch(k_form_rhs, vec_blocks(n), 256, g.stream, n, rho, nullptr, g.s.scalars + 120,
-               4.0 * M_PI, b);
         KState* st = kstate(&g, KS64);
-        launch(k_init_state, 1, 1, g.stream, st, o.max_iter);
-        launch(k_norm_to_tol<double>, vec_blocks(n), 256, g.stream, n, (const double*)b, o.tol, st,
-               red_ctx(&g, 0));
+        launch(k_start_poisson, vec_blocks(n), 256, g.stream, n, 1.0 / (double)n, rho, nullptr, g.s.scalars + 120,
+               4.0 * M_PI, b, o.tol, o.max_iter, st, red_ctx(&g, 0));
         residual<double>(&g, KS64, phi, b, r, 1.0, make_double2(0.0, 0.0));
         KState h;
         fetch_scalars(&g, KS64, KSTATE_DOUBLES, (double*)&h);

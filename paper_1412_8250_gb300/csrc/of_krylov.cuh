@@ -178,17 +178,45 @@ struct OpResidualDirect {
     }
     __host__ __device__ const double* field() const { return reinterpret_cast<const double*>(x); }
     __device__ T load(long long i) const { return x[i]; }
-    __device__ void store(long long i, T c, T lap) {
+    __device__ void store(long long i, T c, T lap) {   // beyond the fixed-point kernel's sizes
+        if constexpr (KT<T>::cplx) store_pre(i, Pre{b[i], c}, lap.x, lap.y, true, false);
+        else store_pre(i, Pre{make_double2(b[i], 0.0)}, lap, 0.0, true, false);
+    }
+    struct Pre {
+        double2 b;   // two real points' right-hand sides, or a complex one's
+        double2 x;   // complex: the field
+    };
+    __device__ Pre pre(long long i, bool act0, bool act1) const {
+        Pre p{};
         if constexpr (KT<T>::cplx) {
-            const double2 bi = b[i];
-            const double2 rv = make_double2(fma(a, lap.x, bi.x) - fma(Q.x, c.x, -Q.y * c.y),
-                                            fma(a, lap.y, bi.y) - fma(Q.x, c.y, Q.y * c.x));
+            if (act0) {
+                p.b = b[i];
+                p.x = x[i];
+            }
+        } else {
+            if (act0) p.b.x = b[i];
+            if (act1) p.b.y = b[i + 1];
+        }
+        return p;
+    }
+    __device__ void store_pre(long long i, const Pre& p, double l0, double l1, bool act0, bool act1) {
+        if constexpr (KT<T>::cplx) {
+            if (!act0) return;
+            const double2 c = p.x;
+            const double2 rv = make_double2(fma(a, l0, p.b.x) - fma(Q.x, c.x, -Q.y * c.y),
+                                            fma(a, l1, p.b.y) - fma(Q.x, c.y, Q.y * c.x));
             r[i] = rv;
             acc[0] = fma(rv.x, rv.x, fma(rv.y, rv.y, acc[0]));
         } else {
-            const double rv = b[i] + lap;
-            r[i] = rv;
-            acc[0] = fma(rv, rv, acc[0]);
+            const double r0 = p.b.x + l0, r1 = p.b.y + l1;
+            if (act0) {
+                r[i] = r0;
+                acc[0] = fma(r0, r0, acc[0]);
+            }
+            if (act1) {
+                r[i + 1] = r1;
+                acc[0] = fma(r1, r1, acc[0]);
+            }
         }
     }
     __device__ void end() {
@@ -729,9 +757,9 @@ inline void replay(of_grid* g, cudaGraphExec_t exec, unsigned long long kernels,
 
 
 // kernels and helpers of of_krylov.cu used by other units
-__global__ void k_form_rhs(long long n, const double* a, const double* b, const double* sum_dev,
+__global__ void k_form_rhs(long long n, double inv_n, const double* a, const double* b, const double* sum_dev,
                            double scale, double* y);
-__global__ void k_sub_mean(long long n, double* x, const double* sum_dev);
+__global__ void k_sub_mean(long long n, double inv_n, double* x, const double* sum_dev);
 KrylovOpts krylov_opts(const of_solve_opts* o);
 
 }  // namespace of

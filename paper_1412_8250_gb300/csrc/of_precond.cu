@@ -1731,7 +1731,7 @@ of_status of_precond_collect(of_grid* g, const double* rho, double shift, int st
         if (shift == 0.0) {
             launch(k_sum_product, vec_blocks(n), 256, g->stream, n, rho, (const double*)nullptr,
                    red_ctx(g, 120));
-            launch(k_form_rhs, vec_blocks(n), 256, g->stream, n, rho, (const double*)nullptr,
+            launch(k_form_rhs, vec_blocks(n), 256, g->stream, n, 1.0 / (double)n, rho, (const double*)nullptr,
                    (const double*)(g->s.scalars + 120), 4.0 * M_PI, (double*)ar.b64);
         } else {
             OF_CUDA(cudaMemcpyAsync(ar.b64, rho, sizeof(double) * n, cudaMemcpyDeviceToDevice, g->stream));
