@@ -268,6 +268,7 @@ enum Slot {
     WS_MG,       // multigrid hierarchy
     WS_NLCGP,    // preconditioned NLCG: the gradient in FP32, its V-cycle, the FP64 direction
     WS_FGM,      // flexible GMRES: Arnoldi and preconditioned vectors
+    WS_AXIS,     // the ions' axis tables and the quadrature of their self terms
     WS_IMG,      // periodic images of the ions and their lists per z-slab (nuclear charge)
     WS_FFT,      // half spectrum of a direct solve
     WS_FFTT,     // its twiddles and symbol tables
