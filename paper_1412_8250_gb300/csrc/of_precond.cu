@@ -119,46 +119,68 @@ __device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) {
 // ---------------------------------------------------------------- forward
 // ---------------------------------------------------------------- forward on the tensor cores
 // Layer 2 is the network's dense contraction: per point z2[o] = b2[o] + sum_t sum_c
-// W2[o][c][t] a1[x+t][c], 432 multiply-adds per output channel.  Over a tile of up to 128
-// consecutive points of one x-row it is the implicit GEMM D[128 x 16] = sum_t A_t B_t^T,
-// A_t[m][c] = a1[x_m + t][c], B_t[o][c] = W2[o][c][t]: 27 tcgen05.mma of shape M=128, N=16,
-// K=16 (BF16 operands, FP32 accumulators in tensor memory), issued by one thread.  The three
-// taps dx = -1, 0, 1 of one (dz, dy) plane read the same staged rows shifted by one row, so a
-// tile stages nine plane rows of length L + 2 (x0 - 1 .. x0 + L, wrapped) and each MMA's A
-// descriptor starts dx + 1 rows into its plane.  Each plane accumulates into its own 16
-// columns (nine short chains instead of one of 27).  Layer 3 (one output channel) is the same
-// contraction with B_t row 0 = W3[.][t] and rows 1-15 zero.  The epilogue reads the
-// accumulators with tcgen05.ld and sums them: layer 2 adds b2, applies GELU and stores BF16
-// (z2 too when training); layer 3 takes column 0, adds b3 and scales.  Layer 1 (one input
-// channel) is one GEMM with the 27 taps as K, padded to 32.
-// Shared-memory operands are K-major without swizzle: core matrices of 8 rows x 16 bytes
-// (8 BF16 channels), rows 16 bytes apart throughout (stride byte offset 128 per 8-row group),
-// channels 8-15 one plane-half further (leading byte offset = ROWS * 16).
+// W2[o][c][t] a1[x+t][c], 432 multiply-adds per output channel, run as an implicit GEMM on
+// tcgen05.mma (BF16 operands, FP32 accumulators in tensor memory).
+// A tile is 16 groups of 8 consecutive points of an x-row (128 rows of the MMA); the groups of
+// all x-rows of one y are numbered through z, so tiles stay full whatever n1 is.  A CTA walks
+// its tile along y.  Each row it meets is an event: for the three z neighbours of every group the
+// 8 points and one to either side are staged once (16-byte cells: 8 BF16 channels, two halves),
+// and nine MMAs multiply them by the taps: per dz an accumulator whose columns hold the three
+// dy blocks (layer 2: N = 48), over dx a chain of three MMAs that read the staged cells
+// shifted by one.  A row's accumulators thus serve the outputs at y + 1, y and y - 1, and an
+// output sums nine column blocks of its three last events, in the order of the planes
+// (dz, dy).  Against nine staged rows and 27 MMAs of N = 16 per output (each reads the whole A
+// operand, 4 KB, from shared memory whatever N is) this is a third of the traffic from L2 and
+// of the operand reads.
+// The first warps copy (or, in layer 1, build) the operands, the next one issues the MMAs, the
+// others read the accumulators and finish: bias and GELU, or GELU' in the backward pass, or layer 3's scale.
+// They meet at mbarriers only, so that copies, MMAs and epilogues of successive rows overlap.
+// Layer 3 (one output channel) has the same form with three of 16 columns used per dz; layer 1
+// (one input channel) is one GEMM per row with the 27 taps as K, padded to 32.
+// Time of one application on 192^3, against one tile per barrier round with every thread in
+// every part: see the layers' kernels.
+// Shared-memory operands are K-major without swizzle: core matrices of 8 rows x 16 bytes,
+// one per group of points (10 cells apart in layers 2 and 3).
 namespace tc {
-constexpr int M = 128;                   // rows per MMA (points per tile, padded)
-constexpr int THREADS = 256;             // two threads per row: channel halves
-constexpr int ROWS = M + 2;              // staged rows per plane: x0 - 1 .. x0 + 128
-constexpr int HALF = ROWS * 16;          // bytes of one channel half of a plane (2080)
-constexpr int PLANE = 2 * HALF;          // 4160
-constexpr int A_BYTES = 9 * PLANE;       // 37440
-constexpr int B_TAP = NC * NC * 2;       // 512 bytes per tap: 16 x 16 BF16
-constexpr int B_BYTES = NT * B_TAP;      // 13824
-constexpr int SMEM = 128 + 2 * A_BYTES + B_BYTES + 64;   // layers 2 and 3: two A buffers
-constexpr int SMEM1 = 128 + A_BYTES + 2 * B_TAP + 64;      // layer 1
-constexpr int ACC_COLS = 256;   // layers 2 and 3: nine 16-column accumulators (144 used); two
-                                // CTAs per SM fill the 512 columns of tensor memory
-// layer 1: A tile 128 rows x 32 taps, four K-blocks of 8 taps (2048 bytes each), then the
-// staged FP32 planes of r
-constexpr int L1_KB = M * 16;
+constexpr int M = 128;                   // rows per MMA (points per tile)
+constexpr int GROUPS = M / 8;
+constexpr int CELLS = 10;                // staged cells per group: its 8 points and their neighbours
+constexpr int HALF = GROUPS * CELLS * 16;   // bytes of one channel half of one z plane (2560)
+constexpr int PLANE = 2 * HALF;
+constexpr int STAGE = 3 * PLANE;            // one event's operand: 15360 bytes
+constexpr int STAGE_CELLS = STAGE / 16;
+constexpr int B_TAP = NC * NC * 2;       // one 16 x 16 BF16 weight tile
+constexpr int L1_KB = M * 16;            // layer 1: 128 rows x 8 taps
 constexpr int L1_STAGE = 4 * L1_KB;
-static_assert(L1_STAGE + 9 * ROWS * 4 <= A_BYTES, "layer-1 staging must fit the A buffer");
-constexpr uint32_t A_LBO = HALF, A_SBO = 128;    // B tiles: (o/8, c/8) at (o/8)*256 + (c/8)*128
-constexpr uint32_t B_LBO = 128, B_SBO = 256;
+constexpr uint32_t A_LBO = HALF, A_SBO = CELLS * 16;
+constexpr uint32_t B_LBO = 128, B_SBO = 256;    // B tiles: (o/8, c/8) at (o/8)*256 + (c/8)*128
 // instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9, 10-12 = 1),
 // both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NC >> 3) << 17) |
-                           ((uint32_t)(M >> 4) << 24);
+constexpr uint32_t idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
 constexpr unsigned long long WAIT_NS = 2000000000ull;   // give up on a completion after 2 s
+
+// Per layer: threads that stage (layer 1: one per row; with the issuing warp 20 warps in layer 2,
+// so that 96 registers are left per thread), columns of one dz accumulator, events whose accumulators are held, staged events,
+// how many of those are copies in flight, warps of an epilogue group, groups (which take
+// alternate events), CTAs per SM.  Layer 2's three events are the least its outputs need and
+// 432 of the 512 columns.
+template <int LAYER> struct Cfg;
+template <> struct Cfg<1> {
+    static constexpr int COPY = 128, N = 16, DZ = 1, SLOTS = 4, STAGES = 4, EPI = 8, SETS = 1, CTAS = 2, COLS = 64, USES = 1;
+    static constexpr int BYTES = L1_STAGE, B_BYTES = 2 * B_TAP;
+};
+template <> struct Cfg<2> {
+    static constexpr int COPY = 96, N = 48, DZ = 3, SLOTS = 3, STAGES = 8, FLIGHT = 6, EPI = 8, SETS = 2, CTAS = 1, COLS = 512, USES = 3;
+    static constexpr int BYTES = STAGE, B_BYTES = 27 * B_TAP;
+};
+template <> struct Cfg<3> {
+    static constexpr int COPY = 96, N = 16, DZ = 3, SLOTS = 5, STAGES = 6, FLIGHT = 4, EPI = 4, SETS = 1, CTAS = 2, COLS = 256, USES = 3;
+    static constexpr int BYTES = STAGE, B_BYTES = 9 * B_TAP;
+};
+template <int LAYER> constexpr int threads() { return Cfg<LAYER>::COPY + 32 + 32 * Cfg<LAYER>::EPI * Cfg<LAYER>::SETS; }
+template <int LAYER> constexpr int smem() { return 128 + Cfg<LAYER>::STAGES * Cfg<LAYER>::BYTES + Cfg<LAYER>::B_BYTES; }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -174,41 +196,41 @@ __device__ __forceinline__ unsigned long long now_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
 // bounded wait for the phase of parity `parity` of an mbarrier: false once limit_ns have passed
-// (at once for limit_ns = 0, without polling)
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns) {
+// (at once for limit_ns = 0, without polling) or when another warp gave up (*quit)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns,
+                                          const volatile int* quit) {
     if (limit_ns == 0) return false;
+    if (mbar_test(bar, parity)) return true;
     const unsigned long long t0 = now_ns();
     for (int k = 0; k < (1 << 22); ++k) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done) return true;
+        if (mbar_test(bar, parity)) return true;
+        if (quit && *quit) return false;
         if ((k & 63) == 63 && now_ns() - t0 > limit_ns) return false;
     }
     return false;
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
+}
+template <int N>
 __device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(tmem), "l"(a), "l"(b), "r"(IDESC), "r"(accumulate) : "memory");
+        :: "r"(tmem), "l"(a), "l"(b), "r"(idesc(N)), "r"(accumulate) : "memory");
 }
-__device__ __forceinline__ void ld8(uint32_t taddr, float (&v)[8]) {
-    uint32_t r[8];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-        : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = __uint_as_float(r[k]);
-}
-// loads without the wait: issue several, then one wait_ld()
+// tensor-memory loads: issue several, then one wait_ld()
 __device__ __forceinline__ void ld8_nowait(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -244,22 +266,24 @@ __device__ __forceinline__ float getp(const __nv_bfloat16* p, long long n, long 
     return __bfloat162float(p[((long long)(c >> 3) * n + i) * 8 + (c & 7)]);
 }
 
-// B tiles (N = 16 output channels o x K = 16), K-major, (o/8, c/8) core matrices at
-// (o/8) * 256 + (c/8) * 128: per tap t for layers 2 and 3, per half h of the 32 padded taps
-// for layer 1
+// B tiles (16 rows x K = 16), K-major, (row/8, c/8) core matrices at (row/8) * 256 + (c/8) * 128.
+// Layer 1: rows are output channels, one tile per half of the 32 padded taps.  Layer 2: per (dz,
+// dx) three tiles, dy = -1, 0, 1, rows output channels.  Layer 3: per (dz, dx) one tile, row dy + 1.
 template <int LAYER>
 __device__ __forceinline__ void fill_b(unsigned char* Bs, const __nv_bfloat16* __restrict__ P, float* bias) {
-    const int ntiles_b = LAYER == 1 ? 2 : NT;
-    for (int k = threadIdx.x; k < ntiles_b * NC * NC; k += blockDim.x) {
+    constexpr int tiles = tc::Cfg<LAYER>::B_BYTES / tc::B_TAP;
+    for (int k = threadIdx.x; k < tiles * NC * NC; k += blockDim.x) {
         const int t = k / (NC * NC), o = (k / NC) % NC, c = k % NC;
-        __nv_bfloat16 w;
+        __nv_bfloat16 w = __float2bfloat16(0.f);
         if (LAYER == 1) {
             const int tap = 16 * t + c;
-            w = tap < NT ? P[OW1 + o * NT + tap] : __float2bfloat16(0.f);
+            if (tap < NT) w = P[OW1 + o * NT + tap];
         } else if (LAYER == 2) {
-            w = P[OW2 + (o * NC + c) * NT + t];
-        } else {
-            w = o == 0 ? P[OW3 + c * NT + t] : __float2bfloat16(0.f);
+            const int dz = t / 9, dx = (t / 3) % 3, dy = t % 3;
+            w = P[OW2 + (o * NC + c) * NT + 9 * dz + 3 * dy + dx];
+        } else if (o < 3) {
+            const int dz = t / 3, dx = t % 3;
+            w = P[OW3 + c * NT + 9 * dz + 3 * o + dx];
         }
         *(__nv_bfloat16*)(Bs + t * tc::B_TAP + (o >> 3) * 256 + (c >> 3) * 128 + (o & 7) * 16 + (c & 7) * 2) = w;
     }
@@ -270,20 +294,50 @@ __device__ __forceinline__ void fill_b(unsigned char* Bs, const __nv_bfloat16* _
                                : (tid == 0 ? __bfloat162float(P[OB3]) : 0.f);
 }
 
-// first point of the x-row of each plane q = 3 (dz + 1) + (dy + 1) around row (y, z)
-__device__ __forceinline__ void plane_bases(const Dims& d, int y, int z, long long (&qb)[9]) {
-    const long long plane = (long long)d.n1 * d.n2;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const int zz = z + q / 3 - 1, yy = y + q % 3 - 1;
-        const int zw = zz < 0 ? zz + d.n3 : (zz >= d.n3 ? zz - d.n3 : zz);
-        const int yw = yy < 0 ? yy + d.n2 : (yy >= d.n2 ? yy - d.n2 : yy);
-        qb[q] = (long long)zw * plane + (long long)yw * d.n1;
+// A block's share of the output rows (tile, y), cut evenly: runs of consecutive y of one tile.
+struct Runs {
+    long long r, end;
+    int n2;
+    long long tile;   // of the run that next() found: rows y0 .. y0 + rows - 1
+    int y0, rows;
+    __device__ __forceinline__ Runs(const Dims& d, long long tiles) : n2(d.n2) {
+        const long long all = tiles * d.n2;
+        r = all * blockIdx.x / gridDim.x;
+        end = all * (blockIdx.x + 1) / gridDim.x;
     }
+    __device__ __forceinline__ bool next() {
+        if (r >= end) return false;
+        tile = r / n2;
+        y0 = (int)(r - tile * n2);
+        rows = (int)min((long long)(n2 - y0), end - r);
+        r += rows;
+        return true;
+    }
+};
+__device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
+// x-row z and first point x of group `g` of a tile; the tiles' last groups past the end repeat
+// the last group (false)
+__device__ __forceinline__ bool group_of(const Dims& d, long long tile, int g, int& z, int& x) {
+    const int gx = (d.n1 + 7) >> 3;
+    const long long all = (long long)d.n3 * gx;
+    long long f = tile * tc::GROUPS + g;
+    const bool in = f < all;
+    if (!in) f = all - 1;
+    z = (int)(f / gx);
+    x = 8 * (int)(f - (long long)z * gx);
+    return in;
+}
+// the point (index without its y) of MMA row m; false for rows past the end of the x-row
+__device__ __forceinline__ bool point_of(const Dims& d, long long tile, int m, long long& i) {
+    int z, x;
+    const bool in = group_of(d, tile, m >> 3, z, x);
+    x += m & 7;
+    i = (long long)z * d.n1 * d.n2 + x;
+    return in && x < d.n1;
 }
 
-__device__ __forceinline__ void mbar_init(uint32_t bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar) : "memory");
+__device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count) : "memory");
 }
 // tensor-memory columns (a power of two >= 32), allocated and freed by one whole warp
 template <int COLS>
@@ -301,32 +355,6 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
                  :: "r"(bar) : "memory");
 }
 
-// Copies the nine plane rows of a tile (staged row j = point x0 - 1 + j of its x-row, wrapped;
-// both channel halves) into an A buffer with 16-byte asynchronous copies, all threads: thread
-// tid takes half h = tid / 128 of staged row j = tid % 128 (and of row 128 + j for j < 2) of
-// every plane.  With the planar activation layout consecutive threads copy consecutive 16
-// bytes, so every 32-byte sector read is used whole.  Commits one copy group.
-__device__ __forceinline__ void stage_planes(uint32_t abuf, const __nv_bfloat16* in, long long n,
-                                             const long long (&qb)[9], int x0, int L, int n1) {
-    const int h = threadIdx.x >> 7;
-#pragma unroll
-    for (int rep = 0; rep < 2; ++rep) {
-        const int j = (threadIdx.x & (tc::M - 1)) + rep * tc::M;
-        if (j < L + 2) {
-            int x = x0 - 1 + j;
-            x = x < 0 ? x + n1 : (x >= n1 ? x - n1 : x);
-            const __nv_bfloat16* src = in + ((long long)h * n + x) * 8;
-            const uint32_t dst = abuf + h * tc::HALF + j * 16;
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
-                             :: "r"(dst + q * tc::PLANE), "l"(src + qb[q] * 8) : "memory");
-        }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-// Layer 1: z1 = W1 * (sgn r / s) + b1, a1 = GELU(z1), as the GEMM D[128 x 16] = A B^T with
 // Data-gradient epilogue (the backward pass runs the forward kernels with the mirrored,
 // transposed weights of of_precond's backward array): the convolution's 8 channels ch*8 ..
 // of point i times GELU' of the forward pre-activation zin, to gout (FP32, [x][16], for the
@@ -351,267 +379,384 @@ __device__ __forceinline__ void epilogue_bwd(const float (&acc)[8], const __nv_b
     if (aout) store8(aout + ((long long)ch * n + i) * 8, g);
 }
 
-// A[m][k] = (sgn r / s)(x_m + t_k) (taps k < 27, zero up to 32) and B[o][k] = W1[o][t_k]: two
-// MMAs of K = 16.  The nine plane rows of r are staged in FP32 (plain loads), each thread
-// builds half of its A row in BF16.  rnout: the input as rounded to BF16 (training).  One CTA
-// of 256 threads per tile; thread tid owns row m = tid % 128 and channels 8 (tid / 128) .. + 7.
-template <bool BWD>
-__global__ void __launch_bounds__(tc::THREADS, 4) k_conv1_tc(Dims d, int nseg, int lseg,
-                                                             const float* __restrict__ rin,
-                                                             const __nv_bfloat16* __restrict__ P,
-                                                             __nv_bfloat16* zout, __nv_bfloat16* aout,
-                                                             float* rnout, const double* s_dev, float sgn,
-                                                             double* err, unsigned long long wait_ns,
-                                                             const __nv_bfloat16* __restrict__ zin,
-                                                             float* gout) {
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    unsigned char* As = sm;
-    unsigned char* Bs = sm + tc::A_BYTES;
-    uint64_t* bar = (uint64_t*)(Bs + 2 * tc::B_TAP);
-    uint32_t* tslot = (uint32_t*)(bar + 1);
-    __shared__ float bias[NC];
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int m = tid & (tc::M - 1), ch = tid >> 7;
-    for (int k = tid; k < tc::A_BYTES / 16; k += tc::THREADS)
-        reinterpret_cast<uint4*>(As)[k] = make_uint4(0, 0, 0, 0);
-    fill_b<1>(Bs, P, bias);
-    const uint32_t bar_a = tc::smem_addr(bar);
-    if (tid == 0) {
-        mbar_init(bar_a);
+// What the kernels of the three layers share: operand ring, barriers, tensor memory.  FULL: an
+// event's operand is staged; EMPTY: its MMAs have read it; ACC: its accumulators are complete;
+// FREE: every output that needs them has loaded them.
+template <int LAYER>
+struct ConvShared {
+    using C = tc::Cfg<LAYER>;
+    uint64_t full[C::STAGES], empty[C::STAGES], acc[C::SLOTS], free[C::SLOTS], last;
+    uint32_t tmem;
+    int quit;
+    alignas(16) float bias[NC];
+};
+template <int LAYER>
+__device__ __forceinline__ uint32_t conv_begin(ConvShared<LAYER>& s, unsigned char* Bs,
+                                               const __nv_bfloat16* __restrict__ P) {
+    using C = tc::Cfg<LAYER>;
+    fill_b<LAYER>(Bs, P, s.bias);
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < C::STAGES; ++k) {
+            mbar_init(tc::smem_addr(&s.full[k]), C::COPY);
+            mbar_init(tc::smem_addr(&s.empty[k]), 1);
+        }
+        for (int k = 0; k < C::SLOTS; ++k) {
+            mbar_init(tc::smem_addr(&s.acc[k]), 1);
+            mbar_init(tc::smem_addr(&s.free[k]), C::USES * C::EPI);
+        }
+        mbar_init(tc::smem_addr(&s.last), 1);
+        s.quit = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tmem_alloc<32>(tslot);
+    if (threadIdx.x < 32) tmem_alloc<C::COLS>(&s.tmem);
     tc::fence_async_smem();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    const uint32_t tmem = *tslot;
-    const uint32_t a_base = tc::smem_addr(As), b_base = tc::smem_addr(Bs);
-    // the input scaled by sgn / RMS (forward), or as it is (data gradient)
-    const double rms = BWD ? 1.0 : *s_dev;
-    const float inv = rms > 0.0 ? sgn * (float)(1.0 / rms) : 0.f;   // 0 for a zero residual
-    const long long ntiles = (long long)d.n2 * d.n3 * nseg;
-    float* rs = reinterpret_cast<float*>(As + tc::L1_STAGE);
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int tile = (int)blockIdx.x; ok && tile < ntiles; tile += (int)gridDim.x) {
-        const int rowi = tile / nseg;
-        const int x0 = (tile - rowi * nseg) * lseg;
-        const int L = min(lseg, d.n1 - x0);
-        const int z = rowi / d.n2;
-        long long qb[9];
-        plane_bases(d, rowi - z * d.n2, z, qb);
-        if (tid < L + 2) {   // staged row j = tid, point x0 - 1 + j (wrapped)
-            int x = x0 - 1 + tid;
-            x = x < 0 ? x + d.n1 : (x >= d.n1 ? x - d.n1 : x);
-            float v[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) v[q] = __ldg(rin + qb[q] + x);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) rs[q * tc::ROWS + tid] = v[q] * inv;
-        }
-        __syncthreads();
-        __nv_bfloat16 row[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            const int t = 16 * ch + u;
-            row[u] = __float2bfloat16(t < NT ? rs[(t / 3) * tc::ROWS + m + t % 3] : 0.f);
-        }
-#pragma unroll
-        for (int kb = 0; kb < 2; ++kb)
-            *(uint4*)(As + (2 * ch + kb) * tc::L1_KB + m * 16) = *reinterpret_cast<const uint4*>(row + 8 * kb);
-        if (rnout && ch == 0 && m < L)   // tap 13 is the point itself
-            rnout[(long long)rowi * d.n1 + x0 + m] = __bfloat162float(row[13]);
-        tc::fence_async_smem();
-        tc::fence_before();
-        __syncthreads();
-        if (tid == 0) {
-            tc::fence_after();
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                tc::mma(tmem, tc::desc(a_base + 2 * h * tc::L1_KB, tc::L1_KB, tc::A_SBO),
-                        tc::desc(b_base + h * tc::B_TAP, tc::B_LBO, tc::B_SBO), h > 0 ? 1u : 0u);
-            mma_commit(bar_a);
-        }
-        const bool seen = tc::mbar_wait(bar_a, phase, wait_ns);
-        phase ^= 1u;
-        ok = __syncthreads_and(seen) != 0;
-        tc::fence_after();
-        if (!ok) break;
-        float acc[8];
-        tc::ld8(tmem + ((uint32_t)((warp & 3) * 32) << 16) + 8 * ch, acc);
-        if (m < L) {
-            const long long i = (long long)rowi * d.n1 + x0 + m;
-            if (BWD)
-                epilogue_bwd(acc, zin, gout, aout, d.n, i, ch);
-            else {
-                float zv[8], g[8];
-#pragma unroll
-                for (int o = 0; o < 8; ++o) {
-                    zv[o] = acc[o] + bias[8 * ch + o];
-                    g[o] = gelu_f(zv[o]);
-                }
-                if (zout) store8(zout + ((long long)ch * d.n + i) * 8, zv);
-                store8(aout + ((long long)ch * d.n + i) * 8, g);
-            }
-        }
-        tc::fence_before();
+    return s.tmem;
+}
+// Every role ends here, whether it ran to its end or gave up: no copy and no MMA outlives the
+// CTA or the tensor memory it writes (bounded by the full limit, whatever wait_ns was).
+template <int LAYER>
+__device__ __forceinline__ void conv_end(ConvShared<LAYER>& s, uint32_t tmem) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (threadIdx.x == tc::Cfg<LAYER>::COPY) {
+        mma_commit(tc::smem_addr(&s.last));
+        tc::mbar_wait(tc::smem_addr(&s.last), 0, tc::WAIT_NS, nullptr);
     }
-    if (!ok) {
-        if (tid == 0) *err = 1.0;
-        // let the MMAs still in flight finish (bounded by the full limit, whatever wait_ns was)
-        // before the tensor memory they write is freed
-        tc::mbar_wait(bar_a, phase ^ 1u, tc::WAIT_NS);
-    }
+    __syncwarp();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    if (warp == 0) tmem_free<32>(tmem);
+    if (threadIdx.x < 32) tmem_free<tc::Cfg<LAYER>::COLS>(tmem);
+}
+template <int LAYER>
+__device__ __forceinline__ void conv_quit(ConvShared<LAYER>& s, double* err) {
+    *(volatile int*)&s.quit = 1;
+    *err = 1.0;
+}
+// parity of the phase in which event e of a ring of R ends
+template <int R>
+__device__ __forceinline__ uint32_t ring_parity(int e) { return (uint32_t)(e / R) & 1u; }
+
+// The issuing thread's part of event e: waits for its operand and for free columns; issue()
+// places the MMAs.
+template <int LAYER, typename F>
+__device__ __forceinline__ bool conv_issue(ConvShared<LAYER>& s, int e, F issue) {
+    using C = tc::Cfg<LAYER>;
+    const int st = e % C::STAGES, sl = e % C::SLOTS;
+    if (!tc::mbar_wait(tc::smem_addr(&s.full[st]), ring_parity<C::STAGES>(e), tc::WAIT_NS, &s.quit)) return false;
+    if (e >= C::SLOTS &&
+        !tc::mbar_wait(tc::smem_addr(&s.free[sl]), ring_parity<C::SLOTS>(e) ^ 1u, tc::WAIT_NS, &s.quit))
+        return false;
+    tc::fence_after();
+    issue(st, sl);
+    mma_commit(tc::smem_addr(&s.empty[st]));
+    mma_commit(tc::smem_addr(&s.acc[sl]));
+    return true;
+}
+// one warp's wait for the accumulators of event e, all lanes alike
+template <int LAYER>
+__device__ __forceinline__ bool conv_acc(ConvShared<LAYER>& s, int e, unsigned long long wait_ns) {
+    using C = tc::Cfg<LAYER>;
+    const bool ok = tc::mbar_wait(tc::smem_addr(&s.acc[e % C::SLOTS]), ring_parity<C::SLOTS>(e), wait_ns, &s.quit);
+    const bool all = __all_sync(0xffffffffu, ok);
+    tc::fence_after();
+    return all;
+}
+// ... and its word that it has loaded what it needs of event e
+template <int LAYER>
+__device__ __forceinline__ void conv_free(ConvShared<LAYER>& s, int e) {
+    if (e < 0) return;
+    tc::fence_before();
+    if ((threadIdx.x & 31) == 0) tc::mbar_arrive(tc::smem_addr(&s.free[e % tc::Cfg<LAYER>::SLOTS]));
+}
+
+// bias, GELU and the stores of 8 channels of point i
+__device__ __forceinline__ void epilogue_fwd(const float (&acc)[8], const float* bias, __nv_bfloat16* zout,
+                                             __nv_bfloat16* aout, long long n, long long i, int ch) {
+    float zv[8], g[8];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+        zv[o] = acc[o] + bias[8 * ch + o];
+        g[o] = gelu_f(zv[o]);
+    }
+    if (zout) store8(zout + ((long long)ch * n + i) * 8, zv);
+    store8(aout + ((long long)ch * n + i) * 8, g);
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// Layer 1: z1 = W1 * (sgn r / s) + b1, a1 = GELU(z1), as the GEMM D[128 x 16] = A B^T with
+// A[m][k] = (sgn r / s)(x_m + t_k) (taps k < 27, zero up to 32) and B[o][k] = W1[o][t_k]: two
+// MMAs of K = 16.  A staging thread owns one point and walks along y with it: it keeps the
+// 3 x 3 x 3 values around it in BF16, reads the nine of the next row while it lays out the
+// present ones, and writes its row of A with four 16-byte stores.  rnout: the input as rounded
+// to BF16 (training).
+template <bool BWD>
+__global__ void __launch_bounds__(tc::threads<1>(), tc::Cfg<1>::CTAS)
+    k_conv1_tc(Dims d, long long tiles, const float* __restrict__ rin, const __nv_bfloat16* __restrict__ P,
+               __nv_bfloat16* zout, __nv_bfloat16* aout, float* rnout, const double* s_dev, float sgn,
+               double* err, unsigned long long wait_ns, const __nv_bfloat16* __restrict__ zin, float* gout) {
+    using C = tc::Cfg<1>;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* As = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    unsigned char* Bs = As + C::STAGES * C::BYTES;
+    __shared__ ConvShared<1> s;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const uint32_t tmem = conv_begin<1>(s, Bs, P);
+    Runs run(d, tiles);
+    int e = 0;
+    bool ok = true;
+    if (warp < 4) {
+        // the input scaled by sgn / RMS (forward), or as it is (data gradient)
+        const double rms = BWD ? 1.0 : *s_dev;
+        const float inv = rms > 0.0 ? sgn * (float)(1.0 / rms) : 0.f;   // 0 for a zero residual
+        while (ok && run.next()) {
+            int z, x;
+            const bool in = group_of(d, run.tile, tid >> 3, z, x) && x + (tid & 7) < d.n1;
+            x = min(x + (tid & 7), d.n1 - 1);
+            const long long plane = (long long)d.n1 * d.n2;
+            const float* src[3] = {rin + wrap1(z - 1, d.n3) * plane, rin + z * plane, rin + wrap1(z + 1, d.n3) * plane};
+            const int xn[3] = {wrap1(x - 1, d.n1), x, wrap1(x + 1, d.n1)};
+            float v[3][3];
+            uint32_t lo[3][3], hi[3][3];   // [dz][dy]: taps dx = -1, 0 and dx = 1
+            auto fetch = [&](int y) {
+                const long long row = (long long)wrap1(y, d.n2) * d.n1;
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) v[a][c] = __ldg(src[a] + row + xn[c]);
+            };
+            auto turn = [&]() {   // the fetched row becomes dy = +1
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    lo[a][0] = lo[a][1];
+                    hi[a][0] = hi[a][1];
+                    lo[a][1] = lo[a][2];
+                    hi[a][1] = hi[a][2];
+                    lo[a][2] = pack_bf16(v[a][0] * inv, v[a][1] * inv);
+                    hi[a][2] = pack_bf16(v[a][2] * inv, 0.f);
+                }
+            };
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) lo[a][b] = hi[a][b] = 0u;
+            fetch(run.y0 - 1);
+            turn();
+            fetch(run.y0);
+            turn();
+            fetch(run.y0 + 1);
+            for (int k = 0; k < run.rows; ++k, ++e) {
+                turn();
+                if (k + 1 < run.rows) fetch(run.y0 + k + 2);
+                uint32_t w[16];
+#pragma unroll
+                for (int q = 0; q < 9; q += 2) {
+                    const uint32_t l0 = lo[q / 3][q % 3], h0 = hi[q / 3][q % 3];
+                    const uint32_t l1 = q < 8 ? lo[(q + 1) / 3 % 3][(q + 1) % 3] : 0u;
+                    const uint32_t h1 = q < 8 ? hi[(q + 1) / 3 % 3][(q + 1) % 3] : 0u;
+                    w[3 * q / 2] = l0;
+                    w[3 * q / 2 + 1] = h0 | (l1 << 16);
+                    w[3 * q / 2 + 2] = (l1 >> 16) | (h1 << 16);
+                }
+                w[15] = 0u;
+                if (rnout && in) {
+                    const long long i = (long long)z * plane + (long long)(run.y0 + k) * d.n1 + x;
+                    rnout[i] = __uint_as_float(lo[1][1] & 0xffff0000u);   // tap 13, the point itself
+                }
+                const int st = e % C::STAGES;
+                ok = e < C::STAGES || tc::mbar_wait(tc::smem_addr(&s.empty[st]), ring_parity<C::STAGES>(e) ^ 1u,
+                                                    tc::WAIT_NS, &s.quit);
+                if (!ok) break;
+                unsigned char* row = As + st * C::BYTES + tid * 16;
+#pragma unroll
+                for (int kb = 0; kb < 4; ++kb)
+                    *(uint4*)(row + kb * tc::L1_KB) = make_uint4(w[4 * kb], w[4 * kb + 1], w[4 * kb + 2], w[4 * kb + 3]);
+                tc::fence_async_smem();
+                tc::mbar_arrive(tc::smem_addr(&s.full[st]));
+            }
+        }
+    } else if (warp == 4) {
+        if (tid == C::COPY) {
+            const uint32_t a_base = tc::smem_addr(As), b_base = tc::smem_addr(Bs);
+            while (ok && run.next())
+                for (int k = 0; ok && k < run.rows; ++k, ++e)
+                    ok = conv_issue<1>(s, e, [&](int st, int sl) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            tc::mma<C::N>(tmem + C::N * sl,
+                                          tc::desc(a_base + st * C::BYTES + 2 * h * tc::L1_KB, tc::L1_KB, 128),
+                                          tc::desc(b_base + h * tc::B_TAP, tc::B_LBO, tc::B_SBO), h > 0 ? 1u : 0u);
+                    });
+        }
+    } else {
+        const int m = (warp & 3) * 32 + (tid & 31), ch = (warp - 5) >> 2;
+        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 8 * ch;
+        while (ok && run.next()) {
+            long long i;
+            const bool in = point_of(d, run.tile, m, i);
+            i += (long long)run.y0 * d.n1;
+            for (int k = 0; k < run.rows; ++k, ++e, i += d.n1) {
+                ok = conv_acc<1>(s, e, wait_ns);
+                if (!ok) break;
+                uint32_t part[8];
+                tc::ld8_nowait(taddr + C::N * (e % C::SLOTS), part);
+                tc::wait_ld();
+                conv_free<1>(s, e);
+                float acc[8];
+#pragma unroll
+                for (int o = 0; o < 8; ++o) acc[o] = __uint_as_float(part[o]);
+                if (in) {
+                    if (BWD) epilogue_bwd(acc, zin, gout, aout, d.n, i, ch);
+                    else epilogue_fwd(acc, s.bias, zout, aout, d.n, i, ch);
+                }
+            }
+        }
+    }
+    if (!ok) conv_quit<1>(s, err);
+    conv_end<1>(s, tmem);
 }
 
 // Layers 2 and 3 (see above).  LAYER 2: in = a1 -> z2 (optional), a2.  LAYER 3: in = a2 ->
-// y = scale (W3 * a2 + b3), scale = *s_dev (1 with s_dev null).  The next tile's plane rows are
-// copied into the other A buffer while the current tile's MMAs and epilogue run; one CTA of 256
-// threads per tile, persistent; err as for layer 1.
+// y = scale (W3 * a2 + b3), scale = *s_dev (1 with s_dev null).  err as for layer 1: set when a
+// completion was not seen within wait_ns.
 template <int LAYER, bool BWD>
-__global__ void __launch_bounds__(tc::THREADS, 2) k_conv_tc(Dims d, int nseg, int lseg,
-                                                            const __nv_bfloat16* __restrict__ in,
-                                                            const __nv_bfloat16* __restrict__ P,
-                                                            __nv_bfloat16* zout, __nv_bfloat16* aout,
-                                                            float* yout, const double* s_dev, double* err,
-                                                            unsigned long long wait_ns,
-                                                            const __nv_bfloat16* __restrict__ zin,
-                                                            float* gout) {
+__global__ void __launch_bounds__(tc::threads<LAYER>(), tc::Cfg<LAYER>::CTAS)
+    k_conv_tc(Dims d, long long tiles, const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ P,
+              __nv_bfloat16* zout, __nv_bfloat16* aout, float* yout, const double* s_dev, double* err,
+              unsigned long long wait_ns, const __nv_bfloat16* __restrict__ zin, float* gout) {
+    using C = tc::Cfg<LAYER>;
+    constexpr int EV = C::DZ * C::N;   // columns of one event
+    static_assert(EV * C::SLOTS <= C::COLS && C::SLOTS >= 3 && C::FLIGHT < C::STAGES, "rings");
     extern __shared__ unsigned char smem_raw[];
-    unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    unsigned char* As = sm;                              // two A buffers
-    unsigned char* Bs = sm + 2 * tc::A_BYTES;
-    uint64_t* bar = (uint64_t*)(Bs + tc::B_BYTES);       // MMA completion
-    uint32_t* tslot = (uint32_t*)(bar + 1);
-    __shared__ float bias[NC];
+    unsigned char* As = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    unsigned char* Bs = As + C::STAGES * C::BYTES;
+    __shared__ ConvShared<LAYER> s;
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int m = tid & (tc::M - 1), ch = tid >> 7;
-    for (int k = tid; k < 2 * tc::A_BYTES / 16; k += tc::THREADS)   // finite values in unused rows
-        reinterpret_cast<uint4*>(As)[k] = make_uint4(0, 0, 0, 0);
-    fill_b<LAYER>(Bs, P, bias);
-    const uint32_t bar_m = tc::smem_addr(bar);
-    if (tid == 0) {
-        mbar_init(bar_m);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) tmem_alloc<tc::ACC_COLS>(tslot);
-    tc::fence_async_smem();
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-    const uint32_t tmem = *tslot;
-    const uint32_t a_base = tc::smem_addr(As), b_base = tc::smem_addr(Bs);
-    const float scale = (LAYER == 3 && s_dev) ? (float)*s_dev : 1.f;
-    const long long ntiles = (long long)d.n2 * d.n3 * nseg;
-    // tile -> x-row rowi = y + n2 z, segment start x0, length L (32-bit: the host keeps the
-    // tile count below 2^31)
-    auto geom = [&](int tile, int& rowi, int& x0, int& L) {
-        rowi = tile / nseg;
-        x0 = (tile - rowi * nseg) * lseg;
-        L = min(lseg, d.n1 - x0);
-    };
-    auto stage = [&](int tile, int b) {
-        int rowi, x0, L;
-        geom(tile, rowi, x0, L);
-        const int z = rowi / d.n2;
-        long long qb[9];
-        plane_bases(d, rowi - z * d.n2, z, qb);
-        stage_planes(a_base + b * tc::A_BYTES, in, d.n, qb, x0, L, d.n1);
-    };
-    if ((long long)blockIdx.x < ntiles) stage((int)blockIdx.x, 0);
-    uint32_t phase = 0;
+    const uint32_t tmem = conv_begin<LAYER>(s, Bs, P);
+    Runs run(d, tiles);
+    int e = 0;   // events so far: a run of `rows` outputs has rows + 2
     bool ok = true;
-    int k = 0;
-    for (int tile = (int)blockIdx.x; tile < ntiles; tile += (int)gridDim.x, ++k) {
-        const int b = k & 1;
-        const long long next = (long long)tile + gridDim.x;
-        if (next < ntiles) {   // the other buffer's MMAs completed in the previous iteration
-            stage((int)next, b ^ 1);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        tc::fence_async_smem();
-        tc::fence_before();
-        __syncthreads();
-        if (tid == 0) {
-            tc::fence_after();
-            const uint32_t abuf = a_base + b * tc::A_BYTES;
-            // tap t reads plane q = t / 3 shifted dx + 1 = t % 3 rows and accumulates into
-            // accumulator q (columns 16 q ..): nine independent chains of three MMAs, issued
-            // dx-major so that consecutive MMAs never share an accumulator
+    if (tid < C::COPY) {
+        constexpr int PER = (tc::STAGE_CELLS + C::COPY - 1) / C::COPY;
+        const uint32_t a_base = tc::smem_addr(As) + tid * 16;
+        const long long plane = (long long)d.n1 * d.n2;
+        auto staged = [&](int ev) {
+            tc::fence_async_smem();
+            tc::mbar_arrive(tc::smem_addr(&s.full[ev % C::STAGES]));
+        };
+        while (ok && run.next()) {
+            // cell tid + COPY p: (dz, half, group, cell j), point x0 - 1 + j of the group's x-row
+            const __nv_bfloat16* src[PER];
 #pragma unroll
-            for (int dx = 0; dx < 3; ++dx)
+            for (int p = 0; p < PER; ++p) {
+                const int c = min(tid + C::COPY * p, tc::STAGE_CELLS - 1);
+                const int j = c % tc::CELLS, g = c / tc::CELLS % tc::GROUPS, hz = c / (tc::CELLS * tc::GROUPS);
+                int z, x;
+                group_of(d, run.tile, g, z, x);
+                x = (x - 1 + j + d.n1) % d.n1;
+                src[p] = in + ((long long)(hz & 1) * d.n + wrap1(z + (hz >> 1) - 1, d.n3) * plane + x) * 8;
+            }
+            for (int k = 0; k < run.rows + 2; ++k, ++e) {
+                const int st = e % C::STAGES;
+                ok = e < C::STAGES || tc::mbar_wait(tc::smem_addr(&s.empty[st]), ring_parity<C::STAGES>(e) ^ 1u,
+                                                    tc::WAIT_NS, &s.quit);
+                if (!ok) break;
+                const long long row = (long long)wrap1(run.y0 - 1 + k, d.n2) * d.n1 * 8;
+                const uint32_t dst = a_base + st * C::BYTES;
 #pragma unroll
-                for (int q = 0; q < 9; ++q) {
-                    const int t = 3 * q + dx;
-                    tc::mma(tmem + NC * q, tc::desc(abuf + q * tc::PLANE + dx * 16, tc::A_LBO, tc::A_SBO),
-                            tc::desc(b_base + t * tc::B_TAP, tc::B_LBO, tc::B_SBO), dx > 0 ? 1u : 0u);
-                }
-            mma_commit(bar_m);
-        }
-        const bool done = tc::mbar_wait(bar_m, phase, wait_ns);
-        ok = __syncthreads_and(done) != 0;
-        tc::fence_after();
-        if (!ok) break;
-        phase ^= 1u;
-        int rowi, x0, L;
-        geom(tile, rowi, x0, L);
-        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        const long long i = (long long)rowi * d.n1 + x0 + m;
-        if (LAYER == 2) {
-            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            uint32_t part[9][8];   // the nine plane accumulators, loaded together
-#pragma unroll
-            for (int q = 0; q < 9; ++q) tc::ld8_nowait(taddr + NC * q + 8 * ch, part[q]);
-            tc::wait_ld();
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-#pragma unroll
-                for (int o = 0; o < 8; ++o) acc[o] += __uint_as_float(part[q][o]);
-            if (m < L) {
-                if (BWD)
-                    epilogue_bwd(acc, zin, gout, aout, d.n, i, ch);
-                else {
-                    float zv[8], g[8];
-#pragma unroll
-                    for (int o = 0; o < 8; ++o) {
-                        zv[o] = acc[o] + bias[8 * ch + o];
-                        g[o] = gelu_f(zv[o]);
-                    }
-                    if (zout) store8(zout + ((long long)ch * d.n + i) * 8, zv);
-                    store8(aout + ((long long)ch * d.n + i) * 8, g);
+                for (int p = 0; p < PER; ++p)
+                    if (tid + C::COPY * p < tc::STAGE_CELLS)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                                     :: "r"(dst + p * C::COPY * 16), "l"(src[p] + row) : "memory");
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                if (e >= C::FLIGHT) {
+                    asm volatile("cp.async.wait_group %0;" :: "n"(C::FLIGHT) : "memory");
+                    staged(e - C::FLIGHT);
                 }
             }
-        } else if (ch == 0) {
-            uint32_t part[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) tc::ld1_nowait(taddr + NC * q, part[q]);
-            tc::wait_ld();
-            float v = 0.f;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) v += __uint_as_float(part[q]);
-            if (m < L) yout[i] = scale * (v + bias[0]);
         }
-        tc::fence_before();   // the next tile's MMAs overwrite the accumulators
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        if (ok)
+            for (int ev = max(0, e - C::FLIGHT); ev < e; ++ev) staged(ev);
+    } else if (tid < C::COPY + 32) {
+        if (tid == C::COPY) {
+            const uint32_t a_base = tc::smem_addr(As), b_base = tc::smem_addr(Bs);
+            while (ok && run.next())
+                for (int k = 0; ok && k < run.rows + 2; ++k, ++e)
+                    ok = conv_issue<LAYER>(s, e, [&](int st, int sl) {
+                        // dx-major: consecutive MMAs never share an accumulator
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                            for (int dz = 0; dz < 3; ++dz)
+                                tc::mma<C::N>(tmem + EV * sl + C::N * dz,
+                                              tc::desc(a_base + st * C::BYTES + dz * tc::PLANE + dx * 16, tc::A_LBO,
+                                                       tc::A_SBO),
+                                              tc::desc(b_base + (3 * dz + dx) * (C::N / 16) * tc::B_TAP, tc::B_LBO,
+                                                       tc::B_SBO),
+                                              dx > 0 ? 1u : 0u);
+                    });
+        }
+    } else {
+        // warps of a group: 32 points (the lanes of tensor memory that the warp can read) and,
+        // in layer 2, 8 channels each; the groups take alternate events
+        const int w = warp - C::COPY / 32 - 1, ch = (w >> 2) & 1, set = w / C::EPI;
+        const int m = (warp & 3) * 32 + (tid & 31);
+        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const float scale = (LAYER == 3 && s_dev) ? (float)*s_dev : 1.f;
+        while (ok && run.next()) {
+            long long i;
+            const bool inside = point_of(d, run.tile, m, i);
+            i += (long long)run.y0 * d.n1;
+            for (int k = 0; k < run.rows + 2; ++k, ++e) {
+                if (C::SETS > 1 && e % C::SETS != set) continue;
+                if (k < 2) {   // nothing ends here yet
+                    ok = conv_acc<LAYER>(s, e, wait_ns);
+                    if (!ok) break;
+                    for (int b = 0; b < 3; ++b) conv_free<LAYER>(s, e - b);
+                    continue;
+                }
+                constexpr int W = LAYER == 2 ? 8 : 1;
+                uint32_t part[3][3][W];   // [dz][dy]
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy) {
+                    const int ev = e - 2 + dy;   // row y + dy - 1
+                    ok = conv_acc<LAYER>(s, ev, wait_ns);
+                    if (!ok) break;
+                    const uint32_t col = taddr + EV * (ev % C::SLOTS);
+#pragma unroll
+                    for (int dz = 0; dz < 3; ++dz) {
+                        if constexpr (LAYER == 2) tc::ld8_nowait(col + C::N * dz + NC * dy + 8 * ch, part[dz][dy]);
+                        else tc::ld1_nowait(col + C::N * dz + dy, part[dz][dy][0]);
+                    }
+                    tc::wait_ld();
+                    conv_free<LAYER>(s, ev);
+                }
+                if (!ok) break;
+                float acc[W];
+#pragma unroll
+                for (int o = 0; o < W; ++o) acc[o] = 0.f;
+#pragma unroll
+                for (int q = 0; q < 9; ++q)
+#pragma unroll
+                    for (int o = 0; o < W; ++o) acc[o] += __uint_as_float(part[q / 3][q % 3][o]);
+                if (inside) {
+                    const long long at = i + (long long)(k - 2) * d.n1;
+                    if constexpr (LAYER == 3) yout[at] = scale * (acc[0] + s.bias[0]);
+                    else if constexpr (BWD) epilogue_bwd(acc, zin, gout, aout, d.n, at, ch);
+                    else epilogue_fwd(acc, s.bias, zout, aout, d.n, at, ch);
+                }
+            }
+        }
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");   // no copy outlives the CTA
-    if (!ok) {
-        if (tid == 0) *err = 1.0;
-        // let the MMAs still in flight finish (bounded by the full limit, whatever wait_ns was)
-        // before the tensor memory they write is freed
-        tc::mbar_wait(bar_m, phase, tc::WAIT_NS);
-    }
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-    if (warp == 0) tmem_free<tc::ACC_COLS>(tmem);
+    if (!ok) conv_quit<LAYER>(s, err);
+    conv_end<LAYER>(s, tmem);
 }
 
 // ---------------------------------------------------------------- backward
@@ -743,9 +888,17 @@ __global__ void __launch_bounds__(256) k_net_loss(long long n, const float* __re
 // out[0] = sum x^2, out[1] = RMS of x
 __global__ void __launch_bounds__(256) k_rms32(long long n, const float* __restrict__ x, RedCtx rc) {
     float p = 0.f;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        p = fmaf(x[i], x[i], p);
+    const long long step = (long long)gridDim.x * blockDim.x;
+    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    // eight loads in flight, summed in order
+    for (; i + 7 * step < n; i += 8 * step) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = __ldg(x + i + k * step);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) p = fmaf(v[k], v[k], p);
+    }
+    for (; i < n; i += step) p = fmaf(x[i], x[i], p);
     double acc[1] = {(double)p};
     if (grid_reduce<1>(acc, rc.partials, rc.counter, rc.out) && threadIdx.x == 0)
         rc.out[1] = sqrt(acc[0] / (double)n);
@@ -1232,14 +1385,22 @@ static void net_check_error(of_grid* g) {
                "tensor-core convolution: an MMA completion was not seen within the wait limit");
 }
 
-// The tensor-core layers: x-rows cut into segments of at most 128 points, persistent grids
-// (layer 1: four CTAs per SM; layers 2 and 3: two, each with two A buffers).
-static void conv_geometry(of_grid* g, int& nseg, int& lseg, long long& tiles) {
-    nseg = (g->d.n1 + tc::M - 1) / tc::M;
-    lseg = (g->d.n1 + nseg - 1) / nseg;
-    tiles = (long long)g->d.n2 * g->d.n3 * nseg;
-    OF_REQUIRE(tiles < (1LL << 31) - 4LL * num_sms(), OF_EINVAL,
-               "grid too large for the network kernels (%lld row segments)", tiles);
+// The tensor-core layers: tiles of 16 groups of 8 points, walked along y by a persistent grid.
+static long long conv_tiles(of_grid* g) {
+    const long long groups = (long long)g->d.n3 * ((g->d.n1 + 7) / 8);
+    OF_REQUIRE((long long)g->d.n2 * g->d.n3 * ((g->d.n1 + tc::M - 1) / tc::M) < (1LL << 31) - 4LL * num_sms(), OF_EINVAL,
+               "grid too large for the network kernels (%lld points)", g->d.n);
+    return (groups + tc::GROUPS - 1) / tc::GROUPS;
+}
+template <int LAYER, typename... KArgs, typename... Args>
+static void launch_conv(of_grid* g, void (*kernel)(KArgs...), int& configured_device, Args... args) {
+    if (configured_device != g->device) {
+        OF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::smem<LAYER>()));
+        configured_device = g->device;
+    }
+    const long long tiles = conv_tiles(g);
+    const int grid = (int)std::min(tiles * g->d.n2, (long long)tc::Cfg<LAYER>::CTAS * num_sms());
+    launch_smem(kernel, grid, tc::threads<LAYER>(), tc::smem<LAYER>(), g->stream, g->d, tiles, args...);
 }
 
 // BWD: the data gradient (the kernel's weights P are then the backward array, its input the
@@ -1250,16 +1411,8 @@ static void launch_conv1_tc(of_grid* g, const float* r, const __nv_bfloat16* P, 
                             unsigned long long wait_ns, const __nv_bfloat16* zin = nullptr,
                             float* gout = nullptr) {
     static int configured_device = -1;
-    if (configured_device != g->device) {
-        OF_CUDA(cudaFuncSetAttribute(k_conv1_tc<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM1));
-        configured_device = g->device;
-    }
-    int nseg, lseg;
-    long long tiles;
-    conv_geometry(g, nseg, lseg, tiles);
-    const int grid = (int)std::max(1LL, std::min(tiles, 4LL * num_sms()));
-    launch_smem(k_conv1_tc<BWD>, grid, tc::THREADS, tc::SMEM1, g->stream, g->d, nseg, lseg, r, P, z1, a1,
-                rn, rms, sgn, g->s.scalars + SC_NET_ERR, wait_ns, zin, gout);
+    launch_conv<1>(g, k_conv1_tc<BWD>, configured_device, r, P, z1, a1, rn, rms, sgn,
+                   g->s.scalars + SC_NET_ERR, wait_ns, zin, gout);
 }
 
 template <int LAYER, bool BWD = false>
@@ -1268,17 +1421,8 @@ static void launch_conv_tc(of_grid* g, const __nv_bfloat16* in, const __nv_bfloa
                            unsigned long long wait_ns, const __nv_bfloat16* zin = nullptr,
                            float* gout = nullptr) {
     static int configured_device = -1;
-    if (configured_device != g->device) {
-        OF_CUDA(cudaFuncSetAttribute(k_conv_tc<LAYER, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     tc::SMEM));
-        configured_device = g->device;
-    }
-    int nseg, lseg;
-    long long tiles;
-    conv_geometry(g, nseg, lseg, tiles);
-    const int grid = (int)std::max(1LL, std::min(tiles, 2LL * num_sms()));
-    launch_smem(k_conv_tc<LAYER, BWD>, grid, tc::THREADS, tc::SMEM, g->stream, g->d, nseg, lseg, in, P,
-                zout, aout, y, s_dev, g->s.scalars + SC_NET_ERR, wait_ns, zin, gout);
+    launch_conv<LAYER>(g, k_conv_tc<LAYER, BWD>, configured_device, in, P, zout, aout, y, s_dev,
+                       g->s.scalars + SC_NET_ERR, wait_ns, zin, gout);
 }
 
 // algorithmic bytes of one application: r read by the RMS pass and by layer 1, a1 and a2
