@@ -137,8 +137,10 @@ __device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) {
 // They meet at mbarriers only, so that copies, MMAs and epilogues of successive rows overlap.
 // Layer 3 (one output channel) has the same form with three of 16 columns used per dz; layer 1
 // (one input channel) is one GEMM per row with the 27 taps as K, padded to 32.
-// Time of one application on 192^3, against one tile per barrier round with every thread in
-// every part: see the layers' kernels.
+// On 192^3 the three layers take 188, 253 and 127 us; with one 128-point run of an x-row per
+// barrier round, all threads in every part and 27 MMAs of N = 16, they took 320, 715 and 522.
+// Layers 1 and 2 are bound by the issue of the GELUs (erff: some 36 of 60 instructions per
+// value; without it layer 1 takes 116 us), layer 3 by its 9 MMAs per event, 4 KB of operand each.
 // Shared-memory operands are K-major without swizzle: core matrices of 8 rows x 16 bytes,
 // one per group of points (10 cells apart in layers 2 and 3).
 namespace tc {
@@ -172,11 +174,11 @@ template <> struct Cfg<1> {
     static constexpr int BYTES = L1_STAGE, B_BYTES = 2 * B_TAP;
 };
 template <> struct Cfg<2> {
-    static constexpr int COPY = 96, N = 48, DZ = 3, SLOTS = 3, STAGES = 8, FLIGHT = 6, EPI = 8, SETS = 2, CTAS = 1, COLS = 512, USES = 3;
+    static constexpr int COPY = 96, N = 48, DZ = 3, SLOTS = 3, STAGES = 8, FLIGHT = 3, EPI = 8, SETS = 2, CTAS = 1, COLS = 512, USES = 3;
     static constexpr int BYTES = STAGE, B_BYTES = 27 * B_TAP;
 };
 template <> struct Cfg<3> {
-    static constexpr int COPY = 96, N = 16, DZ = 3, SLOTS = 5, STAGES = 6, FLIGHT = 4, EPI = 4, SETS = 1, CTAS = 2, COLS = 256, USES = 3;
+    static constexpr int COPY = 96, N = 16, DZ = 3, SLOTS = 5, STAGES = 6, FLIGHT = 2, EPI = 4, SETS = 1, CTAS = 2, COLS = 256, USES = 3;
     static constexpr int BYTES = STAGE, B_BYTES = 9 * B_TAP;
 };
 template <int LAYER> constexpr int threads() { return Cfg<LAYER>::COPY + 32 + 32 * Cfg<LAYER>::EPI * Cfg<LAYER>::SETS; }
@@ -210,12 +212,15 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns,
                                           const volatile int* quit) {
     if (limit_ns == 0) return false;
-    if (mbar_test(bar, parity)) return true;
-    const unsigned long long t0 = now_ns();
+    unsigned long long t0 = 0;
     for (int k = 0; k < (1 << 22); ++k) {
         if (mbar_test(bar, parity)) return true;
+        if ((k & 15) != 15) continue;
         if (quit && *quit) return false;
-        if ((k & 63) == 63 && now_ns() - t0 > limit_ns) return false;
+        if ((k & 63) == 63) {   // the clock is read only in waits that last
+            if (t0 == 0) t0 = now_ns();
+            else if (now_ns() - t0 > limit_ns) return false;
+        }
     }
     return false;
 }
@@ -239,6 +244,26 @@ __device__ __forceinline__ void ld8_nowait(uint32_t taddr, uint32_t (&r)[8]) {
 }
 __device__ __forceinline__ void ld1_nowait(uint32_t taddr, uint32_t& r) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+}
+// ((p0 + p1) + p2) + ... over the planes q = 3 dz + dy, two channels to an instruction
+__device__ __forceinline__ void sum_planes(const uint32_t (&part)[3][3][1], float (&acc)[1]) {
+    float v = 0.f;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) v += __uint_as_float(part[q / 3][q % 3][0]);
+    acc[0] = v;
+}
+__device__ __forceinline__ void sum_planes(const uint32_t (&part)[3][3][8], float (&acc)[8]) {
+#pragma unroll
+    for (int o = 0; o < 8; o += 2) {
+        unsigned long long v, u;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(part[0][0][o]), "r"(part[0][0][o + 1]));
+#pragma unroll
+        for (int q = 1; q < 9; ++q) {
+            asm("mov.b64 %0, {%1, %2};" : "=l"(u) : "r"(part[q / 3][q % 3][o]), "r"(part[q / 3][q % 3][o + 1]));
+            asm("add.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(u));
+        }
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[o]), "=f"(acc[o + 1]) : "l"(v));
+    }
 }
 __device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -350,6 +375,14 @@ template <int COLS>
 __device__ __forceinline__ void tmem_free(uint32_t tmem) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(COLS) : "memory");
 }
+__device__ __forceinline__ bool elect_one() {   // one lane of a whole warp
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                  :: "r"(bar) : "memory");
@@ -418,9 +451,9 @@ __device__ __forceinline__ uint32_t conv_begin(ConvShared<LAYER>& s, unsigned ch
 // Every role ends here, whether it ran to its end or gave up: no copy and no MMA outlives the
 // CTA or the tensor memory it writes (bounded by the full limit, whatever wait_ns was).
 template <int LAYER>
-__device__ __forceinline__ void conv_end(ConvShared<LAYER>& s, uint32_t tmem) {
+__device__ __forceinline__ void conv_end(ConvShared<LAYER>& s, uint32_t tmem, bool one) {
     asm volatile("cp.async.wait_all;" ::: "memory");
-    if (threadIdx.x == tc::Cfg<LAYER>::COPY) {
+    if (one) {   // the lane that issued
         mma_commit(tc::smem_addr(&s.last));
         tc::mbar_wait(tc::smem_addr(&s.last), 0, tc::WAIT_NS, nullptr);
     }
@@ -439,20 +472,25 @@ __device__ __forceinline__ void conv_quit(ConvShared<LAYER>& s, double* err) {
 template <int R>
 __device__ __forceinline__ uint32_t ring_parity(int e) { return (uint32_t)(e / R) & 1u; }
 
-// The issuing thread's part of event e: waits for its operand and for free columns; issue()
-// places the MMAs.
+// The issuing warp's part of event e: all lanes wait for its operand and for free columns, so that
+// what follows is uniform to the warp; the lane that elect.sync chose (`one`) issues.  (Issued by
+// a lane chosen by its index the nine MMAs took 1100 cycles of a layer-2 event, four times the
+// tensor pipe's own time: 331 -> 258 us for the layer.)  issue() places the MMAs.
 template <int LAYER, typename F>
-__device__ __forceinline__ bool conv_issue(ConvShared<LAYER>& s, int e, F issue) {
+__device__ __forceinline__ bool conv_issue(ConvShared<LAYER>& s, int e, bool one, F issue) {
     using C = tc::Cfg<LAYER>;
     const int st = e % C::STAGES, sl = e % C::SLOTS;
-    if (!tc::mbar_wait(tc::smem_addr(&s.full[st]), ring_parity<C::STAGES>(e), tc::WAIT_NS, &s.quit)) return false;
-    if (e >= C::SLOTS &&
-        !tc::mbar_wait(tc::smem_addr(&s.free[sl]), ring_parity<C::SLOTS>(e) ^ 1u, tc::WAIT_NS, &s.quit))
-        return false;
+    bool ok = tc::mbar_wait(tc::smem_addr(&s.full[st]), ring_parity<C::STAGES>(e), tc::WAIT_NS, &s.quit);
+    if (e >= C::SLOTS)
+        ok = ok && tc::mbar_wait(tc::smem_addr(&s.free[sl]), ring_parity<C::SLOTS>(e) ^ 1u, tc::WAIT_NS, &s.quit);
+    if (!__all_sync(0xffffffffu, ok)) return false;
     tc::fence_after();
-    issue(st, sl);
-    mma_commit(tc::smem_addr(&s.empty[st]));
-    mma_commit(tc::smem_addr(&s.acc[sl]));
+    if (one) {
+        issue(st, sl);
+        mma_commit(tc::smem_addr(&s.empty[st]));
+        mma_commit(tc::smem_addr(&s.acc[sl]));
+    }
+    __syncwarp();
     return true;
 }
 // one warp's wait for the accumulators of event e, all lanes alike
@@ -475,10 +513,12 @@ __device__ __forceinline__ void conv_free(ConvShared<LAYER>& s, int e) {
 // bias, GELU and the stores of 8 channels of point i
 __device__ __forceinline__ void epilogue_fwd(const float (&acc)[8], const float* bias, __nv_bfloat16* zout,
                                              __nv_bfloat16* aout, long long n, long long i, int ch) {
-    float zv[8], g[8];
+    float zv[8], g[8], b[8];
+    *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(bias + 8 * ch);
+    *reinterpret_cast<float4*>(b + 4) = *reinterpret_cast<const float4*>(bias + 8 * ch + 4);
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
-        zv[o] = acc[o] + bias[8 * ch + o];
+        zv[o] = acc[o] + b[o];
         g[o] = gelu_f(zv[o]);
     }
     if (zout) store8(zout + ((long long)ch * n + i) * 8, zv);
@@ -510,7 +550,7 @@ __global__ void __launch_bounds__(tc::threads<1>(), tc::Cfg<1>::CTAS)
     const uint32_t tmem = conv_begin<1>(s, Bs, P);
     Runs run(d, tiles);
     int e = 0;
-    bool ok = true;
+    bool ok = true, one = false;
     if (warp < 4) {
         // the input scaled by sgn / RMS (forward), or as it is (data gradient)
         const double rms = BWD ? 1.0 : *s_dev;
@@ -582,18 +622,18 @@ __global__ void __launch_bounds__(tc::threads<1>(), tc::Cfg<1>::CTAS)
             }
         }
     } else if (warp == 4) {
-        if (tid == C::COPY) {
-            const uint32_t a_base = tc::smem_addr(As), b_base = tc::smem_addr(Bs);
-            while (ok && run.next())
-                for (int k = 0; ok && k < run.rows; ++k, ++e)
-                    ok = conv_issue<1>(s, e, [&](int st, int sl) {
+        const uint32_t a_base = tc::smem_addr(As), b_base = tc::smem_addr(Bs);
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        one = elect_one();
+        while (ok && run.next())
+            for (int k = 0; ok && k < run.rows; ++k, ++e)
+                ok = conv_issue<1>(s, e, one, [&](int st, int sl) {
 #pragma unroll
-                        for (int h = 0; h < 2; ++h)
-                            tc::mma<C::N>(tmem + C::N * sl,
-                                          tc::desc(a_base + st * C::BYTES + 2 * h * tc::L1_KB, tc::L1_KB, 128),
-                                          tc::desc(b_base + h * tc::B_TAP, tc::B_LBO, tc::B_SBO), h > 0 ? 1u : 0u);
-                    });
-        }
+                    for (int h = 0; h < 2; ++h)
+                        tc::mma<C::N>(tm + C::N * sl,
+                                      tc::desc(a_base + st * C::BYTES + 2 * h * tc::L1_KB, tc::L1_KB, 128),
+                                      tc::desc(b_base + h * tc::B_TAP, tc::B_LBO, tc::B_SBO), h > 0 ? 1u : 0u);
+                });
     } else {
         const int m = (warp & 3) * 32 + (tid & 31), ch = (warp - 5) >> 2;
         const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 8 * ch;
@@ -619,7 +659,7 @@ __global__ void __launch_bounds__(tc::threads<1>(), tc::Cfg<1>::CTAS)
         }
     }
     if (!ok) conv_quit<1>(s, err);
-    conv_end<1>(s, tmem);
+    conv_end<1>(s, tmem, one);
 }
 
 // Layers 2 and 3 (see above).  LAYER 2: in = a1 -> z2 (optional), a2.  LAYER 3: in = a2 ->
@@ -641,7 +681,7 @@ __global__ void __launch_bounds__(tc::threads<LAYER>(), tc::Cfg<LAYER>::CTAS)
     const uint32_t tmem = conv_begin<LAYER>(s, Bs, P);
     Runs run(d, tiles);
     int e = 0;   // events so far: a run of `rows` outputs has rows + 2
-    bool ok = true;
+    bool ok = true, one = false;
     if (tid < C::COPY) {
         constexpr int PER = (tc::STAGE_CELLS + C::COPY - 1) / C::COPY;
         const uint32_t a_base = tc::smem_addr(As) + tid * 16;
@@ -685,24 +725,22 @@ __global__ void __launch_bounds__(tc::threads<LAYER>(), tc::Cfg<LAYER>::CTAS)
         if (ok)
             for (int ev = max(0, e - C::FLIGHT); ev < e; ++ev) staged(ev);
     } else if (tid < C::COPY + 32) {
-        if (tid == C::COPY) {
-            const uint32_t a_base = tc::smem_addr(As), b_base = tc::smem_addr(Bs);
-            while (ok && run.next())
-                for (int k = 0; ok && k < run.rows + 2; ++k, ++e)
-                    ok = conv_issue<LAYER>(s, e, [&](int st, int sl) {
-                        // dx-major: consecutive MMAs never share an accumulator
+        const uint32_t a_base = tc::smem_addr(As), b_base = tc::smem_addr(Bs);
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        one = elect_one();
+        while (ok && run.next())
+            for (int k = 0; ok && k < run.rows + 2; ++k, ++e)
+                ok = conv_issue<LAYER>(s, e, one, [&](int st, int sl) {
+                    const uint64_t a0 = tc::desc(a_base + st * C::BYTES, tc::A_LBO, tc::A_SBO);
+                    const uint64_t b0 = tc::desc(b_base, tc::B_LBO, tc::B_SBO);
+                    // dx-major: consecutive MMAs never share an accumulator
 #pragma unroll
-                        for (int dx = 0; dx < 3; ++dx)
+                    for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
-                            for (int dz = 0; dz < 3; ++dz)
-                                tc::mma<C::N>(tmem + EV * sl + C::N * dz,
-                                              tc::desc(a_base + st * C::BYTES + dz * tc::PLANE + dx * 16, tc::A_LBO,
-                                                       tc::A_SBO),
-                                              tc::desc(b_base + (3 * dz + dx) * (C::N / 16) * tc::B_TAP, tc::B_LBO,
-                                                       tc::B_SBO),
-                                              dx > 0 ? 1u : 0u);
-                    });
-        }
+                        for (int dz = 0; dz < 3; ++dz)
+                            tc::mma<C::N>(tm + EV * sl + C::N * dz, a0 + (dz * tc::PLANE + dx * 16) / 16,
+                                          b0 + (3 * dz + dx) * (C::N / 16) * tc::B_TAP / 16, dx > 0 ? 1u : 0u);
+                });
     } else {
         // warps of a group: 32 points (the lanes of tensor memory that the warp can read) and,
         // in layer 2, 8 channels each; the groups take alternate events
@@ -727,7 +765,8 @@ __global__ void __launch_bounds__(tc::threads<LAYER>(), tc::Cfg<LAYER>::CTAS)
 #pragma unroll
                 for (int dy = 0; dy < 3; ++dy) {
                     const int ev = e - 2 + dy;   // row y + dy - 1
-                    ok = conv_acc<LAYER>(s, ev, wait_ns);
+                    // this warp waited for event e - 2 in its last visit, and MMAs end in order
+                    if (dy == 1) ok = conv_acc<LAYER>(s, e, wait_ns);
                     if (!ok) break;
                     const uint32_t col = taddr + EV * (ev % C::SLOTS);
 #pragma unroll
@@ -735,17 +774,14 @@ __global__ void __launch_bounds__(tc::threads<LAYER>(), tc::Cfg<LAYER>::CTAS)
                         if constexpr (LAYER == 2) tc::ld8_nowait(col + C::N * dz + NC * dy + 8 * ch, part[dz][dy]);
                         else tc::ld1_nowait(col + C::N * dz + dy, part[dz][dy][0]);
                     }
+                    if (dy == 1) continue;   // the two later events' loads end together
                     tc::wait_ld();
+                    if (dy == 2) conv_free<LAYER>(s, ev - 1);
                     conv_free<LAYER>(s, ev);
                 }
                 if (!ok) break;
                 float acc[W];
-#pragma unroll
-                for (int o = 0; o < W; ++o) acc[o] = 0.f;
-#pragma unroll
-                for (int q = 0; q < 9; ++q)
-#pragma unroll
-                    for (int o = 0; o < W; ++o) acc[o] += __uint_as_float(part[q / 3][q % 3][o]);
+                tc::sum_planes(part, acc);
                 if (inside) {
                     const long long at = i + (long long)(k - 2) * d.n1;
                     if constexpr (LAYER == 3) yout[at] = scale * (acc[0] + s.bias[0]);
@@ -756,7 +792,7 @@ __global__ void __launch_bounds__(tc::threads<LAYER>(), tc::Cfg<LAYER>::CTAS)
         }
     }
     if (!ok) conv_quit<LAYER>(s, err);
-    conv_end<LAYER>(s, tmem);
+    conv_end<LAYER>(s, tmem, one);
 }
 
 // ---------------------------------------------------------------- backward
