@@ -37,15 +37,6 @@ __device__ __forceinline__ double sqrt_newton(double x) {
     return x * y;
 }
 
-// 1/x by Newton's method y <- y (2 - x y), written as e = 1 - x y, y <- y + y e, from a
-// single-precision seed (two FP64 steps: 1e-7 -> 1e-14 -> rounding); x a normal float.
-__device__ __forceinline__ double rcp_newton(double x) {
-    double y = (double)__frcp_rn((float)x);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) y = fma(y, fma(-x, y, 1.0), y);
-    return y;
-}
-
 // e = eps_xc(rho) * rho and v = V_xc(rho) for the exchange (Slater) and PZ correlation.
 __device__ __forceinline__ void lda_xc(double rho, double& e, double& v) {
     const double r = fmax(rho, OF_RHO_FLOOR);
@@ -80,47 +71,69 @@ __device__ __forceinline__ void thomas_fermi(double rho, double& e, double& v) {
     v = (5.0 / 3.0) * OF_CF * c2;
 }
 
-// Energy densities only (line-search evaluations): C_F rho^{5/3} + eps_xc(rho) rho, one
-// reciprocal cube root shared by both terms.
-__device__ __forceinline__ double tf_xc_energy(double rho) {
-    const double r = fmax(rho, OF_RHO_FLOOR);
-    const double t = inv_cbrt(r);
-    const double c = r * t * t;                     // rho^{1/3}
-    const double etf = rho > 0.0 ? OF_CF * rho * c * c : 0.0;
-    const double rs = OF_RS0 * t;
-    double ec;
-    if (rs >= 1.0) {
-        ec = PZ_G1 / (1.0 + PZ_B1 * sqrt_newton(rs) + PZ_B2 * rs);
-    } else {
-        const double lr = log(rs);
-        ec = PZ_A1 * lr + PZ_BB1 + PZ_C1 * rs * lr + PZ_D1 * rs;
-    }
-    return etf + (-0.75 * OF_CX * c + ec) * r;
+// ---- TF and xc at a density given by its amplitude, rho = c2 x^2
+// The forms that the minimisation evaluates at every point, hundreds of times per ground state.
+// GB300 runs FP64 at 2 operations per clock and SM, so these are bound by their count: with t =
+// x^{-1/3} every power needed is a product (rho^{1/3} = c2^{1/3} x t, sqrt(r_s) = ks t), one root
+// stands for the cube root and the square root of lda_xc, each Newton step is of third order (one
+// step from a single-precision seed: 1e-7 -> 1e-21), and seeds are converted by integer shifts
+// (an FP64 conversion costs as much as a multiply-add).  29 FP64 operations per point of the
+// line's energy and slope where two roots, a reciprocal and three conversions took 65: 112 -> 65
+// us on 96^3; the Hamiltonian's sweep, which also divided, 132 -> 72 us.
+struct XcScale {
+    double c2, k3, ks, lo;   // c2^{1/3}, sqrt(OF_RS0) c2^{-1/6}, the least x taken here
+};
+inline XcScale xc_scale(double c2) {
+    const double k3 = cbrt(c2);
+    // rho >= 100 OF_RHO_FLOOR, and x far from the ends of single precision
+    return {c2, k3, sqrt(OF_RS0 / k3), fmax(1e-11, 1e-11 / sqrt(c2))};
 }
-
-// Energy density and its derivative along the line (slope line search): e = C_F rho^{5/3} +
-// eps_xc(rho) rho as in tf_xc_energy, v = dE/drho = V_TF + V_xc, one reciprocal cube root and
-// one Newton reciprocal of the Perdew-Zunger denominator shared by both.
-__device__ __forceinline__ void tf_xc_energy_slope(double rho, double& e, double& v) {
-    const double r = fmax(rho, OF_RHO_FLOOR);
-    const double t = inv_cbrt(r);
-    const double c = r * t * t;                     // rho^{1/3}
-    const double tf = rho > 0.0 ? OF_CF * c * c : 0.0;   // C_F rho^{2/3}
-    const double rs = OF_RS0 * t;
-    double ec, vc;
-    if (rs >= 1.0) {
-        const double sq = sqrt_newton(rs);
-        const double inv = rcp_newton(1.0 + PZ_B1 * sq + PZ_B2 * rs);
+// positive values inside the normal range of single precision
+__device__ __forceinline__ float narrow_positive(double v) {   // truncated
+    return __uint_as_float((((unsigned)__double2hiint(v) - (896u << 20)) << 3) | ((unsigned)__double2loint(v) >> 29));
+}
+__device__ __forceinline__ double widen_positive(float v) {
+    const unsigned b = __float_as_uint(v);
+    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+}
+// rho^{1/3}, eps_c and V_c at rho = c2 x^2; false (nothing computed) outside lo <= x <= 1e15
+__device__ __forceinline__ bool xc_of_amplitude(double x, const XcScale& S, double& c, double& ec, double& vc) {
+    if (!(x >= S.lo && x <= 1e15)) return false;
+    double t = widen_positive(rcbrtf(narrow_positive(x)));
+    const double e = fma(-x, t * t * t, 1.0);       // x^{-1/3} = t (1 - e)^{-1/3}
+    t = fma(t, e * fma(e, 2.0 / 9.0, 1.0 / 3.0), t);
+    c = S.k3 * (x * t);
+    const double sq = S.ks * t;                     // sqrt(r_s)
+    if (sq >= 1.0) {
+        const double den = fma(sq, fma(PZ_B2, sq, PZ_B1), 1.0);
+        double inv = widen_positive(__frcp_rn(narrow_positive(den)));
+        const double f = fma(-den, inv, 1.0);       // 1 / den = inv / (1 - f)
+        inv = fma(inv, fma(f, f, f), inv);
         ec = PZ_G1 * inv;
-        vc = (PZ_G1 + (7.0 / 6.0) * PZ_G1 * PZ_B1 * sq + (4.0 / 3.0) * PZ_G1 * PZ_B2 * rs) * inv * inv;
+        vc = ec * inv * fma(sq, fma((4.0 / 3.0) * PZ_B2, sq, (7.0 / 6.0) * PZ_B1), 1.0);
     } else {
+        const double rs = sq * sq;
         const double lr = log(rs);
         ec = PZ_A1 * lr + PZ_BB1 + PZ_C1 * rs * lr + PZ_D1 * rs;
         vc = (PZ_A1 + (2.0 / 3.0) * PZ_C1 * rs) * lr + (PZ_BB1 - PZ_A1 / 3.0) +
              (1.0 / 3.0) * (2.0 * PZ_D1 - PZ_C1) * rs;
     }
-    e = tf * rho + (-0.75 * OF_CX * c + ec) * r;
-    v = (5.0 / 3.0) * tf - OF_CX * c + vc;
+    return true;
+}
+// v = V_TF + V_xc and the energy densities per rho: eps = C_F rho^{2/3} + eps_xc
+__device__ __forceinline__ void tf_xc_of_amplitude(double w, const XcScale& S, double& eps, double& v) {
+    double c, ec, vc;
+    if (xc_of_amplitude(fabs(w), S, c, ec, vc)) {
+        eps = fma(c, fma(OF_CF, c, -0.75 * OF_CX), ec);
+        v = fma(c, fma((5.0 / 3.0) * OF_CF, c, -OF_CX), vc);
+    } else {   // a vanishing density: the floors of the separate forms
+        const double rho = S.c2 * w * w, r = fmax(rho, OF_RHO_FLOOR);
+        double etf, vtf, exc, vxc;
+        thomas_fermi(rho, etf, vtf);
+        lda_xc(rho, exc, vxc);
+        eps = rho > 0.0 ? etf / rho + exc / r * (r / rho) : 0.0;
+        v = vtf + vxc;
+    }
 }
 
 }  // namespace of

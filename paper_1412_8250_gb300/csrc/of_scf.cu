@@ -26,6 +26,7 @@
 
 #include "of_fix.cuh"
 #include "of_functional.cuh"
+#include "of_pow.cuh"
 #include "of_pool.cuh"
 #include "of_stencil.cuh"
 
@@ -68,17 +69,16 @@ struct OpHamiltonian {
     double* Hu;
     double* Lu;        // may be null
     FnParams fn;
+    XcScale xs;        // of c2 = 1
     RedCtx rc;
     double acc[2];
     __device__ bool begin() { acc[0] = acc[1] = 0.0; return true; }
     __host__ __device__ const double* field() const { return u; }
     __device__ double load(long long i) const { return __ldg(u + i); }
     __device__ void store(long long i, double c, double lap) {
-        const double rho = c * c;
-        double etf, vtf, exc, vxc;
-        thomas_fermi(rho, etf, vtf);
-        lda_xc(rho, exc, vxc);
-        double pot = vtf + vxc + phi[i];
+        double eps, v;
+        tf_xc_of_amplitude(c, xs, eps, v);
+        double pot = v + phi[i];
         if (V) pot += fn.mu * V[i];
         const double h = -0.5 * fn.lam * lap + pot * c;
         Hu[i] = h;
@@ -124,6 +124,7 @@ struct OpEnergy {
     const double* u;
     const double* b;
     const double* phi;
+    XcScale xs;   // of c2 = 1
     RedCtx rc;
     double acc[4];
     __device__ bool begin() { acc[0] = acc[1] = acc[2] = acc[3] = 0.0; return true; }
@@ -131,9 +132,14 @@ struct OpEnergy {
     __device__ double load(long long i) const { return __ldg(u + i); }
     __device__ void store(long long i, double c, double lap) {
         const double rho = c * c;
-        double etf, vtf, exc, vxc;
-        thomas_fermi(rho, etf, vtf);
-        lda_xc(rho, exc, vxc);
+        double etf, exc, cr, ec, vc;
+        if (xc_of_amplitude(fabs(c), xs, cr, ec, vc)) {
+            etf = OF_CF * rho * (cr * cr);
+            exc = fma(-0.75 * OF_CX, cr, ec) * rho;
+        } else {
+            thomas_fermi(rho, etf, vc);
+            lda_xc(rho, exc, vc);
+        }
         acc[0] += etf;
         acc[1] += c * lap;
         acc[2] += exc;
@@ -245,31 +251,35 @@ __global__ void __launch_bounds__(256) k_line_moments(long long n, const double*
 
 // sum of TF + xc energy densities at rho = c2 (u + s d)^2
 __global__ void __launch_bounds__(256) k_line_energy(long long n, const double* u, const double* d,
-                                                     double s, double c2, RedCtx rc) {
+                                                     double s, XcScale xs, RedCtx rc) {
     double acc[1] = {0.0};
     GRID_LOOP(i, n) {
-        const double w = u[i] + s * d[i];
-        acc[0] += tf_xc_energy(c2 * w * w);
+        const double w = fma(s, d[i], u[i]);
+        double eps, v;
+        tf_xc_of_amplitude(w, xs, eps, v);
+        acc[0] = fma(eps, w * w, acc[0]);
     }
+    acc[0] *= xs.c2;
     grid_reduce<1>(acc, rc.partials, rc.counter, rc.out);
 }
 
 // With w = u + s d and rho = c2 w^2: sums of e(rho), v(rho) w^2 and v(rho) w d, e the TF + xc
 // energy density and v = de/drho.  The line derivative of the TF + xc energy follows from them.
 __global__ void __launch_bounds__(256) k_line_energy_slope(long long n, const double* u,
-                                                           const double* d, double s, double c2,
+                                                           const double* d, double s, XcScale xs,
                                                            RedCtx rc) {
     double acc[3] = {0.0, 0.0, 0.0};
     GRID_LOOP(i, n) {
         const double di = d[i];
         const double w = fma(s, di, u[i]);
-        double e, v;
-        tf_xc_energy_slope(c2 * w * w, e, v);
-        const double vw = v * w;
-        acc[0] += e;
-        acc[1] += vw * w;
-        acc[2] += vw * di;
+        double eps, v;
+        tf_xc_of_amplitude(w, xs, eps, v);
+        const double w2 = w * w;
+        acc[0] = fma(eps, w2, acc[0]);
+        acc[1] = fma(v, w2, acc[1]);
+        acc[2] = fma(v * w, di, acc[2]);
     }
+    acc[0] *= xs.c2;
     grid_reduce<3>(acc, rc.partials, rc.counter, rc.out);
 }
 
@@ -304,23 +314,37 @@ __global__ void k_density_plus(long long n, const double* u, const double* b, do
     GRID_LOOP(i, n) y[i] = u[i] * u[i] + b[i];
 }
 
+// uf^{2 alpha} and uf^{2 beta}, uf > 0: one logarithm and two exponentials in integer arithmetic
+// (of_pow.cuh); pow() for amplitudes and exponents outside its range.
+__device__ __forceinline__ void two_powers(double uf, const PowExp& ea, const PowExp& eb, double& a, double& b) {
+    bool ok = false;
+    int k;
+    long long f;
+    if (ea.fixed != 0 && eb.fixed != 0 && log2_fixed(uf, k, f)) ok = exp2_fixed(ea, k, f, a) && exp2_fixed(eb, k, f, b);
+    if (!ok) {
+        a = pow(uf, ea.e);
+        b = pow(uf, eb.e);
+    }
+}
+
 // g_a = max(u, floor)^{2 alpha}, g_b = max(u, floor)^{2 beta}
-__global__ void k_powers(long long n, const double* u, double two_a, double two_b, double* ga,
-                         double* gb) {
+__global__ void k_powers(long long n, const double* u, PowExp ea, PowExp eb, double* ga, double* gb) {
     GRID_LOOP(i, n) {
-        const double uf = fmax(u[i], OF_U_FLOOR);
-        ga[i] = pow(uf, two_a);
-        gb[i] = pow(uf, two_b);
+        double a, b;
+        two_powers(fmax(u[i], OF_U_FLOOR), ea, eb, a, b);
+        ga[i] = a;
+        gb[i] = b;
     }
 }
 
 // The density powers of the second-order kernel term: g[j] = u^{2(j + alpha)} and
 // g[3 + j] = u^{2(j + beta)}, j = 0..2 (u raised to the floor)
-__global__ void k_powers6(long long n, const double* u, double two_a, double two_b, double* g) {
+__global__ void k_powers6(long long n, const double* u, PowExp ea, PowExp eb, double* g) {
     GRID_LOOP(i, n) {
         const double uf = fmax(u[i], OF_U_FLOOR);
         const double rho = uf * uf;
-        const double a = pow(uf, two_a), b = pow(uf, two_b);
+        double a, b;
+        two_powers(uf, ea, eb, a, b);
         g[i] = a;
         g[n + i] = a * rho;
         g[2 * n + i] = a * rho * rho;
@@ -906,7 +930,7 @@ static bool nlcg(of_grid* g, const FnParams& fn, double Ne, ScfVecs& v, double* 
     bool converged = false;
     for (int q = 0; q <= max_iter; ++q) {
         launch_field<false>(g, OpHamiltonian{u, phi, fn.mu != 0.0 ? V : nullptr, v.Hu, v.Lu, fn,
-                                                red_ctx(g, SC_UHU)});
+                                                xc_scale(1.0), red_ctx(g, SC_UHU)});
         launch(k_gradient, nb, 256, g->stream, n, v.Hu, u, g->s.scalars + SC_UHU, dV / Ne,
                                               q > 0 ? v.rp : nullptr, v.r, red_ctx(g, SC_RR));
         OF_LAUNCH_CHECK();
@@ -1000,7 +1024,7 @@ static bool nlcg(of_grid* g, const FnParams& fn, double Ne, ScfVecs& v, double* 
         auto energy = [&](double s) -> double {
             const double c2 = Ne / (uu + 2.0 * s * ud + s * s * dd);
             ProfScope ps(g, PC_LINE, 2.0 * sizeof(double) * (double)n);
-            launch(k_line_energy, nb, 256, g->stream, n, u, v.d, s, c2, red_ctx(g, SC_LINE));
+            launch(k_line_energy, nb, 256, g->stream, n, u, v.d, s, xc_scale(c2), red_ctx(g, SC_LINE));
             OF_LAUNCH_CHECK();
             const double tfxc = sc(g, SC_LINE) * dV;
             const double vw = -0.5 * fn.lam * c2 * (uLu_ + 2.0 * s * uLd + s * s * dLd);
@@ -1017,7 +1041,7 @@ static bool nlcg(of_grid* g, const FnParams& fn, double Ne, ScfVecs& v, double* 
             const double c2 = Ne / q;
             const double c2p = -c2 * (2.0 * ud + 2.0 * s * dd) / q;
             ProfScope ps(g, PC_LINE, 2.0 * sizeof(double) * (double)n);
-            launch(k_line_energy_slope, nb, 256, g->stream, n, u, v.d, s, c2, red_ctx(g, SC_SLOPE));
+            launch(k_line_energy_slope, nb, 256, g->stream, n, u, v.d, s, xc_scale(c2), red_ctx(g, SC_SLOPE));
             OF_LAUNCH_CHECK();
             double t[3];
             fetch_scalars(g, SC_SLOPE, 3, t);
@@ -1146,7 +1170,7 @@ static double lr_potential_l2(of_grid* g, const of_functional* fn, double kf2, c
     double* scratch = (double*)ws(g, WS_LR, sizeof(double) * 8 * (size_t)n);
     double* gp = scratch;            // six density powers
     double* f00 = scratch + 6 * n;   // -(1/kf2) L_h u^{2 alpha}, -(1/kf2) L_h u^{2 beta}
-    launch(k_powers6, nb, 256, g->stream, n, u, 2.0 * fn->alpha, 2.0 * fn->beta, gp);
+    launch(k_powers6, nb, 256, g->stream, n, u, pow_exp(2.0 * fn->alpha), pow_exp(2.0 * fn->beta), gp);
     OF_LAUNCH_CHECK();
     launch_field<false>(g, OpScaledLap{gp, f00, -1.0 / kf2});
     launch_field<false>(g, OpScaledLap{gp + 3 * n, f00 + n, -1.0 / kf2});
@@ -1193,7 +1217,7 @@ static double lr_potential_impl(of_grid* g, const of_functional* fn, double kf2,
     const int npairs = fn->n_terms / 2;
     double* scratch = (double*)ws(g, WS_LR, sizeof(double) * 4 * (size_t)n);
     double *ga = scratch, *gb = scratch + n, *fa = scratch + 2 * n, *fb = scratch + 3 * n;
-    launch(k_powers, nb, 256, g->stream, n, u, 2.0 * fn->alpha, 2.0 * fn->beta, ga, gb);
+    launch(k_powers, nb, 256, g->stream, n, u, pow_exp(2.0 * fn->alpha), pow_exp(2.0 * fn->beta), ga, gb);
     OF_LAUNCH_CHECK();
     // f_e = -(1/kf2) L u^{2e}  (the m = n = 0 right-hand side of Sec. 3.1)
     launch_field<false>(g, OpScaledLap{ga, fa, -1.0 / kf2});
@@ -1321,7 +1345,7 @@ static double grad_sq_sum(of_grid* g, const double* u) {
 static void energy_terms(of_grid* g, const of_functional* fn, const double* u, const double* b,
                          const double* phi, double t_lr_sum, double e_self, double e_c,
                          int vw_energy, of_scf_result* res) {
-    launch_field<false>(g, OpEnergy{u, b, phi, red_ctx(g, SC_EN)});
+    launch_field<false>(g, OpEnergy{u, b, phi, xc_scale(1.0), red_ctx(g, SC_EN)});
     double e[4];
     fetch_scalars(g, SC_EN, 4, e);
     const double dV = g->dV;
@@ -1518,7 +1542,7 @@ of_status of_hamiltonian_apply(of_grid* g, const of_functional* fn, const double
     }
     try {
         launch_field<false>(g, OpHamiltonian{u, phi, fn->mu != 0.0 ? vlr : nullptr, hu, nullptr,
-                                                fn_params(fn), red_ctx(g, SC_UHU)});
+                                                fn_params(fn), xc_scale(1.0), red_ctx(g, SC_UHU)});
         return OF_OK;
     } catch (const Error& e) {
         return e.code;
