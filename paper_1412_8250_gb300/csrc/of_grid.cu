@@ -7,6 +7,7 @@
 #include <cmath>
 
 #include "of_fix.cuh"
+#include "of_ring.cuh"
 
 namespace of {
 
@@ -115,7 +116,7 @@ void laplacian(of_grid* g, of_dtype dt, const void* x, void* y) {
     if (dt == OF_F64) {
         launch_field<false>(g, OpLap<double>{(const double*)x, (double*)y});
     } else if (dt == OF_F32) {
-        launch_stencil<float, 2>(g, g->w32, OpLap<float>{(const float*)x, (float*)y});
+        launch_field32(g, OpLap<float>{(const float*)x, (float*)y}, (const float*)y);
     } else {
         OF_REQUIRE(false, OF_EINVAL, "unknown dtype %d", (int)dt);
     }
