@@ -199,11 +199,10 @@ __device__ __forceinline__ void fix_planes(const longlong2 (&col)[BZ + 2 * N], c
     }
 }
 
+// One sweep over this block's bricks: op.store or op.store_pre at every point.
 template <int N, bool CPLX, bool ISO, int BZ, class Op>
-__global__ void __launch_bounds__(FX_THREADS, 3)
-fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int bricks, Op op) {
-    pdl_enter();
-    if (!op.begin()) return;
+__device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& W, const FixScale& fs, bool vec, int bx,
+                                          int by, int bricks, Op& op) {
     constexpr int HX = CPLX ? 2 * N : ((N + 1) & ~1);   // staged halo doubles each side in x
     constexpr int RW = fix_row_width<N, CPLX>();
     constexpr int ROWS = FX_BY + 2 * N;
@@ -380,7 +379,21 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
             }
         }
     }
+}
+
+template <int N, bool CPLX, bool ISO, int BZ, class Op>
+__global__ void __launch_bounds__(FX_THREADS, 3)
+fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int bricks, Op op) {
+    pdl_enter();
+    if (!op.begin()) return;
+    fix_sweep<N, CPLX, ISO, BZ>(d, W, fs, vec, bx, by, bricks, op);
     op.end();
+}
+
+inline FixScale fix_scale(of_grid* g) {
+    FixScale fs;
+    for (int a = 0; a < 3; ++a) fs.s[a] = std::ldexp(1.0, fix_shift(g->N)) / (fix_denominator(g->N) * g->h[a] * g->h[a]);
+    return fs;
 }
 
 template <int N, bool CPLX, bool ISO, int BZ, class Op>
@@ -426,8 +439,7 @@ void launch_field(of_grid* g, Op op) {
     }
     const int cls = OpInfo<Op>::cls >= 0 ? OpInfo<Op>::cls : PC_STENCIL_F64;
     ProfScope ps(g, cls, (double)OpInfo<Op>::words * (CPLX ? 16.0 : 8.0) * (double)g->d.n);
-    FixScale fs;
-    for (int a = 0; a < 3; ++a) fs.s[a] = std::ldexp(1.0, fix_shift(g->N)) / (fix_denominator(g->N) * g->h[a] * g->h[a]);
+    const FixScale fs = fix_scale(g);
     const bool iso = fs.s[0] == fs.s[1] && fs.s[1] == fs.s[2];
     switch (g->N * 2 + (iso ? 1 : 0)) {
         case 2: launch_fix_depth<1, CPLX, false>(g, fs, op); break;

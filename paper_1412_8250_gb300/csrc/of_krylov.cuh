@@ -459,6 +459,11 @@ inline void launch_krylov_update(of_grid* g, long long n, T* x, T* r, const T* p
     launch_pdl(krylov_update<T, PRECOND>, blocks, 256, 0, g->stream, n, x, r, p, Ap, st, rc);
 }
 
+// Plain FP64 CG on grids whose bricks are all resident at once, every iteration in one cooperative
+// launch (of_cg.cu): false where the grid is larger, nothing done.  Else the state read back.
+bool cg_resident(of_grid* g, int st_off, double* x, double* r, double* pa, double* pb, double* Ap, double a, double q,
+                 KState* h);
+
 inline int vec_blocks(long long n) { return red_blocks(n, 256 * 4); }
 
 // Preconditioned-CG scalars from the grid-reduced sums s = (r^T z, sum z, sum r) (projected:
