@@ -4,8 +4,8 @@
 Step = one complete ground state of the 108-atom 3x3x3 FCC Al-like cell (a = 7.6 bohr,
 +-0.1 bohr seeded displacements, Gaussian ions Z = 3), 96^3 grid, 12th-order FD, WT-type
 kernel functional, followed by the forces: of_scf_ground_state + of_forces through the C
-ABI.  The chosen form runs the Poisson and kernel solves as FP32 Krylov sweeps with FP64
-iterative refinement (Poisson inner CG preconditioned by a multigrid V-cycle); --precision
+ABI.  The chosen form solves the Poisson and kernel systems by direct FP32 corrections under FP64
+iterative refinement; --precision
 f64 runs the plain FP64 CG form.  The working set (~0.4 GB) sits in L2 between kernels of one
 step, so L2 is flushed (a 256 MiB write) between timed steps, outside the timed events.
 
@@ -41,20 +41,19 @@ WORKLOAD_DETAIL = {
     "nlcg": {"tol": 1e-7, "line_search": "root of dE/ds (secant), line_tol 1e-3",
              "inexact": "NLCG of outer step k stops at max(1e-7, 0.03 x fixed-point error of "
                         "step k-1); the last outer step at 1e-7",
-             "preconditioner": "chosen form: (-L_h + 0.01) (-L_h + 1.5)^-2 on the gradient (two "
-                               "multigrid V-cycles and one FP32 sweep), preconditioned "
+             "preconditioner": "chosen form: (-L_h + 0.01) (-L_h + 1.5)^-2 on the gradient (one "
+                               "direct FP32 solve), preconditioned "
                                "Polak-Ribiere (the real-space NLCG preconditioner Sec. 5.5 calls "
                                "for); plain FP64 form: none"},
-    "poisson": {"tol": 1e-10, "form": "FP32 multigrid-preconditioned CG passes to 3e-4 of "
-                                      "their starting residual, FP64 refinement"},
-    "kernel_solves": {"form": "FP32 COCG preconditioned by the V-cycle of -L + kf2 |Q|, FP64 "
-                              "refinement", "tol": "max(1e-10, min(1e-5, 1e-2 x previous "
+    "poisson": {"tol": 1e-10, "form": "direct FP32 corrections, FP64 refinement"},
+    "kernel_solves": {"form": "direct FP32 corrections, FP64 refinement", "tol": "max(1e-10, min(1e-5, 1e-2 x previous "
                                                   "fixed-point error))"},
 }
 GOLDEN_AL108 = os.path.join(ROOT, "tests", "golden", "al108_wt.json")
-# DRAM bytes (read + write) of one FP32 order-12 sweep of a 320^3 grid by the fast-path stencil,
-# from the ncu capture summarised in profiles/stencil_fp32_320.md (145.9 + 91.9 MB)
-STENCIL320_DRAM_BYTES = 237.8e6
+# DRAM bytes (read + write) of one order-12 sweep of a 320^3 grid, FP32 and FP64, from the ncu
+# capture summarised in profiles/sweeps_and_transforms.md (163.0 + 92.7 and 453.3 + 235.5 MB)
+STENCIL320_DRAM_BYTES = 255.7e6
+STENCIL320_F64_DRAM_BYTES = 688.8e6
 # DRAM bytes that one V-cycle plus one COCG iteration of the 96^3 complex FP32 pass moves,
 # summed over its kernels launched one by one from a cold L2 (ncu; the kernels' table is in
 # profiles/mg_cocg_pass_kernels_96.md)
@@ -305,9 +304,9 @@ def batched_compare(torch, B, W, reps=2):
     """64 uneven cells (reps 2..4 per axis, 64-128 points per axis, half with a vacancy, seed 3):
     the Poisson problem of each cell's initial density (uniform electrons plus its Gaussian
     nuclear charge), solved to relative residual 1e-10 by (a) one batched call of grouped
-    launches (plain FP32 CG + FP64 refinement), (b) one batched call in the multigrid form
-    (per-cell multigrid PCG over concurrent streams), (c) the single-grid solver cell by cell
-    with the same plain CG, (d) cell by cell with the multigrid-preconditioned CG."""
+    launches (plain FP32 CG + FP64 refinement), (b) one batched call in the default mixed form
+    (per-cell direct corrections over concurrent streams; reported under its earlier key), (c) the
+    single-grid solver cell by cell with the same plain CG, (d) cell by cell in the default mixed form."""
     cells = W.batched_cells()
     stream = torch.cuda.current_stream()
     grids, rhos, phis = [], [], []
@@ -382,7 +381,7 @@ def learned_compare(torch, B, W, steps=400, theta=0.3):
     4-atom 32^3 and the 108-atom 96^3 cells (64 residuals each; four Adam runs per cell, batch
     4), then used in the FP32 flexible CG of the Poisson solve of the 864-atom 6x6x6 cell,
     192^3 grid, same spacing, to true relative residual 1e-10; against the same solve with
-    plain (Jacobi) FP32 CG, plain FP64 CG and multigrid-preconditioned FP32 CG."""
+    plain (Jacobi) FP32 CG, plain FP64 CG and the default mixed form (key multigrid_pcg_mixed)."""
     import numpy as np
     stream = torch.cuda.current_stream()
     torch.cuda.synchronize()
@@ -465,7 +464,7 @@ def learned_shifted_compare(torch, B, W, g864, cell864, steps, theta):
     the FP32 flexible GMRES(8) of the same shifted system on the 864-atom 192^3 grid (a
     right-hand side not trained on) to true relative residual 1e-10; against the same solver
     with every network step refused (plain inner CG), plain FP32 COCG, plain FP64 COCG and
-    multigrid-preconditioned FP32 COCG.  Iterations count the inner steps too."""
+    the default mixed form (key multigrid_pcocg_mixed).  Iterations count the inner steps too."""
     import numpy as np
     from paper_1412_8250_gb300 import functionals as Fn
     fn = Fn.wt()
@@ -1488,7 +1487,7 @@ def main():
                                 "duration also spans the work beside it")
     roofline_320 = roofline_320_f64 = alu = None
     if stencil320:
-        roofline_320 = {"kernel": "stencil2_kernel (of_laplacian_apply, FP32, order 12, 320^3)",
+        roofline_320 = {"kernel": "ring_kernel (of_laplacian_apply, FP32, order 12, 320^3)",
                         "bound": "hbm", "achieved": stencil320["f32"]["gbs"], "peak": peak,
                         "unit": "GB/s", "frac": stencil320["f32"]["gbs"] / peak,
                         "traffic": STENCIL320_DRAM_BYTES, "bytes_per_launch": 8.0 * 320 ** 3,
@@ -1497,7 +1496,8 @@ def main():
         alu = alu_peaks(B, torch)
         roofline_320_f64 = {"kernel": "fix_kernel (of_laplacian_apply, FP64, order 12, 320^3)",
                             "bound": "hbm", "achieved": stencil320["f64"]["gbs"], "peak": peak,
-                            "unit": "GB/s", "frac": stencil320["f64"]["gbs"] / peak, "traffic": None,
+                            "unit": "GB/s", "frac": stencil320["f64"]["gbs"] / peak,
+                            "traffic": STENCIL320_F64_DRAM_BYTES,
                             "bytes_per_launch": 16.0 * 320 ** 3, "peak_kind": peak_kind,
                             "note": "instruction issue and latency of the integer sums, 5x the "
                                     "rate the FP64 pipe allows"}
