@@ -300,7 +300,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // Sums of K per-thread values over the block, into sums[K] of shared memory (the caller's barrier
-// makes them visible).  Up to 4 sums of at most 256 threads go through shared memory, warp k adding the
+// makes them visible).  Up to 16 sums of at most 256 threads go through shared memory, warp k adding the
 // values of sum k: an FP64 add occupies the pipe for 16 clocks per warp, and shuffles in every
 // warp took 45 of them per 256 threads and sum where this takes 13.
 template <int K>
@@ -308,16 +308,16 @@ __device__ __forceinline__ void block_sums(const double (&v)[K], double* sums) {
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const int nthreads = blockDim.x * blockDim.y * blockDim.z;
     const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
-    constexpr bool FLAT = K <= 4;
-    __shared__ double sh[FLAT ? 256 : 32][K > 0 ? K : 1];
+    constexpr bool FLAT = K <= 16;
+    __shared__ double sh[K > 0 ? K : 1][FLAT ? 256 : 32];
     __syncthreads();   // readers of an earlier call's values
     if (FLAT && nthreads <= 256) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) sh[tid][k] = v[k];
+        for (int k = 0; k < K; ++k) sh[k][tid] = v[k];
         __syncthreads();
         for (int k = warp; k < K; k += nwarps) {
             double s = 0.0;
-            for (int t = lane; t < nthreads; t += 32) s += sh[t][k];
+            for (int t = lane; t < nthreads; t += 32) s += sh[k][t];
             s = warp_sum(s);
             if (lane == 0) sums[k] = s;
         }
@@ -326,11 +326,11 @@ __device__ __forceinline__ void block_sums(const double (&v)[K], double* sums) {
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const double s = warp_sum(v[k]);
-        if (lane == 0) sh[warp][k] = s;
+        if (lane == 0) sh[k][warp] = s;
     }
     __syncthreads();
     for (int k = warp; k < K; k += nwarps) {
-        double s = lane < nwarps ? sh[lane][k] : 0.0;
+        double s = lane < nwarps ? sh[k][lane] : 0.0;
         s = warp_sum(s);
         if (lane == 0) sums[k] = s;
     }
