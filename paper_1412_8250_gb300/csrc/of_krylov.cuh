@@ -203,8 +203,8 @@ struct OpResidualDirect {
         if constexpr (KT<T>::cplx) {
             if (!act0) return;
             const double2 c = p.x;
-            const double2 rv = make_double2(fma(a, l0, p.b.x) - fma(Q.x, c.x, -Q.y * c.y),
-                                            fma(a, l1, p.b.y) - fma(Q.x, c.y, Q.y * c.x));
+            const double2 rv = make_double2(fma(a, l0, fma(-Q.x, c.x, fma(Q.y, c.y, p.b.x))),
+                                            fma(a, l1, fma(-Q.x, c.y, fma(-Q.y, c.x, p.b.y))));
             r[i] = rv;
             acc[0] = fma(rv.x, rv.x, fma(rv.y, rv.y, acc[0]));
         } else {
