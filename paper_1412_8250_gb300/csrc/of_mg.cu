@@ -1,5 +1,5 @@
 // Geometric multigrid V-cycle used as the preconditioner of the FP32 inner CG of the Poisson
-// solve.  The paper (Sec. 5.5) names multigrid as the way to stop the Poisson iteration count
+// solve where the direct corrections (of_fft.cu) do not apply or stall.  The paper (Sec. 5.5) names multigrid as the way to stop the Poisson iteration count
 // from growing with system size; this is that preconditioner on the periodic grid.
 //
 //  level 0   : the order-2N operator A = -L_h of Eq. FD:Laplacian (FP32)
