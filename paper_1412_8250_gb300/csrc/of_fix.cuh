@@ -13,16 +13,22 @@
 // Brick of 16 units x 8 rows x 8 planes per block of 128 threads, a unit being two neighbouring
 // doubles of a row (two real points, or one complex point).  The brick and its x-y halo are staged
 // once in shared memory as fixed point; each thread takes the z halo of its own column straight
-// from global memory.  The block's exponent is one above the largest of its z halo and of eight
-// staged rows spread over the brick.  A staged value beyond that, a value that is not finite, or a
-// stretch of staged values (8 x 1 x 8 points) that is not zero but 2^6 and more below the largest,
-// for which 60 bits would keep less than the 53 of FP64, makes the block take FP64 arithmetic
-// instead.  So a value's error is at most 2^-53 of the largest value of its stretch, and ordinary
-// fields take the integer path everywhere.
+// from global memory.  The block's range is 4/3 or more of the largest of its z halo and of eight
+// staged rows spread over the brick, and is set anew, from all values, where a staged one lies beyond
+// it; a value that is not finite makes the block take FP64 arithmetic instead.  So does every point
+// whose own value and whose six next ones (in z those of the brick) are all below 2^53 units of the
+// fixed point (2^-7 of its range), where 60 bits would keep fewer than the 53 of FP64.  At the others a staged value is cut off by at most 2^-53 of the largest of those
+// seven, and the sum is no less accurate than the FP64 one (on random and smooth stencils just above
+// the limit the RMS error is 0.3 .. 1 of it at orders 6 and 12, up to 1.5 at order 2 where the centre
+// alone is small).  A complex value counts by the larger of its parts.  Ordinary fields take the integer
+// path but for a few points where value and slope are small together (about ten in an electrostatic
+// potential on 96^3), fields that fall by powers of ten across a brick take FP64 arithmetic.
 //
-// Measured on a GB300 (order 12): 96^3 69.1 -> 12.7 us, 320^3 2.4 ms -> 0.41 ms (13.7 -> 80 GPts/s); now
-// bound by instruction issue and latency at 12 warps per SM (157 registers; 4.9 staged values per
-// point with their conversions, ~8 integer operations per distance).  Tried: both loads and
+// Measured on a GB300 (order 12): 96^3 69.1 us in FP64 arithmetic -> 13.4, 192^3 514 -> 101 (70 GPts/s), of
+// which the looks at each point's neighbours, and the code they add, are 0.8 and 10; where nearly every
+// point takes FP64 arithmetic after all (a Gaussian in the middle of 96^3) 69.  Bound by instruction issue
+// and latency at 12 warps per SM (168 registers; 4.9 staged values per point with their conversions, ~8
+// integer operations per distance).  Tried before the looks (12.7 us, 80 GPts/s at 320^3): both loads and
 // conversions of two slots in flight 13.8 us / 74 GPts/s (spills), two blocks per SM without spills
 // 16.1 / 80, 4 planes per brick 16.1 / 70, 16 rows 16.3 / 81, 16 rows of 4 planes 18.2 / 69.
 #pragma once
@@ -57,6 +63,13 @@ OF_FIX_HD long long fix_from_bits(int hi, unsigned lo, int E) {
     const long long v = (long long)((m << 7) >> s), sign = (long long)(hi >> 31);
     return (v ^ sign) - sign;
 }
+
+// magnitude of v's high word: |v| > 2^53 - 2^32 where it is at least FIX_FINE
+OF_FIX_HD unsigned fix_mag(long long v) {
+    const int h = (int)(v >> 32);
+    return (unsigned)(h < 0 ? -h : h);
+}
+constexpr unsigned FIX_FINE = 1u << 21;
 
 // A sum s of neighbours (64 bits) times W, by its two 32-bit limbs: the sum of W s is h 2^32 + p - n
 struct FixAcc {
@@ -110,6 +123,7 @@ uintptr_t fix_bits(const Op& op) {
 }
 
 constexpr int FX_UX = 16, FX_BY = 8, FX_THREADS = FX_UX * FX_BY;
+constexpr int FX_ITEMS = 32;   // units of a warp that its lanes take together in FP64 arithmetic
 
 struct FixScale {
     double s[3];   // 2^fix_shift / (D h_a^2)
@@ -199,6 +213,39 @@ __device__ __forceinline__ void fix_planes(const longlong2 (&col)[BZ + 2 * N], c
     }
 }
 
+// Those of the planes `small` (bits), in which the thread's unit is below `least`, in which a point of
+// it and its six neighbours all are; the neighbours in z only within the brick.
+template <int N, bool CPLX, int BZ>
+__device__ __forceinline__ unsigned fix_coarse(const long long* own, unsigned small, unsigned least) {
+    constexpr int RW = fix_row_width<N, CPLX>(), CPL = (FX_BY + 2 * N) * RW;
+    unsigned coarse = 0;
+#pragma unroll 1
+    for (; small; small &= small - 1u) {
+        const int k = __ffs((int)small) - 1;
+        const long long* b = own + k * CPL;
+        unsigned m0 = 0, m1 = 0;
+        auto near = [&](const long long* p) {
+            const longlong2 v = *reinterpret_cast<const longlong2*>(p);
+            m0 |= fix_mag(v.x);
+            m1 |= fix_mag(v.y);
+        };
+        near(b + RW);
+        near(b - RW);
+        near(k + 1 < BZ ? b + CPL : b);
+        near(k > 0 ? b - CPL : b);
+        if constexpr (CPLX) {
+            near(b + 2);
+            near(b - 2);
+            m0 = m1 = m0 | m1;
+        } else {
+            m0 |= fix_mag(b[-1]);
+            m1 |= fix_mag(b[2]);
+        }
+        coarse |= min(m0, m1) < least ? 1u << k : 0u;
+    }
+    return coarse;
+}
+
 // One sweep over this block's bricks: op.store or op.store_pre at every point.
 template <int N, bool CPLX, bool ISO, int BZ, class Op>
 __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& W, const FixScale& fs, bool vec, int bx,
@@ -215,41 +262,44 @@ __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& 
     constexpr bool ALL = SPT * BZ <= 8;   // thin bricks: every slot's loads in flight at once
     extern __shared__ __align__(16) long long fix_smem[];
     __shared__ int yoff[ROWS], zoff[BZ + 2 * N], xoff[RW];   // periodic offsets in doubles (< 2^31)
-    __shared__ int wmax[FX_THREADS / 32];
+    __shared__ int wtop[2][FX_THREADS / 32];
+    __shared__ unsigned char items[FX_THREADS / 32][FX_ITEMS];
+    __shared__ __align__(16) double2 taken[FX_THREADS / 32][FX_ITEMS];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + FX_UX * ty;
     const int RF = CPLX ? 2 * d.n1 : d.n1, PF = RF * d.n2;
     // Staged row and first column of each of this thread's slots.  The first FX_BY rows of the order
     // are spread evenly over the staged rows, so that the first slot's values (from which, with
     // the z halo, the block's exponent comes) sample the whole brick.
-    int srow[SPT], scol[SPT];
-#pragma unroll
-    for (int m = 0; m < SPT; ++m) {
+    auto slot = [&](int m, int& row, int& col) {
         const int sl = tid + m * FX_THREADS;
-        srow[m] = -1;
-        scol[m] = 0;
+        row = -1;
+        col = 0;
         if (sl < ROWS * FX_UX) {
             int j = sl / FX_UX;
             auto spread = [](int i) { return (i * (ROWS - 1) + 3) / (FX_BY - 1); };
             if (j < FX_BY) {
-                srow[m] = spread(j);
+                row = spread(j);
             } else {
                 j -= FX_BY;   // the j-th row that is not one of those
                 for (int i = 0; i < FX_BY; ++i) j += spread(i) <= j;
-                srow[m] = j;
+                row = j;
             }
-            scol[m] = HX + 2 * (sl % FX_UX);
+            col = HX + 2 * (sl % FX_UX);
         } else if (sl < SLOTS) {
             const int q = sl - ROWS * FX_UX, side = (q / PH) & 1, c = q % PH;
             if (c < HX / 2) {
-                srow[m] = N + q / (2 * PH);
-                scol[m] = 2 * c + (side ? HX + 32 : 0);
+                row = N + q / (2 * PH);
+                col = 2 * c + (side ? HX + 32 : 0);
             }
         }
-    }
+    };
+    int srow[SPT], scol[SPT];
+#pragma unroll
+    for (int m = 0; m < SPT; ++m) slot(m, srow[m], scol[m]);
     // two doubles of a chunk: one 16-byte load where rows and the field allow it (a chunk
     // starts at an even double and is contiguous across the wrap when rows are even)
-    auto load2 = [&](int base, int x0, int x1) -> double2 {
-        return fix_load(op, (unsigned)(base + x0), (unsigned)(base + x1), vec);
+    auto load2 = [&](int base, int x0, int x1, bool v) -> double2 {
+        return fix_load(op, (unsigned)(base + x0), (unsigned)(base + x1), v);
     };
     auto expo = [](double a) { return (__double2hiint(a) >> 20) & 0x7ff; };
 
@@ -264,66 +314,102 @@ __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& 
             else xoff[t] = wrap_index(x0 - HX + t, d.n1);
         }
         __syncthreads();
-        // the z halo of this thread's own column and its first slot in every plane; the largest
-        // exponent among them, plus two, is the block's
+        // the z halo of this thread's own column and its first slot in every plane, the sample that the
+        // block's exponent comes from
         const int own = yoff[N + ty], oc0 = xoff[HX + 2 * tx], oc1 = xoff[HX + 2 * tx + 1];
         longlong2 col[BZ + 2 * N];
         double2 v[ALL ? SPT : 1][BZ];
         auto load_slot = [&](int m, double2 (&v)[BZ]) {
             if (srow[m] < 0) return;
             const int o = yoff[srow[m]], c0 = xoff[scol[m]], c1 = xoff[scol[m] + 1];
+            // (the branch around the loads: in each of them it made the compiler issue both forms)
+            if (vec) {
 #pragma unroll
-            for (int k = 0; k < BZ; ++k) v[k] = load2(zoff[N + k] + o, c0, c1);
+                for (int k = 0; k < BZ; ++k) v[k] = load2(zoff[N + k] + o, c0, c1, true);
+            } else {
+#pragma unroll
+                for (int k = 0; k < BZ; ++k) v[k] = load2(zoff[N + k] + o, c0, c1, false);
+            }
         };
-        auto top = [&](double2 q) { return max(expo(q.x), expo(q.y)); };
         double2 zr[2 * N];
+        if (vec) {
 #pragma unroll
-        for (int j = 0; j < 2 * N; ++j) zr[j] = load2(zoff[j < N ? j : j + BZ] + own, oc0, oc1);
+            for (int j = 0; j < 2 * N; ++j) zr[j] = load2(zoff[j < N ? j : j + BZ] + own, oc0, oc1, true);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 2 * N; ++j) zr[j] = load2(zoff[j < N ? j : j + BZ] + own, oc0, oc1, false);
+        }
 #pragma unroll
         for (int m = 0; m < (ALL ? SPT : 1); ++m) load_slot(m, v[m]);
-        int emax = 0;
+        auto block_max = [&](int v, int (&slot)[FX_THREADS / 32]) {
+            const int w = __reduce_max_sync(0xffffffffu, v);
+            if ((tid & 31) == 0) slot[tid >> 5] = w;
+            __syncthreads();
+            int t = 0;
 #pragma unroll
-        for (int j = 0; j < 2 * N; ++j) emax = max(emax, top(zr[j]));
+            for (int k = 0; k < FX_THREADS / 32; ++k) t = max(t, slot[k]);
+            return t;
+        };
+        int first = 0;   // the largest exponent and mantissa of the sample
+        auto sample = [&](double2 q) {
+            first = max(first, max(__double2hiint(q.x) & 0x7fffffff, __double2hiint(q.y) & 0x7fffffff));
+        };
+#pragma unroll
+        for (int j = 0; j < 2 * N; ++j) sample(zr[j]);
 #pragma unroll
         for (int m = 0; m < (ALL ? SPT : 1); ++m)
             if (srow[m] >= 0) {
 #pragma unroll
-                for (int k = 0; k < BZ; ++k) emax = max(emax, top(v[m][k]));
+                for (int k = 0; k < BZ; ++k) sample(v[m][k]);
             }
-        emax = __reduce_max_sync(0xffffffffu, emax);
-        if ((tid & 31) == 0) wmax[tid >> 5] = emax;
-        __syncthreads();
-#pragma unroll
-        for (int w = 0; w < FX_THREADS / 32; ++w) emax = max(emax, wmax[w]);
-        const int E = max(emax + 1, 128);   // 128: zeros stay zeros, what else is that small takes FP64
-        bool bad = E > 2046;
+        // 2^(E - 1022) is 4/3 of the sample's largest or more; 128: what is that small takes FP64
+        int E = max((block_max(first, wtop[0]) + 0x80000) >> 20, 128);
         auto fix = [&](double2 q) {
             return make_longlong2(fix_from_bits(__double2hiint(q.x), (unsigned)__double2loint(q.x), E),
                                   fix_from_bits(__double2hiint(q.y), (unsigned)__double2loint(q.y), E));
         };
-        auto stage = [&](int m, double2 (&v)[BZ]) {
-            int lo = 0;   // largest exponent of the stretch: this slot's planes in four neighbouring lanes
+        int top = 0, bits = 0;
+        auto seen = [&](double2 q) {
+            top = max(top, max(expo(q.x), expo(q.y)));
+            bits |= __double2hiint(q.x) | __double2loint(q.x);
+            bits |= __double2hiint(q.y) | __double2loint(q.y);
+        };
+#pragma unroll
+        for (int j = 0; j < 2 * N; ++j) seen(zr[j]);
+#pragma unroll
+        for (int m = 0; m < SPT; ++m) {
+            double2 (&q)[BZ] = v[ALL ? m : 0];
+            if (!ALL && m > 0) load_slot(m, q);
             if (srow[m] >= 0) {
                 long long* dst = fix_smem + srow[m] * RW + scol[m];
 #pragma unroll
                 for (int k = 0; k < BZ; ++k) {
-                    lo = max(lo, top(v[k]));
-                    *reinterpret_cast<longlong2*>(dst + k * CPL) = fix(v[k]);
+                    seen(q[k]);
+                    *reinterpret_cast<longlong2*>(dst + k * CPL) = fix(q[k]);
                 }
             }
-            bad |= lo > E;
-            lo = max(lo, __shfl_xor_sync(0xffffffffu, lo, 1));
-            lo = max(lo, __shfl_xor_sync(0xffffffffu, lo, 2));
-            bad |= lo != 0 && lo < E - 7;
-        };
+        }
+        // the block's largest exponent, with 2^16 where a bit is set anywhere
+        const int all = block_max(top | (bits != 0 ? 1 << 16 : 0), wtop[1]);
+        if ((all & 0xffff) > E && (all & 0xffff) <= 2046) {
+            // a staged value above the sample's range: once more, with its exponent (a short loop: cold code)
+            E = all & 0xffff;
+#pragma unroll 1
+            for (int m = 0; m < SPT; ++m) {
+                int row, c;
+                slot(m, row, c);
+                if (row < 0) continue;
+#pragma unroll 1
+                for (int k = 0; k < BZ; ++k) {
+                    const int o = zoff[N + k] + yoff[row];
+                    *reinterpret_cast<longlong2*>(fix_smem + k * CPL + row * RW + c) =
+                        fix(fix_load(op, (unsigned)(o + xoff[c]), (unsigned)(o + xoff[c + 1]), false));
+                }
+            }
+            __syncthreads();
+        }
 #pragma unroll
         for (int j = 0; j < 2 * N; ++j) col[j < N ? j : j + BZ] = fix(zr[j]);
-#pragma unroll
-        for (int m = 0; m < SPT; ++m) {
-            if (!ALL && m > 0) load_slot(m, v[0]);
-            stage(m, v[ALL ? m : 0]);
-        }
-        const bool fp64 = __syncthreads_or(bad) != 0;
         const int y = y0 + ty, xe = x0 + 2 * tx;         // first double of this thread's unit
         const bool act0 = y < d.n2 && xe < RF, act1 = act0 && xe + 1 < RF;
         const long long i0 = (long long)y * d.n1 + (CPLX ? xe / 2 : xe);
@@ -332,15 +418,10 @@ __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& 
             if constexpr (HasPre<Op>::value) return op.pre((long long)(z0 + k) * d.n1 * d.n2 + i0, act0, act1);
             else return 0;
         };
-        auto cur = fetch(0), next = cur;
-        auto ahead = [&](int k) {
-            if (k < nz) next = fetch(k);
-        };
-        auto put = [&](int k, double l0, double l1) {
+        auto store = [&](int k, auto&& p, double l0, double l1) {
             const long long i = (long long)(z0 + k) * d.n1 * d.n2 + i0;
             if constexpr (HasPre<Op>::value) {
-                op.store_pre(i, cur, l0, l1, act0, act1);
-                cur = next;
+                op.store_pre(i, p, l0, l1, act0, act1);
             } else if constexpr (CPLX) {
                 if (act0) op.store(i, op.load(i), make_double2(l0, l1));
             } else {
@@ -348,41 +429,124 @@ __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& 
                 if (act1) op.store(i + 1, op.load(i + 1), l1);
             }
         };
-        if (!fp64) {
+        // FP64 arithmetic straight from global memory (code that is cold when it runs, and one block holds up a
+        // sweep of a small grid: short loops, and the op's own code only where points are many)
+        constexpr int XS = CPLX ? 2 : 1;
+        auto at = [&](int j, int r, int c) {
+            const int o = zoff[j] + yoff[r];
+            return fix_load(op, (unsigned)(o + xoff[c]), (unsigned)(o + xoff[c + 1]), false);
+        };
+        const int lane = tid & 31, warp = tid >> 5;
+        unsigned coarse = act0 ? (1u << nz) - 1u : 0u;   // planes left to FP64 arithmetic
+        if (E <= 2046 && (all & 0xffff) <= E) {
             const long long* own_s = fix_smem + (ty + N) * RW + HX + 2 * tx;
 #pragma unroll
             for (int k = 0; k < BZ; ++k) col[N + k] = *reinterpret_cast<const longlong2*>(own_s + k * CPL);
-            const double unit = __hiloint2double((E - 1082 + 1023) << 20, 0);
-            fix_planes<N, CPLX, ISO, BZ>(col, own_s, nz, fs.s[0] * unit, fs.s[1] * unit, fs.s[2] * unit, ahead, put);
-        } else {
-            // FP64 arithmetic, straight from global memory
-            constexpr int XS = CPLX ? 2 : 1;
-            const int cx = HX + 2 * tx, ry = N + ty;
-            for (int k = 0; k < nz; ++k) {
-                ahead(k + 1);
-                auto at = [&](int j, int r, int c) {
-                    const int o = zoff[j] + yoff[r];
-                    return fix_load(op, (unsigned)(o + xoff[c]), (unsigned)(o + xoff[c + 1]), false);
-                };
-                double2 acc = at(N + k, ry, cx);
-                acc = make_double2(W.centre * acc.x, W.centre * acc.y);
-                auto tap = [&](double w, double2 a, double2 b) {
-                    acc.x = fma(w, a.x + b.x, acc.x);
-                    acc.y = fma(w, a.y + b.y, acc.y);
-                };
-                for (int p = 1; p <= N; ++p) {
-                    tap(W.w[2][p], at(N + k + p, ry, cx), at(N + k - p, ry, cx));
-                    tap(W.w[0][p], at(N + k, ry, cx + p * XS), at(N + k, ry, cx - p * XS));
-                    tap(W.w[1][p], at(N + k, ry + p, cx), at(N + k, ry - p, cx));
-                }
-                put(k, acc.x, acc.y);
+            const unsigned least = all ? FIX_FINE : 0u;
+            // planes in which the unit's first and second value are below the limit; a complex value counts once
+            unsigned s0 = 0, s1 = 0;
+#pragma unroll
+            for (int k = 0; k < BZ; ++k) {
+                const unsigned m0 = fix_mag(col[N + k].x), m1 = fix_mag(col[N + k].y);
+                s0 |= (CPLX ? m0 | m1 : m0) < least ? 1u << k : 0u;
+                s1 |= !CPLX && m1 < least ? 1u << k : 0u;
             }
+            if constexpr (CPLX) s1 = s0;
+            int mine = 0, total = 0;
+            // what the neighbours that this lane and those beside it hold leave to a closer look: both of the
+            // unit (complex: the next lane's), next in z, one of the two in y
+            const unsigned sy = __shfl_xor_sync(0xffffffffu, s0 | s1 << 16, FX_UX);
+            auto column = [](unsigned s) { return (s << 1 | 1u) & (s >> 1 | 1u << (BZ - 1)); };
+            unsigned small = s0 & s1 & ((column(s0) & sy) | (column(s1) & sy >> 16));
+            if constexpr (CPLX) small &= __shfl_xor_sync(0xffffffffu, s0, 1);
+            // a warp in which eight units pass none of this in any plane leaves all its points
+            bool leave = __popc(__ballot_sync(0xffffffffu, small == (1u << BZ) - 1u)) >= 8;
+            if (!leave && __any_sync(0xffffffffu, small != 0)) {
+                const unsigned c = fix_coarse<N, CPLX, BZ>(own_s, small, least) & coarse;
+                const int count = __popc(c);
+                total = __reduce_add_sync(0xffffffffu, count);
+                leave = total > FX_ITEMS;
+                if (!leave && total > 0) {   // eight lanes to a unit, four units at a time
+                    mine = count;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(0xffffffffu, mine, o);
+                        if (lane >= o) mine += v;
+                    }
+                    mine -= count;
+                    int q = mine;
+                    for (unsigned r = c; r; r &= r - 1u) items[warp][q++] = (unsigned char)((__ffs((int)r) - 1) * 32 + lane);
+                    __syncwarp();
+#pragma unroll 1
+                    for (int q0 = 0; q0 < total; q0 += 4) {
+                        const int qi = min(q0 + (lane >> 3), total - 1), e = items[warp][qi], k = N + (e >> 5);
+                        const int cx = HX + 2 * (e & (FX_UX - 1)), ry = N + (warp * 32 + (e & 31)) / FX_UX;
+                        double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+                        for (int t0 = 0; t0 <= 6 * N; t0 += 8) {   // 2N taps of each axis, the centre
+                            const int t = t0 + (lane & 7), a = t / (2 * N), h = t - a * 2 * N, p = h / 2 + 1, o = h & 1 ? -p : p;
+                            if (t > 6 * N) continue;
+                            const double2 v = at(k + (a == 2 ? o : 0), ry + (a == 1 ? o : 0), cx + (a == 0 ? o * XS : 0));
+                            const double w = a == 3 ? W.centre : W.w[a][p];
+                            acc.x = fma(w, v.x, acc.x);
+                            acc.y = fma(w, v.y, acc.y);
+                        }
+#pragma unroll
+                        for (int o = 4; o > 0; o >>= 1) {
+                            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+                            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+                        }
+                        if ((lane & 7) == 0) taken[warp][qi] = acc;
+                    }
+                    __syncwarp();
+                    small = c;
+                }
+            }
+            if (total == 0) small = 0;   // now the planes whose values stand in `taken`
+            if (!leave) {
+                coarse = 0;
+                const double unit = __hiloint2double((E - 1082 + 1023) << 20, 0);
+                auto cur = fetch(0), next = cur;
+                fix_planes<N, CPLX, ISO, BZ>(
+                    col, own_s, nz, fs.s[0] * unit, fs.s[1] * unit, fs.s[2] * unit,
+                    [&](int k) {
+                        if (k < nz) next = fetch(k);
+                    },
+                    [&](int k, double l0, double l1) {
+                        if ((small >> k) & 1u) {
+                            const double2 v = taken[warp][mine++];
+                            l0 = v.x;
+                            l1 = v.y;
+                        }
+                        store(k, cur, l0, l1);
+                        cur = next;
+                    });
+                __syncwarp();   // before the next brick's values
+            }
+        }
+        const int cx = HX + 2 * tx, ry = N + ty;
+#pragma unroll 1
+        for (; coarse; coarse &= coarse - 1u) {
+            const int k = __ffs((int)coarse) - 1;
+            double2 acc = at(N + k, ry, cx);
+            acc = make_double2(W.centre * acc.x, W.centre * acc.y);
+            auto tap = [&](double w, double2 a, double2 b) {
+                acc.x = fma(w, a.x + b.x, acc.x);
+                acc.y = fma(w, a.y + b.y, acc.y);
+            };
+#pragma unroll 1
+            for (int p = 1; p <= N; ++p) {
+                tap(W.w[2][p], at(N + k + p, ry, cx), at(N + k - p, ry, cx));
+                tap(W.w[0][p], at(N + k, ry, cx + p * XS), at(N + k, ry, cx - p * XS));
+                tap(W.w[1][p], at(N + k, ry + p, cx), at(N + k, ry - p, cx));
+            }
+            store(k, fetch(k), acc.x, acc.y);
         }
     }
 }
 
 template <int N, bool CPLX, bool ISO, int BZ, class Op>
-__global__ void __launch_bounds__(FX_THREADS, 3)
+__global__ void __launch_bounds__(FX_THREADS, N == 1 ? 4 : 3)
 fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int bricks, Op op) {
     pdl_enter();
     if (!op.begin()) return;
