@@ -29,6 +29,7 @@ struct Fft {
     bool ok = false;
     FftPlan plan[3], z_back;   // z_back: the radices of plan[2] reversed
     const float* sym[3];     // l_a(k), k < n_a
+    double lmax = 0.0;       // the largest eigenvalue of -L_h
 };
 
 void fft_destroy(Fft* f) { delete f; }
@@ -49,6 +50,7 @@ static Fft& fft_tables(of_grid* g) {
     const int n[3] = {g->d.n1, g->d.n2, g->d.n3};
     std::vector<float> host;
     size_t off[6];
+    f.lmax = 0.0;
     for (int a = 0; a < 3; ++a) {
         OF_REQUIRE(fft_make_plan(n[a], f.plan[a]), OF_EINVAL, "direct solve: no transform of %d points", n[a]);
         off[a] = host.size();
@@ -58,6 +60,7 @@ static Fft& fft_tables(of_grid* g) {
             host.push_back((float)std::sin(t));
         }
         off[3 + a] = host.size();
+        double top = 0.0;
         for (int k = 0; k < n[a]; ++k) {
             double l = 0.0;
             for (int p = 1; p <= g->N; ++p) {
@@ -65,7 +68,9 @@ static Fft& fft_tables(of_grid* g) {
                 l += 4.0 * g->w64.w[a][p] * s * s;
             }
             host.push_back((float)l);
+            top = std::max(top, l);
         }
+        f.lmax += top;
         if (host.size() & 1) host.push_back(0.f);   // the twiddles of the next axis are float2
     }
     float* dev = (float*)ws(g, WS_FFTT, sizeof(float) * host.size());
@@ -360,7 +365,11 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_y(FftPlan P, int lg, FftCol
 }
 
 // symbol of the inverse: kind 0: 1 / l (0 for the constant mode); 1: 1 / (l + s1);
-// 2: (l + s0) / (l + s1)^2; 3: 1 / (a l + Q).  norm = 1 / (n1 n2 n3).
+// 2: (l + s0) / (l + s1)^2; 3: 1 / (a l + Q), 0 where |a l + Q|^2 <= s0.  norm = 1 / (n1 n2 n3).
+// s0 of kind 3 is (2^-20 S)^2, S = |a| l_max + |Q|: a symbol below that is known in FP32, to a few 2^-24
+// of S, with less than two digits, and the FP32 rounding of a solution that holds S / |a l + Q| times the
+// residual changes the residual by more than 1/16: such a mode, which could make a pass raise the
+// residual by orders, is left to the Krylov solvers.
 struct FftFilter {
     int kind;
     float a, qr, qi, s0, s1, norm;
@@ -370,7 +379,7 @@ struct FftFilter {
         if (kind == 3) {
             const float dr = fmaf(a, l, qr), di = qi;
             const float den = fmaf(dr, dr, di * di);
-            const float m = den > 1e-30f ? norm / den : 0.f;   // a singular mode is left alone
+            const float m = den > s0 ? norm / den : 0.f;
             const float gr = dr * m, gi = -di * m;
             return make_float2(gr * v.y + gi * v.x, gr * v.x - gi * v.y);
         }
@@ -651,6 +660,8 @@ void fft_correct_shifted(of_grid* g, const double2* r, double2* x, double a, dou
     f.a = (float)a;
     f.qr = (float)Q.x;
     f.qi = (float)Q.y;
+    const double least = std::ldexp(std::fabs(a) * fft_tables(g).lmax + std::hypot(Q.x, Q.y), -20);
+    f.s0 = (float)(least * least);
     fft_apply<true>(g, LdCplx64{r, st, 0}, StAccumCplx64{x, st, 0}, f, &st->done);
 }
 

@@ -556,7 +556,8 @@ static of_status solve_formed(of_grid* g, T64* x, double a, double2 Q, const Kry
         h.rr = 0.0;
     }
     // further direct passes while each gains a factor of ten; a system whose symbol nearly vanishes
-    // somewhere (a l + Q close to 0) gains less and is left to the Krylov solvers below
+    // somewhere (a l + Q close to 0) keeps those modes (FftFilter), gains less and is left to the Krylov
+    // solvers below
     for (bool gains = direct; gains && bb > 0.0 && h.rr > h.tol2 && total_iters < o.max_iter;) {
         const double before = h.rr;
         direct_passes(1);
