@@ -274,7 +274,9 @@ __global__ void __launch_bounds__(256) k_self_box(const AtomBox* boxes, double h
 }
 
 // Block (ion, plane): the same sums over the plane's points outside the ball, in FP32, to
-// part[(J max_planes + pl) 4 ..] (added in FP64 across warps and planes).
+// part[(J max_planes + pl) 4 ..] (added in FP64 across warps and planes).  Which points those are is
+// decided as k_pseudocharge_gather decides it, in FP64 wherever FP32 (r2 to 1e-6 of itself) may not tell:
+// one point of the surface counts up to 1e-14 of the sum, and there may be dozens.
 __global__ void __launch_bounds__(256) k_self_corners(const AtomBox* boxes, double h1, double h2, double h3, Gauss q,
                                                       AxisTables T, double* part, int max_planes) {
     const int J = blockIdx.x, pl = blockIdx.y;
@@ -283,21 +285,30 @@ __global__ void __launch_bounds__(256) k_self_corners(const AtomBox* boxes, doub
     if (pl < B.len[2]) {
         const Axis* tx = T.t + (long long)J * 3 * T.max_len;
         const Axis* ty = tx + T.max_len;
-        const float z2 = (float)ty[T.max_len + pl].d2, rc2 = (float)(q.rc * q.rc);
+        const double z2d = ty[T.max_len + pl].d2;
+        const float z2 = (float)z2d, rc2 = (float)(q.rc * q.rc), near = rc2 * (1.f - 5e-6f), far = rc2 * (1.f + 5e-6f);
         const float c2 = (float)(-q.inv2s2 * 1.4426950408889634);   // exp as 2^x
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         const float x0 = (float)(B.lo[0] * h1 - B.R[0]), y0 = (float)(B.lo[1] * h2 - B.R[1]);
         for (int ii = lane; ii < B.len[0]; ii += 32) {
             const float dx = x0 + ii * (float)h1, xz2 = (float)tx[ii].d2 + z2;
+            auto add = [&](float dy, float r2) {
+                const float v = exp2f(r2 * c2) * rsqrtf(r2);
+                acc[0] += v;
+                acc[1] = fmaf(v, dx, acc[1]);
+                acc[2] = fmaf(v, dy, acc[2]);
+            };
+            bool close = false;   // a point of the column whose side FP32 may not tell
             for (int jj = warp; jj < B.len[1]; jj += blockDim.x >> 5) {
                 const float dy = y0 + jj * (float)h2, r2 = fmaf(dy, dy, xz2);
-                if (r2 > rc2) {
-                    const float v = exp2f(r2 * c2) * rsqrtf(r2);
-                    acc[0] += v;
-                    acc[1] = fmaf(v, dx, acc[1]);
-                    acc[2] = fmaf(v, dy, acc[2]);
-                }
+                close |= fabsf(r2 - rc2) <= 1e-5f * rc2;
+                if (r2 > far) add(dy, r2);
             }
+            if (close)
+                for (int jj = warp; jj < B.len[1]; jj += blockDim.x >> 5) {
+                    const float dy = y0 + jj * (float)h2, r2 = fmaf(dy, dy, xz2);
+                    if (r2 <= far && r2 > near && !((tx[ii].d2 + ty[jj].d2) + z2d <= q.rc * q.rc)) add(dy, r2);
+                }
         }
         acc[3] = acc[0] * (float)((B.lo[2] + pl) * h3 - B.R[2]);
     }
