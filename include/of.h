@@ -202,6 +202,11 @@ void of_default_scf_opts(of_scf_opts* o);
 of_status of_grid_create(int n1, int n2, int n3, double L1, double L2, double L3,
                          int fd_half_order, void* stream, of_grid** out);
 of_status of_grid_destroy(of_grid* g);
+/* Failure detection: the FP64 CG of small grids runs all its iterations in one cooperative launch,
+ * whose blocks give up waiting at a grid barrier after `seconds` (default 2; 0 <= seconds <= 60);
+ * the launch then ends and its call returns OF_ETIMEOUT, the grid stays usable.  0 makes every
+ * block give up at its first barrier, which exercises that path without a fault. */
+of_status of_grid_set_wait_limit(of_grid* g, double seconds);
 
 /* y = L_h x: the order-2N central-difference Laplacian of Eq. FD:Laplacian, indices wrapped
  * periodically (Sec. 4).  dtype OF_F64: x, y are double*; OF_F32: float*.  x != y. */

@@ -101,6 +101,7 @@ _SIGNATURES = {
     "of_default_scf_opts": (None, [C.POINTER(of_scf_opts)]),
     "of_grid_create": (_I, [_I, _I, _I, _D, _D, _D, _I, _P, C.POINTER(_P)]),
     "of_grid_destroy": (_I, [_P]),
+    "of_grid_set_wait_limit": (_I, [_P, _D]),
     "of_laplacian_apply": (_I, [_P, _I, _P, _P]),
     "of_poisson_solve": (_I, [_P, _P, _P, C.POINTER(of_solve_opts), C.POINTER(of_solve_info)]),
     "of_kernel_solve": (_I, [_P, _P, _I, C.POINTER(_D), C.POINTER(_D), _D, _P,
@@ -227,6 +228,10 @@ def of_grid_create(n, L, fd_half_order=6, stream=None):
 
 def of_grid_destroy(h):
     return _check(load().of_grid_destroy(h), "of_grid_destroy")
+
+
+def of_grid_set_wait_limit(h, seconds):
+    return _check(load().of_grid_set_wait_limit(h, float(seconds)), "of_grid_set_wait_limit")
 
 
 def of_laplacian_apply(h, dtype, x, y):

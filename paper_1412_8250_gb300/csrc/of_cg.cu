@@ -44,17 +44,16 @@ struct OpCg {
     }
 };
 
-constexpr unsigned long long CG_WAIT_NS = 2000000000ull;
-
 __device__ __forceinline__ unsigned long long cg_now() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
 
-// All blocks' sum of v (every thread's share), the same bits in every block; false: gave up.
-// `target`: arrivals that end this barrier.
-__device__ __forceinline__ bool cg_total(double v, double* partials, unsigned* bar, unsigned target, double& total) {
+// All blocks' sum of v (every thread's share), the same bits in every block; false: gave up (at once,
+// without polling, for wait_ns = 0).  `target`: arrivals that end this barrier.
+__device__ __forceinline__ bool cg_total(double v, double* partials, unsigned* bar, unsigned target,
+                                         unsigned long long wait_ns, double& total) {
     __shared__ double sums[1];
     __shared__ int ok;
     const int tid = threadIdx.x + FX_UX * threadIdx.y, nb = gridDim.x;
@@ -69,12 +68,12 @@ __device__ __forceinline__ bool cg_total(double v, double* partials, unsigned* b
         volatile unsigned* quit = bar + 1;
         int got = 0;
         unsigned long long t0 = 0;
-        for (int k = 0; k < (1 << 26); ++k) {
+        for (int k = 0; wait_ns != 0 && k < (1 << 26); ++k) {
             if (*count >= target) { got = 1; break; }
             if ((k & 255) == 255) {
                 if (*quit) break;
                 if (t0 == 0) t0 = cg_now();
-                else if (cg_now() - t0 > CG_WAIT_NS) break;
+                else if (cg_now() - t0 > wait_ns) break;
             }
         }
         if (!got) *quit = 1u;
@@ -98,7 +97,8 @@ __device__ __forceinline__ bool cg_total(double v, double* partials, unsigned* b
 template <int N, bool ISO, int BZ>
 __global__ void __launch_bounds__(FX_THREADS, BZ == 2 ? 3 : 2)
 cg_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int bricks, double* __restrict__ x, double* r,
-          double* pa, double* pb, double* Ap, double a, double q, KState* st, double* partials, unsigned* bar) {
+          double* pa, double* pb, double* Ap, double a, double q, KState* st, double* partials, unsigned* bar,
+          unsigned long long wait_ns) {
     if (st->done != 0.0) return;
     const double tol2 = st->tol2, maxit = st->maxit;
     double beta = st->beta_re, rho = st->rho_re, rr = st->rr, iters = st->iters;
@@ -111,7 +111,7 @@ cg_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int 
         op.acc = 0.0;
         fix_sweep<N, false, ISO, BZ>(d, W, fs, vec, bx, by, bricks, op);
         target += gridDim.x;
-        ok = cg_total(op.acc, partials, bar, target, pAp);
+        ok = cg_total(op.acc, partials, bar, target, wait_ns, pAp);
         if (!ok) break;
         if (!(pAp > 0.0)) {
             breakdown = 1.0;
@@ -155,7 +155,7 @@ cg_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int 
             }
         }
         target += gridDim.x;
-        ok = cg_total(acc, partials + OF_MAX_RED_BLOCKS, bar, target, rr);
+        ok = cg_total(acc, partials + OF_MAX_RED_BLOCKS, bar, target, wait_ns, rr);
         if (!ok) break;
         iters += 1.0;
         if (rr <= tol2 || iters >= maxit) {
@@ -215,7 +215,8 @@ static bool cg_launch(const CgLaunch& c) {
     OF_CUDA(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), g->stream));
     Weights<double> W = g->w64;
     FixScale fs = c.fs;
-    void* args[] = {&d, &W, &fs, &vec, &bx, &by, &bricks, &x, &r, &pa, &pb, &Ap, &a, &q, &st, &partials, &bar};
+    unsigned long long wait_ns = g->wait_ns;
+    void* args[] = {&d, &W, &fs, &vec, &bx, &by, &bricks, &x, &r, &pa, &pb, &Ap, &a, &q, &st, &partials, &bar, &wait_ns};
     ProfScope ps(g, PC_CG_F64, 0.0);
     OF_CUDA(cudaLaunchCooperativeKernel((const void*)cg_kernel<N, ISO, BZ>, dim3(bricks), dim3(FX_UX, FX_BY), args, smem,
                                         g->stream));

@@ -212,6 +212,15 @@ of_status of_grid_destroy(of_grid* g) {
     return OF_OK;
 }
 
+of_status of_grid_set_wait_limit(of_grid* g, double seconds) {
+    if (!g || !(seconds >= 0.0) || seconds > 60.0) {
+        set_error("of_grid_set_wait_limit: need a handle and 0 <= seconds <= 60");
+        return OF_EINVAL;
+    }
+    for (of_grid* h = g; h; h = h->twin) h->wait_ns = (unsigned long long)(seconds * 1e9);
+    return OF_OK;
+}
+
 of_status of_laplacian_apply(of_grid* g, of_dtype dtype, const void* x, void* y) {
     if (!g || !x || !y) { set_error("of_laplacian_apply: null argument"); return OF_EINVAL; }
     if (x == y) { set_error("of_laplacian_apply: x and y must not alias"); return OF_EINVAL; }

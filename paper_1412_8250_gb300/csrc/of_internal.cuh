@@ -207,6 +207,8 @@ struct of_grid {
     void* worker = nullptr;
     void (*worker_destroy)(void*) = nullptr;
     void* graphs = nullptr;              // cached CUDA graphs (of_krylov.cu)
+    // limit of the cooperative kernels' waits at grid barriers (of_grid_set_wait_limit)
+    unsigned long long wait_ns = 2000000000ull;
     // the Krylov loops launch every iteration directly instead of capturing and caching CUDA
     // graphs (which create a capture stream and executable graphs)
     bool no_graphs = false;

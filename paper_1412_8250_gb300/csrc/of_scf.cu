@@ -710,6 +710,7 @@ static of_grid* twin_of(of_grid* g) {
         const of_status s = of_grid_create(g->d.n1, g->d.n2, g->d.n3, g->L[0], g->L[1], g->L[2], g->N,
                                            g->twin_stream, &t);
         if (s != OF_OK) throw Error{s};
+        t->wait_ns = g->wait_ns;
         g->twin = t;
         if (g->prof && g->prof->every > 0) of_profile_enable(t, g->prof->every);
     }
