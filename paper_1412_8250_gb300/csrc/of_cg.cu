@@ -69,7 +69,7 @@ __device__ __forceinline__ bool cg_total(double v, double* partials, unsigned* b
         int got = 0;
         unsigned long long t0 = 0;
         for (int k = 0; wait_ns != 0 && k < (1 << 26); ++k) {
-            if (*count >= target) { got = 1; break; }
+            if ((int)(*count - target) >= 0) { got = 1; break; }   // (both wrap: 2^32 / 2 blocks iterations)
             if ((k & 255) == 255) {
                 if (*quit) break;
                 if (t0 == 0) t0 = cg_now();
