@@ -218,8 +218,15 @@ static bool cg_launch(const CgLaunch& c) {
     unsigned long long wait_ns = g->wait_ns;
     void* args[] = {&d, &W, &fs, &vec, &bx, &by, &bricks, &x, &r, &pa, &pb, &Ap, &a, &q, &st, &partials, &bar, &wait_ns};
     ProfScope ps(g, PC_CG_F64, 0.0);
-    OF_CUDA(cudaLaunchCooperativeKernel((const void*)cg_kernel<N, ISO, BZ>, dim3(bricks), dim3(FX_UX, FX_BY), args, smem,
-                                        g->stream));
+    const cudaError_t err = cudaLaunchCooperativeKernel((const void*)cg_kernel<N, ISO, BZ>, dim3(bricks),
+                                                        dim3(FX_UX, FX_BY), args, smem, g->stream);
+    // a context that is given part of the SMs, or none of whose launches may be cooperative, refuses: the
+    // solve then runs as separate launches
+    if (err == cudaErrorCooperativeLaunchTooLarge || err == cudaErrorNotSupported) {
+        cudaGetLastError();
+        return false;
+    }
+    OF_CUDA(err);
     __atomic_add_fetch(&g_launch_count, 1ull, __ATOMIC_RELAXED);
     ps.end_timing();
     fetch_scalars(g, c.st_off, KSTATE_DOUBLES, (double*)c.h);
