@@ -51,13 +51,9 @@ WORKLOAD_DETAIL = {
 }
 GOLDEN_AL108 = os.path.join(ROOT, "tests", "golden", "al108_wt.json")
 # DRAM bytes (read + write) of one order-12 sweep of a 320^3 grid, FP32 and FP64, from the ncu
-# capture summarised in profiles/sweeps_and_transforms.md (163.0 + 92.7 and 453.3 + 235.5 MB)
+# capture summarised in profiles/sweeps_and_transforms.md (163.0 + 92.7 and 484.3 + 238.2 MB)
 STENCIL320_DRAM_BYTES = 255.7e6
-STENCIL320_F64_DRAM_BYTES = 688.8e6
-# DRAM bytes that one V-cycle plus one COCG iteration of the 96^3 complex FP32 pass moves,
-# summed over its kernels launched one by one from a cold L2 (ncu; the kernels' table is in
-# profiles/mg_cocg_pass_kernels_96.md)
-COCG96_DRAM_BYTES_PER_ITERATION = 167e6
+STENCIL320_F64_DRAM_BYTES = 722.5e6
 GOLDEN_SMALL = os.path.join(ROOT, "tests", "golden", "ground_states.json")
 
 
@@ -305,7 +301,7 @@ def batched_compare(torch, B, W, reps=2):
     the Poisson problem of each cell's initial density (uniform electrons plus its Gaussian
     nuclear charge), solved to relative residual 1e-10 by (a) one batched call of grouped
     launches (plain FP32 CG + FP64 refinement), (b) one batched call in the default mixed form
-    (per-cell direct corrections over concurrent streams; reported under its earlier key), (c) the
+    (per-cell direct corrections over concurrent streams), (c) the
     single-grid solver cell by cell with the same plain CG, (d) cell by cell in the default mixed form."""
     cells = W.batched_cells()
     stream = torch.cuda.current_stream()
@@ -336,20 +332,20 @@ def batched_compare(torch, B, W, reps=2):
             p.zero_()
             B.of_poisson_solve(g, r, p, opts)
 
-    def run_batched_mg():
+    def run_batched_direct():
         for p in phis:
             p.zero_()
         return B.of_poisson_solve_batched(grids, rhos, phis, om)
 
     out = {}
     run_batched()   # tunes the blocking, captures the graph
-    run_batched_mg()
+    run_batched_direct()
     run_seq(o)
     run_seq(om)
     for name, fn in [("batched_plain_cg_s", run_batched),
-                     ("batched_multigrid_concurrent_s", run_batched_mg),
+                     ("batched_direct_concurrent_s", run_batched_direct),
                      ("sequential_plain_cg_s", lambda: run_seq(o)),
-                     ("sequential_multigrid_pcg_s", lambda: run_seq(om))]:
+                     ("sequential_direct_s", lambda: run_seq(om))]:
         ts = []
         for _ in range(reps):
             torch.cuda.synchronize()
@@ -381,7 +377,7 @@ def learned_compare(torch, B, W, steps=400, theta=0.3):
     4-atom 32^3 and the 108-atom 96^3 cells (64 residuals each; four Adam runs per cell, batch
     4), then used in the FP32 flexible CG of the Poisson solve of the 864-atom 6x6x6 cell,
     192^3 grid, same spacing, to true relative residual 1e-10; against the same solve with
-    plain (Jacobi) FP32 CG, plain FP64 CG and the default mixed form (key multigrid_pcg_mixed)."""
+    plain (Jacobi) FP32 CG, plain FP64 CG and the default mixed form (key direct_mixed)."""
     import numpy as np
     stream = torch.cuda.current_stream()
     torch.cuda.synchronize()
@@ -421,7 +417,7 @@ def learned_compare(torch, B, W, steps=400, theta=0.3):
     for name, o in (("jacobi_cg_mixed", opts(B.OF_F32, 1, False)),
                     ("learned_fcg_mixed", opts(B.OF_F32, 1, True)),
                     ("plain_cg_f64", opts(B.OF_F64, 1, False)),
-                    ("multigrid_pcg_mixed", opts(B.OF_F32, 0, False))):
+                    ("direct_mixed", opts(B.OF_F32, 0, False))):
         phi.zero_()
         B.of_poisson_solve(g, rho, phi, o)     # workspace, graphs
         phi.zero_()
@@ -464,7 +460,7 @@ def learned_shifted_compare(torch, B, W, g864, cell864, steps, theta):
     the FP32 flexible GMRES(8) of the same shifted system on the 864-atom 192^3 grid (a
     right-hand side not trained on) to true relative residual 1e-10; against the same solver
     with every network step refused (plain inner CG), plain FP32 COCG, plain FP64 COCG and
-    the default mixed form (key multigrid_pcocg_mixed).  Iterations count the inner steps too."""
+    the default mixed form (key direct_mixed).  Iterations count the inner steps too."""
     import numpy as np
     from paper_1412_8250_gb300 import functionals as Fn
     fn = Fn.wt()
@@ -514,7 +510,7 @@ def learned_shifted_compare(torch, B, W, g864, cell864, steps, theta):
                     ("learned_fgmres_mixed", opts(B.OF_F32, 1, True)),
                     ("fgmres_plain_inner_cg_mixed", opts(B.OF_F32, 1, True, 2.0)),
                     ("plain_cocg_f64", opts(B.OF_F64, 1, False)),
-                    ("multigrid_pcocg_mixed", opts(B.OF_F32, 0, False))):
+                    ("direct_mixed", opts(B.OF_F32, 0, False))):
         Wc.zero_()
         B.of_kernel_solve(g864, f, [Pk], [Qk], kf2_864, Wc, o)     # workspace, graphs
         Wc.zero_()
@@ -1137,8 +1133,8 @@ def config5(args):
                                    "a=7.6 bohr, +-0.1 bohr displacements, seed 5), 320^3, "
                                    "12th-order FD, WT-type kernel (sigma=1.2, r_c=10); ground "
                                    "state + forces"},
-            "mixed_multigrid_s": t_mixed,
-            "mixed_multigrid_plain_nlcg_s": t_plain_nlcg,
+            "mixed_s": t_mixed,
+            "mixed_plain_nlcg_s": t_plain_nlcg,
             "plain_nlcg_counts": {"outer_iterations": res_p.outer_iterations,
                                   "nlcg_steps": res_p.nlcg_iterations,
                                   "energy_difference_ha_per_atom":
@@ -1180,7 +1176,7 @@ def batched_ground_states(torch, B, Fn, W, ncells):
     benchmark's options): one batched call (each cell's solver on its own stream of a pool,
     driven by its own host thread) against the same ground states one after another.  An
     untimed batched call cut short (one outer iteration of three NLCG steps) first creates
-    every cell's workspace, multigrid hierarchy and graphs."""
+    every cell's workspace, transform plans and graphs."""
     cells = W.batched_cells()[:ncells]
     stream = torch.cuda.current_stream()
     grids = [B.of_grid_create(c.n, c.L, 6, stream) for c in cells]
@@ -1455,28 +1451,6 @@ def main():
                     "bytes_model": "every field a fused sweep reads or writes, once per point of "
                                    "its level (CG iteration 10 words, Chebyshev step 6, residual "
                                    "3, transfers 1-2 per fine point), halos not counted"}
-        if dom["kernel"] in ("mg_pcg_pass_graph", "mg_cocg_pass_graph") and prof:
-            # the same time against the Krylov iterations' own bytes only (10 words per point
-            # per iteration: FP32 for CG, complex FP32 for COCG), the V-cycle's sweeps left out
-            cocg = dom["kernel"] == "mg_cocg_pass_graph"
-            passes = sum(p["launches"] for p in prof if p["kernel"] == dom["kernel"])
-            its = (res.kernel_iterations if cocg else res.poisson_iterations) * args.steps / max(1, passes)
-            cg_bytes = its * (80.0 if cocg else 40.0) * cell.n_points
-            roofline["cg_iterations_per_launch"] = its
-            roofline["frac_cg_bytes_only"] = cg_bytes / (dom["mean_ms"] * 1e-3) / 1e9 / peak
-            if cocg and cell.n_points == 96 ** 3:
-                roofline["traffic"] = its * COCG96_DRAM_BYTES_PER_ITERATION
-                roofline["traffic_note"] = (
-                    "ncu dram__bytes_read.sum + dram__bytes_write.sum of the pass's kernels "
-                    "launched one by one from a cold L2 (OF_NO_GRAPHS=1, 28 iterations of the "
-                    "first kernel map: 167 MB per V-cycle + COCG iteration), scaled by the "
-                    "iterations per pass; inside the graphs the fields stay in L2")
-            roofline["note"] = ("latency-bound: at 96^3 every field stays in L2 and one "
-                                "preconditioned iteration is a chain of ~17 dependent launches"
-                                + ("; up to four shifted systems are solved at once (a chain of "
-                                   "twin handles), so a pass's events also span the passes "
-                                   "beside it and its mean duration overstates its own time"
-                                   if cocg else ""))
         if dom["kernel"] == "fft_direct_solve":
             roofline["bytes_model"] = ("one direct FP32 correction: the residual read and the solution "
                                        "read and written in FP64, the half spectrum moved through "

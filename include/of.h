@@ -64,7 +64,8 @@ typedef struct of_grid of_grid;
 typedef struct of_precond of_precond;   /* learned preconditioner (of_precond_create) */
 
 /* Krylov solve options.  tol is the target of the true FP64 relative residual
- * ||b - A x|| / ||b||.  precision OF_F64: CG/COCG entirely in FP64.  OF_F32: iterative
+ * ||b - A x|| / ||b||.  precision OF_F64: CG/COCG entirely in FP64 (the Laplacians summed in 64-bit
+ * fixed point, no less accurate at any point than FP64 sums).  OF_F32: iterative
  * refinement -- FP64 residual, FP32 solve of the correction, FP64 update -- repeated until tol.
  * The correction of each pass is direct (the periodic operator is diagonal in Fourier space; a
  * pass counts as one iteration) on grids of at most 2048 points per axis, unless no_multigrid or
@@ -72,7 +73,10 @@ typedef struct of_precond of_precond;   /* learned preconditioner (of_precond_cr
  * still needs, when that is less): preconditioned by a multigrid V-cycle beyond 2048 points
  * (Poisson and shifted systems whose grid coarsens), plain with no_multigrid, or with the learned
  * network when precond is set (see of_precond_create).  A direct pass that gains less than a
- * factor of ten (a shifted system that is singular to FP32) also continues with those.
+ * factor of ten (a shifted system whose symbol, at some mode, is below 2^-20 of its largest: such a
+ * mode gets no direct correction) also continues with those.  check_every: iterations queued between
+ * looks at the stopping flag; without effect on direct passes and on FP64 CG of small grids, which
+ * runs in one launch.
  * Zero fields take defaults (tol 1e-10, max_iter 20000, inner_tol 1e-5,
  * check_every 8, precond_theta 0.3). */
 typedef struct {

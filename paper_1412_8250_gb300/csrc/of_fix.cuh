@@ -24,8 +24,9 @@
 // path but for a few points where value and slope are small together (about ten in an electrostatic
 // potential on 96^3), fields that fall by powers of ten across a brick take FP64 arithmetic.
 //
-// Measured on a GB300 (order 12): 96^3 69.1 us in FP64 arithmetic -> 13.4, 192^3 514 -> 101 (70 GPts/s), of
-// which the looks at each point's neighbours, and the code they add, are 0.8 and 10; where nearly every
+// Measured on a GB300 (order 12): 96^3 69.1 us in FP64 arithmetic -> 13.4, 192^3 514 -> 101, 320^3 2.4 ms ->
+// 0.44 (74 GPts/s), of which the looks at each point's neighbours, and the code they add, are 0.8, 10 and 45 us;
+// where nearly every
 // point takes FP64 arithmetic after all (a Gaussian in the middle of 96^3) 69.  Bound by instruction issue
 // and latency at 12 warps per SM (168 registers; 4.9 staged values per point with their conversions, ~8
 // integer operations per distance).  Tried before the looks (12.7 us, 80 GPts/s at 320^3): both loads and
@@ -556,7 +557,7 @@ fix_kernel(Dims d, Weights<double> W, FixScale fs, bool vec, int bx, int by, int
 
 // Spacings equal but for the rounding of h = L / n (which moves 1 / h^2 by up to 2^-52 an axis, and its
 // own three operations by as much again) count as equal: their mean for the three axes, so that the
-// sums of all axes share one conversion (96^3: order 12 18.9 -> 12.7 us, order 2 14.3 -> 7.4).
+// sums of all axes share one conversion (96^3: order 12 18.9 -> 12.7 us, order 2 14.3 -> 7.4, when measured).
 inline FixScale fix_scale(of_grid* g) {
     FixScale fs;
     for (int a = 0; a < 3; ++a) fs.s[a] = std::ldexp(1.0, fix_shift(g->N)) / (fix_denominator(g->N) * g->h[a] * g->h[a]);

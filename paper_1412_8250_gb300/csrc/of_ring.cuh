@@ -9,8 +9,8 @@
 // What bounds it is the shared-memory pipe: per 8 points 24 64-bit reads for the x taps, 12 for
 // the y taps (four rows share one column) and 4 for the queue, 0.31 wavefronts per point; with two
 // rows per thread, and the queue's and the tile's planes fetched apart through registers, it was
-// 0.48 and two fetches, and odd n1 took a scalar kernel.  320^3, order 12: 95 -> 66 us
-// (495 GPts/s; HBM's floor is 39), order 6 128 -> 56, order 2 95 -> 53; 319 x 320 x 320 178 -> 93.
+// 0.48 and two fetches, and odd n1 took a scalar kernel.  320^3, order 12: 95 -> 71 us
+// (462 GPts/s, 68 us in a row of calls; HBM's floor is 39), order 6 128 -> 56, order 2 95 -> 53; 319 x 320 x 320 178 -> 93.
 // The blocks share all (tile, plane) pairs evenly; a run of planes costs 2N more of its own points
 // at its start, hence the rule on planes per block in launch_ring.
 #pragma once
