@@ -124,7 +124,10 @@ uintptr_t fix_bits(const Op& op) {
 }
 
 constexpr int FX_UX = 16, FX_BY = 8, FX_THREADS = FX_UX * FX_BY;
-constexpr int FX_ITEMS = 32;   // units of a warp that its lanes take together in FP64 arithmetic
+// Units of a warp that its lanes take together in FP64 arithmetic.  Eight in the complex Krylov sweep: its tile
+// (72 KB) and its two sums leave three blocks per SM 592 bytes more each (with 32 units, at two blocks, FP64
+// COCG on 192^3 took 36.8 ms instead of 33.5).
+template <bool CPLX, class Op> constexpr int fix_items() { return CPLX && !HasPre<Op>::value ? 8 : 32; }
 
 struct FixScale {
     double s[3];   // 2^fix_shift / (D h_a^2)
@@ -260,12 +263,13 @@ __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& 
     constexpr int PH = (HX / 2 + 3) / 4 * 4;
     constexpr int SLOTS = ROWS * FX_UX + FX_BY * 2 * PH;
     constexpr int SPT = (SLOTS + FX_THREADS - 1) / FX_THREADS;
+    constexpr int ITEMS = fix_items<CPLX, Op>();
     constexpr bool ALL = SPT * BZ <= 8;   // thin bricks: every slot's loads in flight at once
     extern __shared__ __align__(16) long long fix_smem[];
     __shared__ int yoff[ROWS], zoff[BZ + 2 * N], xoff[RW];   // periodic offsets in doubles (< 2^31)
     __shared__ int wtop[2][FX_THREADS / 32];
-    __shared__ unsigned char items[FX_THREADS / 32][FX_ITEMS];
-    __shared__ __align__(16) double2 taken[FX_THREADS / 32][FX_ITEMS];
+    __shared__ unsigned char items[FX_THREADS / 32][ITEMS];
+    __shared__ __align__(16) double2 taken[FX_THREADS / 32][ITEMS];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + FX_UX * ty;
     const int RF = CPLX ? 2 * d.n1 : d.n1, PF = RF * d.n2;
     // Staged row and first column of each of this thread's slots.  The first FX_BY rows of the order
@@ -466,7 +470,7 @@ __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& 
                 const unsigned c = fix_coarse<N, CPLX, BZ>(own_s, small, least) & coarse;
                 const int count = __popc(c);
                 total = __reduce_add_sync(0xffffffffu, count);
-                leave = total > FX_ITEMS;
+                leave = total > ITEMS;
                 if (!leave && total > 0) {   // eight lanes to a unit, four units at a time
                     mine = count;
 #pragma unroll
