@@ -24,8 +24,8 @@
 // path but for a few points where value and slope are small together (about ten in an electrostatic
 // potential on 96^3), fields that fall by powers of ten across a brick take FP64 arithmetic.
 //
-// Measured on a GB300 (order 12): 96^3 69.1 us in FP64 arithmetic -> 13.4, 192^3 514 -> 101, 320^3 2.4 ms ->
-// 0.44 (74 GPts/s), of which the looks at each point's neighbours, and the code they add, are 0.8, 10 and 45 us;
+// Measured on a GB300 (order 12): 96^3 69.1 us in FP64 arithmetic -> 12.9, 192^3 514 -> 99, 320^3 2.4 ms ->
+// 0.43 (76 GPts/s), of which the looks at each point's neighbours, and the code they add, are 0.3, 8 and 40 us;
 // where nearly every
 // point takes FP64 arithmetic after all (a Gaussian in the middle of 96^3) 69.  Bound by instruction issue
 // and latency at 12 warps per SM (168 registers; 4.9 staged values per point with their conversions, ~8
@@ -373,14 +373,15 @@ __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& 
             return make_longlong2(fix_from_bits(__double2hiint(q.x), (unsigned)__double2loint(q.x), E),
                                   fix_from_bits(__double2hiint(q.y), (unsigned)__double2loint(q.y), E));
         };
+        // beyond the sample: the largest exponent; and, where the sample is that small, all values' bits
         int top = 0, bits = 0;
-        auto seen = [&](double2 q) {
-            top = max(top, max(expo(q.x), expo(q.y)));
-            bits |= __double2hiint(q.x) | __double2loint(q.x);
-            bits |= __double2hiint(q.y) | __double2loint(q.y);
+        auto mark = [&](double2 q) {
+            bits |= __double2hiint(q.x) | __double2loint(q.x) | __double2hiint(q.y) | __double2loint(q.y);
         };
+        if (E == 128) {
 #pragma unroll
-        for (int j = 0; j < 2 * N; ++j) seen(zr[j]);
+            for (int j = 0; j < 2 * N; ++j) mark(zr[j]);
+        }
 #pragma unroll
         for (int m = 0; m < SPT; ++m) {
             double2 (&q)[BZ] = v[ALL ? m : 0];
@@ -389,13 +390,17 @@ __device__ __forceinline__ void fix_sweep(const Dims& d, const Weights<double>& 
                 long long* dst = fix_smem + srow[m] * RW + scol[m];
 #pragma unroll
                 for (int k = 0; k < BZ; ++k) {
-                    seen(q[k]);
+                    if (!ALL && m > 0) top = max(top, max(expo(q[k].x), expo(q[k].y)));
                     *reinterpret_cast<longlong2*>(dst + k * CPL) = fix(q[k]);
+                }
+                if (E == 128) {
+#pragma unroll
+                    for (int k = 0; k < BZ; ++k) mark(q[k]);
                 }
             }
         }
-        // the block's largest exponent, with 2^16 where a bit is set anywhere
-        const int all = block_max(top | (bits != 0 ? 1 << 16 : 0), wtop[1]);
+        // the largest exponent beyond the sample, with 2^16 where a bit is set anywhere (or the sample not small)
+        const int all = block_max(top | (bits != 0 || E > 128 ? 1 << 16 : 0), wtop[1]);
         if ((all & 0xffff) > E && (all & 0xffff) <= 2046) {
             // a staged value above the sample's range: once more, with its exponent (a short loop: cold code)
             E = all & 0xffff;
